@@ -55,10 +55,11 @@ struct WsHeader {
     int total;           // total samples of the batch (sum of n)
     int n_kept;          // fine stage: samples kept after the tau_f test
     unsigned done;       // block-completion counter of the loss reduction
-    float loss_acc;      // sum over rays of ||C_hat - C||^2
+    double loss_acc;     // sum over rays of ||C_hat - C||^2 (+ auxiliary terms): one add per block, up to
+                         // thousands, which in FP32 cost the loss 1e-6 (two-ray blocks, 8192 rays)
     int aux;             // 1: the last forward had a target and auxiliary loss weights (rtarget valid)
     int xcache;          // 1: the last forward stored the colour kernels' input panels (xcache valid)
-    int pad[57];
+    int pad[56];
 };
 static_assert(sizeof(WsHeader) == 256, "WsHeader size");
 

@@ -146,7 +146,7 @@ __device__ void finish_loss_fine(const RenderArgs &A, float part) {
     if (threadIdx.x == 0) {
         float s = 0.0f;
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-        atomicAdd(&A.hdr->loss_acc, s);
+        atomicAdd(&A.hdr->loss_acc, (double)s);
         __threadfence();
         unsigned prev = atomicAdd(&A.hdr->done, 1u);
         last = (prev == gridDim.x - 1);
@@ -154,8 +154,8 @@ __device__ void finish_loss_fine(const RenderArgs &A, float part) {
     __syncthreads();
     if (last && threadIdx.x == 0 && A.loss_out) {
         __threadfence();
-        float tot = atomicAdd(&A.hdr->loss_acc, 0.0f);
-        A.loss_out[0] = A.R > 0 ? tot / (float)A.R : 0.0f;
+        const double tot = atomicAdd(&A.hdr->loss_acc, 0.0);
+        A.loss_out[0] = A.R > 0 ? (float)(tot / (double)A.R) : 0.0f;
     }
 }
 
