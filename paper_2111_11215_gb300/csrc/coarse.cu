@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_fwd_kernel(RenderArgs A
     const bool aux = A.target && (A.w_pt != 0.0f || A.w_bg != 0.0f);
     for (int r = warp; r < A.R; r += nwarps) {
         const RayRec rr = A.rays[r];
+        flag_bad_ray(A, rr, lane);
         float tg[3] = {0.0f, 0.0f, 0.0f};
         if (aux)
             for (int ch = 0; ch < 3; ++ch) tg[ch] = A.target[3 * r + ch];
@@ -316,7 +317,7 @@ void launch_coarse_bwd(const RenderArgs &A, cudaStream_t s) {
     ProfScope ps_(DVGO_K_COARSE_BWD, s);
     const int g = coarse_grid(A.R);
     // the longest ray's optical depths per warp (at most kMaxSamplesPerRay: 16 KB a block)
-    const int cap = (int)(A.max_samples / A.R);
+    const int cap = A.cap;
     const size_t smem = sizeof(float) * (kCoarseThreads / 32) * (cap + kMaxChunks);
     if (A.act_order == DVGO_ACT_PRE) coarse_bwd_kernel<DVGO_ACT_PRE><<<g, kCoarseThreads, smem, s>>>(A, cap);
     else if (A.act_order == DVGO_ACT_IN) coarse_bwd_kernel<DVGO_ACT_IN><<<g, kCoarseThreads, smem, s>>>(A, cap);

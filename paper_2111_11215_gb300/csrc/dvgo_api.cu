@@ -173,6 +173,7 @@ RenderArgs make_args(const dvgo_params *p, const dvgo_grid_desc *dd, const float
         A.xcache = L.xcache ? reinterpret_cast<unsigned char *>(b + L.xcache) : nullptr;
     }
     A.max_samples = L.max_samples;
+    A.cap = R > 0 ? (int)(L.max_samples / R) : 0;
     if (p->mode == DVGO_MODE_FINE && p->freespace && p->freespace->density) {
         const dvgo_freespace &f = *p->freespace;
         A.fs_density = f.density;
@@ -217,10 +218,14 @@ int check_ws(const WsLayout &L, void *ws, size_t bytes) {
     return DVGO_OK;
 }
 
-__global__ void sample_counts_kernel(const RayRec *rays, const WsHeader *hdr, int R, int *counts, int *total) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < R) counts[i] = rays[i].n;
-    if (i == 0 && total) *total = hdr->total;
+__global__ void sample_counts_kernel(const RayRec *rays, int R, int *counts, int *total) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = i < R ? rays[i].n : 0;
+    if (i < R) counts[i] = n;
+    if (total) {
+        const int sum = __reduce_add_sync(0xffffffffu, n);
+        if ((threadIdx.x & 31) == 0 && sum) atomicAdd(total, sum);
+    }
 }
 
 int launch_status() {
@@ -397,9 +402,10 @@ int dvgo_sample_counts(const void *ws, int n_rays, int *counts_out, int *total_o
     int blocks = (n_rays + 255) / 256;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     ProfScope ps_(DVGO_K_AUX, s);
-    sample_counts_kernel<<<blocks > 0 ? blocks : 1, 256, 0, s>>>(
-        reinterpret_cast<const RayRec *>(b + L.rays), reinterpret_cast<const WsHeader *>(b + L.header), n_rays,
-        counts_out, total_out);
+    if (total_out) cudaMemsetAsync(total_out, 0, sizeof(int), s);
+    if (blocks > 0)
+        sample_counts_kernel<<<blocks, 256, 0, s>>>(reinterpret_cast<const RayRec *>(b + L.rays), n_rays, counts_out,
+                                                    total_out);
     return launch_status();
 }
 

@@ -3,7 +3,6 @@
 // Data flow of one render (all on the caller's stream, no host synchronisation):
 //   ray_setup        per ray, FP64: normalise d, clip to the box, count samples, store the ray
 //                    in lattice coordinates (Sec. 4.2 fine-stage sampling, Eq. coarse_sample)
-//   scan_counts      exclusive scan of the per-ray counts -> first sample slot of every ray
 //   coarse_fwd/bwd   warp per ray: gather, post-activation, warp-scan compositing (Sec. 2/3/4.1)
 //   fine_density     warp per ray: density gather + post-activation, per-sample optical depth,
 //                    compact list of the kept samples (Sec. 4.2 free space skipping)
@@ -44,15 +43,14 @@ struct RayRec {
     float dir[3];        // normalised direction (FP32, positional encoding input)
     float p;             // jitter in [0, 1)
     int n;               // number of samples
-    int off;             // first sample slot (exclusive scan of n)
+    int off;             // first sample slot, ray * slots per ray (-1: zero / non-finite direction, n = 0)
 };
 static_assert(sizeof(RayRec) == 128, "RayRec layout");
-static_assert(offsetof(RayRec, off) == offsetof(RayRec, n) + 4 && offsetof(RayRec, n) % 8 == 0, "RayRec (n, off) pair");
 
 // Workspace header (first 256 bytes of the workspace).
 struct WsHeader {
     int flags;           // bit 0: a ray of the last forward had a zero / non-finite direction
-    int total;           // total samples of the batch (sum of n)
+    int pad0;
     int n_kept;          // fine stage: samples kept after the tau_f test
     unsigned done;       // block-completion counter of the loss reduction
     double loss_acc;     // sum over rays of ||C_hat - C||^2 (+ auxiliary terms): one add per block, up to
@@ -101,7 +99,8 @@ struct RenderArgs {
     int2 *kept;                 // compact list of kept samples: (slot, ray)
     unsigned char *xcache;      // BF16 tensor-core path: the forward's X panel of every tile (16 KiB
                                 // each, swizzled as in shared memory), reloaded by the backward
-    long long max_samples;
+    long long max_samples;      // slots of the whole batch: R * cap
+    int cap;                    // sample slots per ray (the longest possible ray)
     // outputs
     float *rgb_out, *tfinal_out, *loss_out, *dloss_out;
     // backward inputs / outputs
@@ -154,6 +153,17 @@ __device__ __forceinline__ float bg_entropy_dT(float TK) {
 // FP64 value -> fixed point (round to nearest).
 __device__ __forceinline__ long long to_fx(double v) { return __double2ll_rn(v * 0x1p40); }
 
+// a / b correctly rounded, from y = 1 / b correctly rounded (no over- or underflow in between): q = a y
+// corrected once is within an ulp, and the second correction by the exact remainder then rounds
+// correctly (Markstein, "Computation of elementary functions on the IBM RISC System/6000", 1990).  Five
+// FP64 operations where a division takes about twenty: a clip divides three times by the direction's
+// length and twice by each of its components.
+__host__ __device__ __forceinline__ double div_by(double a, double b, double y) {
+    double q = a * y;
+    q = fma(fma(-q, b, a), y, q);
+    return fma(fma(-q, b, a), y, q);
+}
+
 // Ray / box clip in FP64 with every operation separately rounded (no FMA contraction), in the
 // order the sample count depends on (Sec. 4.2 fine-stage points sampling):
 //   len = sqrt((dx*dx + dy*dy) + dz*dz), dn = d / len;
@@ -178,11 +188,15 @@ __device__ __forceinline__ Clip slab_clip(const double o[3], const double d[3], 
     c.lo = t_near;
     c.hi = t_far;
     if (c.ok) {
+        // (FP32 inputs: |d| / len is 0 or above 1e-84 and every quotient below 1e124)
+        const double inv_len = __drcp_rn(len);
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            c.dn[a] = __ddiv_rn(d[a], len);
+            c.dn[a] = div_by(d[a], len, inv_len);
             if (c.dn[a] != 0.0) {
-                const double t1 = __ddiv_rn(__dsub_rn(mn[a], o[a]), c.dn[a]);
-                const double t2 = __ddiv_rn(__dsub_rn(mx[a], o[a]), c.dn[a]);
+                const double inv = __drcp_rn(c.dn[a]);
+                const double t1 = div_by(__dsub_rn(mn[a], o[a]), c.dn[a], inv);
+                const double t2 = div_by(__dsub_rn(mx[a], o[a]), c.dn[a], inv);
                 const double tl = t1 < t2 ? t1 : t2;
                 const double th = t1 < t2 ? t2 : t1;
                 if (tl > c.lo) c.lo = tl;
@@ -356,6 +370,12 @@ __device__ __forceinline__ bool known_free(const RenderArgs &A, const long long 
     for (int q = 0; q < 8; ++q)
         s = fmaf(corner_weight(c, q), __ldg(A.fs_density + corner_index(c, q, A.fs_ny, A.fs_nz, A.fs_packed)), s);
     return -expm1f(-softplusf(s + A.fs_shift_b) * A.fs_step) < A.fs_tau;
+}
+
+// A ray with a zero / non-finite direction sets bit 0 of the flag word, in the kernel that follows the
+// ray set-up (which clears the word).
+__device__ __forceinline__ void flag_bad_ray(const RenderArgs &A, const RayRec &r, int lane) {
+    if (lane == 0 && r.off < 0) atomicOr(&A.hdr->flags, 1);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(kDensityThreads, DVGO_DENSITY_MIN_BLOCKS) fine
     int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int r = warp; r < A.R; r += nwarps) {
         const RayRec rr = A.rays[r];
+        flag_bad_ray(A, rr, lane);
         float carry = 0.0f;          // optical depth before this chunk, as the compositing pass forms it
         for (int base = 0; base < rr.n; base += 64) {
             if (isinf(carry)) {      // terminated: T = 0 from here on

@@ -1,4 +1,4 @@
-// ray_setup.cu -- per-ray clipping and sample counting, and the exclusive scan of the counts.
+// ray_setup.cu -- per-ray clipping and sample counting, and the workspace layout.
 //
 // Sec. 4.2 (fine-stage points sampling): the near and far bounds of every ray become the two
 // ends of its intersection with the grid's bounding box (the near bound stays put when the
@@ -21,15 +21,26 @@ namespace dvgo {
 
 namespace {
 
-__global__ void __launch_bounds__(64) ray_setup_kernel(RenderArgs A, const float *__restrict__ rays_o,
-                                                        const float *__restrict__ rays_d,
-                                                        const float *__restrict__ jitter, double3 bmin,
-                                                        double3 bmax, double3 scale, double t_near,
-                                                        double t_far, double step, double cap,
-                                                        int n_expl) {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
+// Thread per ray.  Every ray owns cap sample slots (the workspace is sized for the longest ray), so a
+// ray's first slot is ray * cap and no scan of the counts runs before the sample passes: one scan block
+// took 14 us for 8,192 rays and 97 us for 65,536.  Bound by the FP64 pipe (2 lanes a clock per SM), hence
+// the divisions by known reciprocals (div_by) and no position that the sampling in use does not read.
+// Records and encodings are written from registers, 16 bytes a store: staging them through shared memory
+// would give whole-line stores, but the set-up runs beside the feature-grid Adam, whose loads take the
+// SM's whole L1, and a block with shared memory then waits for the Adam to end (152 us instead of 20).
+// Set-up and scan before, set-up alone now (events around the launches): 8,192 rays 32 -> 13 us, 65,536
+// rays 126 -> 27 us.
+constexpr int kSetupThreads = 64;
+
+__global__ void __launch_bounds__(kSetupThreads) ray_setup_kernel(RenderArgs A, const float *__restrict__ rays_o,
+                                                                   const float *__restrict__ rays_d,
+                                                                   const float *__restrict__ jitter, double3 bmin,
+                                                                   double3 bmax, double3 scale, double t_near,
+                                                                   double t_far, double step, double inv_step,
+                                                                   double cap, int n_expl) {
+    const int r = blockIdx.x * kSetupThreads + threadIdx.x;
     if (r == 0) {
-        A.hdr->total = 0;
+        A.hdr->flags = 0;
         A.hdr->n_kept = 0;
         A.hdr->done = 0u;
         A.hdr->loss_acc = 0.0;
@@ -44,111 +55,55 @@ __global__ void __launch_bounds__(64) ray_setup_kernel(RenderArgs A, const float
     double p = jitter ? (double)jitter[r] : 0.5;
 
     const Clip cl = slab_clip(o, d, mn, mx, t_near, t_far);
-    const bool ok = cl.ok;
     const double lo = cl.lo, hi = cl.hi;
-    const double *dn = cl.dn;
-    RayRec rec;
+    alignas(16) RayRec rec;
     int n = 0;
     if (hi > lo) {
-        double q = __ddiv_rn(__dsub_rn(hi, lo), step);
+        double q = div_by(__dsub_rn(hi, lo), step, inv_step);
         q = __dsub_rn(q, p);
         double c = ceil(q);
         if (c > cap) c = cap;
         n = c > 0.0 ? (int)c : 0;
         if (n_expl >= 0) n = n_expl;   // explicit samples: all or nothing
     }
-    const bool uniform = n > 0 && n_expl < 0;
-    const double t_first = uniform ? fma(p, step, lo) : 0.0;   // t of sample 0 of the uniform stepping
+    const bool uniform = n_expl < 0;
+    const double t_first = uniform ? fma(p, step, lo) : lo;   // t of sample 0 of the uniform stepping
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double uo = __dmul_rn(__dsub_rn(o[a], mn[a]), sc[a]);
-        rec.e[a] = __dmul_rn(dn[a], sc[a]);
-        rec.dir[a] = (float)dn[a];
+        rec.e[a] = __dmul_rn(cl.dn[a], sc[a]);
+        rec.dir[a] = (float)cl.dn[a];
         // fixed-point values only where they are used: in range for any sample inside the box
-        rec.uefx[a] = n > 0 ? to_fx(fma(lo, rec.e[a], uo)) : 0;
-        rec.u0fx[a] = uniform ? to_fx(fma(t_first, rec.e[a], uo)) : 0;
-        rec.dfx[a] = uniform ? to_fx(step * rec.e[a]) : 0;
+        const long long u = n > 0 ? to_fx(fma(t_first, rec.e[a], uo)) : 0;
+        rec.uefx[a] = uniform ? 0 : u;
+        rec.u0fx[a] = uniform ? u : 0;
+        rec.dfx[a] = uniform && n > 0 ? to_fx(step * rec.e[a]) : 0;
     }
     rec.t_enter = lo;
     rec.p = (float)p;
+    rec.n = n;
+    rec.off = cl.ok ? r * A.cap : -1;
+    const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(&rec);
+    ulonglong2 *g = reinterpret_cast<ulonglong2 *>(A.rays + r);
+#pragma unroll
+    for (int k = 0; k < (int)sizeof(RayRec) / 16; ++k) g[k] = w[k];
     if (A.texit) A.texit[r] = hi;
     if (A.pe) {
         // positional encoding of the normalised direction (fine-stage MLP input, Supp. A, k_d = 4):
         // [d, sin(2^k d_c) (c-major), cos(2^k d_c) (c-major)]
-        float *pe = A.pe + (size_t)r * kPeStride;
+        float pe[kPeStride];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            float dv = rec.dir[a];
-            pe[a] = dv;
-            for (int k = 0; k < 4; ++k) {
-                float sv, cv;
-                sincosf(ldexpf(dv, k), &sv, &cv);
-                pe[3 + a * 4 + k] = sv;
-                pe[15 + a * 4 + k] = cv;
-            }
+            pe[a] = rec.dir[a];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sincosf(ldexpf(rec.dir[a], k), &pe[3 + a * 4 + k], &pe[15 + a * 4 + k]);
         }
+#pragma unroll
         for (int k = 27; k < kPeStride; ++k) pe[k] = 0.0f;
-    }
-    rec.n = n;
-    rec.off = ok ? 0 : -1;   // -1 marks a ray with a zero / non-finite direction for the scan
-    A.rays[r] = rec;
-}
-
-// Exclusive scan of RayRec::n into RayRec::off by one block; the total and the flag word (a ray
-// with a zero / non-finite direction) go to the header.  The block is small (256 threads) so that
-// it fits on an SM beside the HBM-bound Adam step of another stream; a 1024-thread block does not,
-// and would wait for the whole Adam.  It works in rounds of 256 x kScanPer rays: thread t takes
-// the contiguous run of kScanPer rays at base + kScanPer t and issues all their (n, off) loads at
-// once (one load latency per round, not one per ray), the run sums are scanned across the block
-// with warp shuffles, and the offsets are written from registers.
-constexpr int kScanThreads = 256;
-constexpr int kScanPer = 16;
-
-__global__ void __launch_bounds__(kScanThreads) scan_counts_kernel(RenderArgs A) {
-    constexpr int NW = kScanThreads / 32;
-    __shared__ int warp_tot[NW];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    int carry = 0, bad = 0;
-    for (int base = 0; base < A.R; base += kScanThreads * kScanPer) {
-        const int beg = base + tid * kScanPer;
-        int n[kScanPer], local = 0;
+        float4 *gp = reinterpret_cast<float4 *>(A.pe + (size_t)r * kPeStride);
 #pragma unroll
-        for (int k = 0; k < kScanPer; ++k) {
-            n[k] = 0;
-            if (beg + k < A.R) {
-                const int2 no = *reinterpret_cast<const int2 *>(&A.rays[beg + k].n);   // (n, off)
-                n[k] = no.x;
-                bad |= no.y < 0;
-            }
-            local += n[k];
-        }
-        // inclusive warp scan of the run sums, then the warp totals
-        int v = local;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += t;
-        }
-        if (lane == 31) warp_tot[wid] = v;
-        __syncthreads();
-        int before = 0, total = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const int t = warp_tot[w];
-            before += w < wid ? t : 0;
-            total += t;
-        }
-        __syncthreads();   // warp_tot is rewritten by the next round
-        int run = carry + before + v - local;
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k) {
-            if (beg + k < A.R) A.rays[beg + k].off = run;
-            run += n[k];
-        }
-        carry += total;
-    }
-    bad = __syncthreads_or(bad);
-    if (tid == 0) {
-        A.hdr->total = carry;
-        A.hdr->flags = bad ? 1 : 0;
+        for (int k = 0; k < kPeStride / 4; ++k)
+            gp[k] = make_float4(pe[4 * k], pe[4 * k + 1], pe[4 * k + 2], pe[4 * k + 3]);
     }
 }
 
@@ -160,18 +115,11 @@ void launch_ray_setup(const RenderArgs &A, const float *rays_o, const float *ray
     double3 bmax = make_double3(g.xyz_max[0], g.xyz_max[1], g.xyz_max[2]);
     double3 sc = make_double3((double)(g.nx - 1) / (bmax.x - bmin.x), (double)(g.ny - 1) / (bmax.y - bmin.y),
                               (double)(g.nz - 1) / (bmax.z - bmin.z));
-    int blocks = (A.R + 63) / 64;
-    if (blocks < 1) blocks = 1;
-    {
-        ProfScope ps_(DVGO_K_RAY_SETUP, s);
-        ray_setup_kernel<<<blocks, 64, 0, s>>>(A, rays_o, rays_d, jitter, bmin, bmax, sc, (double)p.t_near,
-                                           (double)p.t_far, (double)p.step, (double)cap,
-                                           A.ts ? A.n_expl : -1);
-    }
-    {
-        ProfScope ps_(DVGO_K_SCAN, s);
-        scan_counts_kernel<<<1, kScanThreads, 0, s>>>(A);
-    }
+    const int blocks = (A.R + kSetupThreads - 1) / kSetupThreads;
+    ProfScope ps_(DVGO_K_RAY_SETUP, s);
+    ray_setup_kernel<<<blocks, kSetupThreads, 0, s>>>(A, rays_o, rays_d, jitter, bmin, bmax, sc, (double)p.t_near,
+                                                      (double)p.t_far, (double)p.step, 1.0 / (double)p.step,
+                                                      (double)cap, A.ts ? A.n_expl : -1);
 }
 
 WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache) {
