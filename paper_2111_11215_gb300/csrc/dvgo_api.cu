@@ -76,6 +76,28 @@ long long max_samples(const dvgo_params *p, const dvgo_grid_desc *g, int R, cons
     return per * (long long)R;
 }
 
+// Where the cell mask is used: it costs one pass over the density grid (13 us at 160^3, 8 us at 101^3) and
+// saves the gathers and activations of the samples in empty cells.  65,536 rays of a frame at 160^3 (10 M
+// samples, 4.1 M cells): density pass 180 us without, 42 + 13 us with it; 8,192 rays at 101^3 with known
+// free space (0.87 M samples, 1.0 M cells): 42 us without, 23 + 8 us with it.  The bound R * cap counts three
+// to four times the samples of a usual batch; at half the cells the two forms cost the same within a
+// few us.  Explicit samples may lie outside the lattice, where interpolation is not bounded by the corners.
+size_t mask_words(const dvgo_params *p, const dvgo_grid_desc *g, int R, const dvgo_samples *ex) {
+    if (p->mode != DVGO_MODE_FINE || ex || !(p->tau_f > 0.0f && p->tau_f < 1.0f) || !isfinite(p->shift_b)) return 0;
+    const long long cells = (long long)g->nx * g->ny * g->nz;
+    if (max_samples(p, g, R, ex) < cells / 2) return 0;
+    return (size_t)g->nx * g->ny * ((g->nz + 31) / 32);
+}
+
+// Raw density whose alpha = 1 - exp(-softplus(v + b) step) is tau_f (1 - 1e-4): below it, the FP32
+// evaluation of alpha (a few ulp off) is below tau_f too.
+float mask_threshold(const dvgo_params *p) {
+    const double y = -log1p(-(double)p->tau_f * (1.0 - 1e-4)) / (double)p->step;   // softplus value
+    const double z = y > 30.0 ? y : log(expm1(y));
+    const double v = z - (double)p->shift_b;
+    return (float)(v - 1e-6 * (fabs(v) + fabs((double)p->shift_b)));   // v + b rounds in FP32
+}
+
 int check_common(const dvgo_params *p, const dvgo_grid_desc *dd, const float *density, const dvgo_grid_desc *cd,
                  const void *cgrid, const dvgo_mlp *mlp, int R, const float *ro, const float *rd,
                  const dvgo_samples *ex) {
@@ -167,10 +189,18 @@ RenderArgs make_args(const dvgo_params *p, const dvgo_grid_desc *dd, const float
     if (p->mode == DVGO_MODE_FINE) {
         A.pe = reinterpret_cast<float *>(b + L.pe);
         A.texit = reinterpret_cast<double *>(b + L.texit);
-        A.samp = reinterpret_cast<float4 *>(b + L.samp);
+        A.rayk = reinterpret_cast<int2 *>(b + L.rayk);
+        A.stau = reinterpret_cast<float *>(b + L.stau);
+        A.kidx = reinterpret_cast<unsigned short *>(b + L.kidx);
+        A.scol = reinterpret_cast<float4 *>(b + L.scol);
         A.sgrad = reinterpret_cast<float4 *>(b + L.sgrad);
         A.kept = reinterpret_cast<int2 *>(b + L.kept);
         A.xcache = L.xcache ? reinterpret_cast<unsigned char *>(b + L.xcache) : nullptr;
+        if (L.mask) {
+            A.mask = reinterpret_cast<unsigned *>(b + L.mask);
+            A.mask_wpr = (dd->nz + 31) / 32;
+            A.mask_thr = mask_threshold(p);
+        }
     }
     A.max_samples = L.max_samples;
     A.cap = R > 0 ? (int)(L.max_samples / R) : 0;
@@ -273,7 +303,7 @@ size_t dvgo_workspace_size(const dvgo_params *p, const dvgo_grid_desc *density, 
                            const dvgo_samples *ex) {
     if (!p || !density || n_rays < 0 || !grid_ok(density) || !(p->step > 0.0f)) return 0;
     long long S = max_samples(p, density, n_rays, ex);
-    return ws_layout(n_rays, S, p->mode, xcache_on(p)).total;
+    return ws_layout(n_rays, S, p->mode, xcache_on(p), mask_words(p, density, n_rays, ex)).total;
 }
 
 // The stream waits for the caller's event (if any) before the first kernel that reads cgrid.
@@ -294,7 +324,7 @@ int dvgo_render_fwd(const dvgo_params *p, const dvgo_grid_desc *dd, const float 
     if (st) return st;
     if (R > 0 && !rgb_out) return DVGO_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    WsLayout L = ws_layout(R, max_samples(p, dd, R, ex), p->mode, xcache_on(p));
+    WsLayout L = ws_layout(R, max_samples(p, dd, R, ex), p->mode, xcache_on(p), mask_words(p, dd, R, ex));
     if ((st = check_ws(L, ws, ws_bytes))) return st;
     if (R == 0) {
         if (loss_out) cudaMemsetAsync(loss_out, 0, sizeof(float), s);
@@ -312,6 +342,7 @@ int dvgo_render_fwd(const dvgo_params *p, const dvgo_grid_desc *dd, const float 
         wait_cgrid(p, s);
         launch_coarse_fwd(A, s);
     } else {
+        if (A.mask) launch_empty_cells(A, s);
         launch_fine_density(A, s);
         wait_cgrid(p, s);
         if (p->mlp_prec == DVGO_MLP_BF16) {
@@ -334,7 +365,7 @@ int dvgo_render_bwd(const dvgo_params *p, const dvgo_grid_desc *dd, const float 
     if (R > 0 && (!grad_rgb || !grad_density || !grad_cgrid)) return DVGO_ERR_INVALID_ARG;
     if (p->mode == DVGO_MODE_FINE && !grad_mlp) return DVGO_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    WsLayout L = ws_layout(R, max_samples(p, dd, R, ex), p->mode, xcache_on(p));
+    WsLayout L = ws_layout(R, max_samples(p, dd, R, ex), p->mode, xcache_on(p), mask_words(p, dd, R, ex));
     if ((st = check_ws(L, ws, ws_bytes))) return st;
     if (R == 0) return DVGO_OK;
     RenderArgs A = make_args(p, dd, density, cd, cgrid, mlp, R, ex, ws, L);
@@ -417,7 +448,7 @@ int dvgo_touched_points(const dvgo_params *p, const dvgo_grid_desc *dd, int R, c
     if (ex && (!ex->t || !ex->dt || ex->n_per_ray < 1)) return DVGO_ERR_INVALID_ARG;
     if (p->freespace && p->freespace->density && !grid_ok(&p->freespace->desc)) return DVGO_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    WsLayout L = ws_layout(R, max_samples(p, dd, R, ex), p->mode, xcache_on(p));
+    WsLayout L = ws_layout(R, max_samples(p, dd, R, ex), p->mode, xcache_on(p), mask_words(p, dd, R, ex));
     int st = check_ws(L, ws, ws_bytes);
     if (st) return st;
     RenderArgs A = make_args(p, dd, nullptr, dd, nullptr, nullptr, R, ex, ws, L);

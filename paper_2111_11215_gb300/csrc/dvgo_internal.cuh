@@ -4,8 +4,11 @@
 //   ray_setup        per ray, FP64: normalise d, clip to the box, count samples, store the ray
 //                    in lattice coordinates (Sec. 4.2 fine-stage sampling, Eq. coarse_sample)
 //   coarse_fwd/bwd   warp per ray: gather, post-activation, warp-scan compositing (Sec. 2/3/4.1)
-//   fine_density     warp per ray: density gather + post-activation, per-sample optical depth,
-//                    compact list of the kept samples (Sec. 4.2 free space skipping)
+//   empty_cells      (uniform steps, tau_f > 0, many samples) one bit per lattice cell: no sample in it
+//                    can reach tau_f
+//   fine_density     warp per ray: density gather + post-activation, optical depths of the kept
+//                    samples, packed at the front of the ray's slots, and the batch's list of kept
+//                    samples (Sec. 4.2 free space skipping)
 //   fine_colour      persistent CTAs over tiles of kept samples: feature gather + PE + MLP
 //   fine_composite   warp per ray: transmittance scan, C_hat, loss (Eq. volume_rendering)
 //   fine_bwd_*       composite backward + density scatter (warp per ray), then the colour tile
@@ -25,7 +28,7 @@ constexpr int kWarp = 32;
 constexpr int kMaxFeat = 16;
 constexpr int kPeStride = 32;                      // floats per ray of the direction encoding
 constexpr int kMaxChunks = 64;                    // backward kernels: rays of <= 64 x 32 samples
-constexpr int kMaxSamplesPerRay = 32 * kMaxChunks;
+constexpr int kMaxSamplesPerRay = 32 * kMaxChunks;   // (j and k of a kept sample then fit 16 bits each)
 
 // Lattice coordinates of samples are carried in 64-bit fixed point with kFxBits fractional bits
 // (resolution 9e-13 lattice units, range +-8.4e6): the per-sample position then needs no FP64
@@ -63,7 +66,8 @@ static_assert(sizeof(WsHeader) == 256, "WsHeader size");
 
 // Workspace layout; every block 256-byte aligned.
 struct WsLayout {
-    size_t header, rays, rayout, rtarget, pe, texit, samp, sgrad, kept, xcache, total;   // xcache 0: none
+    size_t header, rays, rayout, rtarget, pe, texit, rayk, stau, kidx, scol, sgrad, kept, mask, xcache, total;
+                                 // mask, xcache 0: none
     long long max_samples;
 };
 
@@ -94,9 +98,16 @@ struct RenderArgs {
     int fs_packed;              // the known-free-space grid in DVGO_LAYOUT_PACKED
     float *pe;                  // fine: per ray [d (3), sin (12), cos (12), 0 x 5] (kPeStride floats)
     double *texit;              // fine: per ray clipped exit distance
-    float4 *samp;               // per sample slot: (tau, r, g, b)
-    float4 *sgrad;              // per sample slot: (unused, dL/dc)
-    int2 *kept;                 // compact list of kept samples: (slot, ray)
+    // A ray's kept samples sit in order at the front of its cap slots: slot ray * cap + j is the j-th.
+    int2 *rayk;                 // fine: per ray (kept samples, first terminated sample or INT_MAX)
+    float *stau;                // per slot: optical depth tau (density pass)
+    unsigned short *kidx;       // per slot: sample index k along the ray
+    float4 *scol;               // per slot: (r, g, b, tau) (colour kernels)
+    float4 *sgrad;              // per slot: (0, dL/do), o the output layer's value before the sigmoid
+    int2 *kept;                 // compact list of kept samples: (j | k << 16, ray)
+    unsigned *mask;             // one bit per lattice cell, set where a sample may reach tau_f (nullable)
+    int mask_wpr;               // its words per lattice row
+    float mask_thr;             // raw density below which alpha < tau_f
     unsigned char *xcache;      // BF16 tensor-core path: the forward's X panel of every tile (16 KiB
                                 // each, swizzled as in shared memory), reloaded by the backward
     long long max_samples;      // slots of the whole batch: R * cap
@@ -436,13 +447,14 @@ __device__ __forceinline__ float seg_sum(float v, const Seg &s, int lane) {
 // Host-side launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------------------------
 
-// xcache: add the block of the BF16 colour kernels' X panels (fine mode), after all others so
-// that the other offsets do not depend on it.
-WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache = false);
+// mask_words, xcache: add the blocks of the cell mask and of the BF16 colour kernels' X panels (fine
+// mode), after all others so that the other offsets do not depend on them.
+WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache = false, size_t mask_words = 0);
 void launch_ray_setup(const RenderArgs &A, const float *rays_o, const float *rays_d, const float *jitter,
                       const dvgo_params &p, const dvgo_grid_desc &g, long long cap, cudaStream_t s);
 void launch_coarse_fwd(const RenderArgs &A, cudaStream_t s);
 void launch_coarse_bwd(const RenderArgs &A, cudaStream_t s);
+void launch_empty_cells(const RenderArgs &A, cudaStream_t s);
 void launch_fine_density(const RenderArgs &A, cudaStream_t s);
 void launch_fine_colour_fwd(const RenderArgs &A, cudaStream_t s);
 void launch_fine_composite_fwd(const RenderArgs &A, cudaStream_t s);

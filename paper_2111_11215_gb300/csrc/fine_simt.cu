@@ -100,11 +100,11 @@ __device__ void gather_tile(Smem<PEX> &S, const RenderArgs &A, int tile, int n_k
     float xw = 0.0f;   // world coordinate of axis q - 1 (PE(x), threads q = 1..3)
     if (valid) {
         int2 kv = A.kept[e];
-        slot = kv.x;
         ray = kv.y;
         rp = A.rays + ray;
         const RayRec &rr = *rp;
-        int k = slot - rr.off;
+        slot = rr.off + (kv.x & 0xffff);
+        const int k = kv.x >> 16;
         float dt;
         Cell c = sample_cell(A, rr, ray, k, dt);
         if (PEX && q > 0) {
@@ -252,7 +252,9 @@ __global__ void __launch_bounds__(NT, 1) fine_colour_fwd_kernel(RenderArgs A) {
         int s = threadIdx.x & 63, ch = threadIdx.x >> 6;
         if (ch < 3 && S.slot[s] >= 0) {
             float c = sigmoidf_(out_logit(S, s, ch));
-            reinterpret_cast<float *>(A.samp + S.slot[s])[1 + ch] = c;
+            reinterpret_cast<float *>(A.scol + S.slot[s])[ch] = c;
+        } else if (ch == 3 && S.slot[s] >= 0) {
+            reinterpret_cast<float *>(A.scol + S.slot[s])[3] = A.stau[S.slot[s]];   // tau goes with the colour
         }
     }
 }
@@ -289,18 +291,10 @@ __global__ void __launch_bounds__(NT, 1) fine_colour_bwd_kernel(RenderArgs A) {
         __syncthreads();
         gemm_fwd<HID>(S.h1, S.w2, S.b2, S.h2);
         __syncthreads();
-        // output layer + sigmoid backward
+        // dout = dL/dc c (1 - c), formed by the compositing backward with the forward's colour c
         {
             int s = tid & 63, ch = tid >> 6;
-            if (ch < 3) {
-                float d = 0.0f;
-                if (S.slot[s] >= 0) {
-                    float c = sigmoidf_(out_logit(S, s, ch));
-                    float dc = reinterpret_cast<const float *>(A.sgrad + S.slot[s])[1 + ch];
-                    d = dc * c * (1.0f - c);
-                }
-                S.dout[s * 3 + ch] = d;
-            }
+            if (ch < 3) S.dout[s * 3 + ch] = S.slot[s] >= 0 ? reinterpret_cast<const float *>(A.sgrad + S.slot[s])[1 + ch] : 0.0f;
         }
         __syncthreads();
         // dW3, db3 (need H2 before it is overwritten)

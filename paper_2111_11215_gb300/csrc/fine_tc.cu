@@ -247,19 +247,18 @@ __device__ __forceinline__ void produce_row(const RenderArgs &A, SmemTC &S, int 
     float fx = 0.0f, fy = 0.0f, fz = 0.0f, d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
     if (kv.y >= 0) {
         float dt;
-        const Cell c = cell_pre(A, rp, kv.y, kv.x - rp.off, dt);
-        slot = kv.x;
+        const Cell c = cell_pre(A, rp, kv.y, kv.x >> 16, dt);
+        slot = rp.off + (kv.x & 0xffff);
         cbase = cell_base(c, A.ny, A.nz, PK);
         fx = c.fx;
         fy = c.fy;
         fz = c.fz;
         if (BWD) {
-            // dout = dL/dc c (1 - c) with the colour c the forward left in the sample record
-            // (the same kernel arithmetic on the same operands, so the layer-3 recompute is skipped)
-            const float4 gc = A.sgrad[slot], cv = A.samp[slot];
-            d0 = gc.y * cv.y * (1.0f - cv.y);
-            d1 = gc.z * cv.z * (1.0f - cv.z);
-            d2 = gc.w * cv.w * (1.0f - cv.w);
+            // dout = dL/dc c (1 - c), formed by the compositing backward with the forward's colour c
+            const float4 gc = A.sgrad[slot];
+            d0 = gc.y;
+            d1 = gc.z;
+            d2 = gc.w;
         }
 #pragma unroll
         for (int q = 0; q < (cached ? 0 : 4); ++q) {   // corner pairs (x bit, y bit) with z = 0, 1 adjacent
@@ -523,6 +522,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             fence_after();
             if (!ok) break;
             const int slot = S.sm.slot[i & 3][r];
+            const float tau = slot >= 0 ? __ldg(A.stau + slot) : 0.0f;   // goes with the colour
             // ---- layer 1: Z1 = X W1 ----
             if (r == 0) {
 #pragma unroll 1
@@ -587,12 +587,9 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             if (!wait_mma()) { ok = false; break; }
             float o[16];
             tmem_ld16(taddr(tb, warp, F_O), o);
-            if (slot >= 0) {
-                float *sp = reinterpret_cast<float *>(A.samp + slot);
-                sp[1] = sigmoidf_(o[0] + S.sm.b3[0]);
-                sp[2] = sigmoidf_(o[1] + S.sm.b3[1]);
-                sp[3] = sigmoidf_(o[2] + S.sm.b3[2]);
-            }
+            if (slot >= 0)
+                A.scol[slot] = make_float4(sigmoidf_(o[0] + S.sm.b3[0]), sigmoidf_(o[1] + S.sm.b3[1]),
+                                           sigmoidf_(o[2] + S.sm.b3[2]), tau);
             group_sync();   // TMEM reads and panel reads done before this group's next MMAs
         }
         if (r == 0 && A.xcache) bulk_wait_all();   // the copies are complete before the kernel ends
@@ -639,7 +636,6 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
                 commit(&S.sm.mma);
             }
             if (!wait_mma()) { ok = false; break; }
-            if (!BWD && tid == 0) mbar_arrive(&S.sm.empty[b]);   // X[b] is free once layer 1 is done
             // ---- epilogue 1: H1 = relu(Z1), my 64 columns ----
             uint32_t m1lo = 0u, m1hi = 0u;   // ReLU masks of my 64 columns
 #pragma unroll 1
@@ -706,30 +702,6 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
 #pragma unroll
                     for (int k = 0; k < 32; k += 8) panel_store8(S.dz2 + hc * kPanelBytes, r, 32 * g + k, dz + k);
                 }
-            }
-            if (!BWD) {
-                consumer_publish();
-                // ---- layer 3: O = H2 W3 (N = 16, columns 0-2 used) ----
-                if (tid == 0) {
-#pragma unroll 1
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma(tb + COL_O, desc_kmajor(h2_, kk), desc_mnmajor(w3p_, kk), idesc_bf16(128, 16, 0, 1),
-                            kk > 0);
-                    commit(&S.sm.mma);
-                }
-                if (!wait_mma()) { ok = false; break; }
-                float o[16];
-                tmem_ld16(taddr(tb, warp, COL_O), o);
-                const float c0 = sigmoidf_(o[0] + S.sm.b3[0]), c1 = sigmoidf_(o[1] + S.sm.b3[1]),
-                            c2 = sigmoidf_(o[2] + S.sm.b3[2]);
-                if (slot >= 0 && hc == 0) {
-                    float *sp = reinterpret_cast<float *>(A.samp + slot);
-                    sp[1] = c0;
-                    sp[2] = c1;
-                    sp[3] = c2;
-                }
-                consumer_sync();   // TMEM reads done before the next tile's MMAs
-                continue;
             }
             // ---- backward: H2 and dZ2 published for batch A ----
             consumer_publish();

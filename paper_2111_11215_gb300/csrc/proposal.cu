@@ -77,14 +77,17 @@ __global__ void __launch_bounds__(256) weight_bins_kernel(RenderArgs A, int nbin
         for (int b = lane; b < nbins; b += 32) bins[wib][b] = 0.0f;
         __syncwarp();
         float carry = 0.0f, wsum = 0.0f;
-        for (int base = 0; base < rr.n; base += 32) {
-            const int k = base + lane;
-            const float tau = k < rr.n ? A.samp[rr.off + k].x : 0.0f;
+        const int nk = A.rayk[r].x;   // the kept samples; the others have weight 0
+        const size_t off = (size_t)r * A.cap;
+        for (int base = 0; base < nk; base += 32) {
+            const int j = base + lane;
+            const float tau = j < nk ? A.stau[off + j] : 0.0f;
             const float incl = warp_incl_scan(tau, lane);
             float excl = __shfl_up_sync(0xffffffffu, incl, 1);
             if (lane == 0) excl = 0.0f;
             const float w = expf(-(carry + excl)) * -expm1f(-tau);
-            if (k < rr.n) {
+            if (j < nk) {
+                const int k = A.kidx[off + j];
                 int b = (int)floor(__dmul_rn(__dadd_rn((double)k, (double)rr.p), bin_scale));
                 b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
                 atomicAdd(&bins[wib][b], w);
@@ -561,7 +564,10 @@ int dvgo_weight_bins(const dvgo_params *p, const dvgo_grid_desc *dd, int n_rays,
     A.R = n_rays;
     A.step = p->step;
     A.rays = reinterpret_cast<RayRec *>(b + L.rays);
-    A.samp = reinterpret_cast<float4 *>(b + L.samp);
+    A.cap = (int)cap;
+    A.rayk = reinterpret_cast<int2 *>(b + L.rayk);
+    A.stau = reinterpret_cast<float *>(b + L.stau);
+    A.kidx = reinterpret_cast<unsigned short *>(b + L.kidx);
     A.texit = reinterpret_cast<double *>(b + L.texit);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int blocks = (n_rays + 7) / 8;

@@ -122,28 +122,30 @@ void launch_ray_setup(const RenderArgs &A, const float *rays_o, const float *ray
                                                       (double)cap, A.ts ? A.n_expl : -1);
 }
 
-WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache) {
+WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache, size_t mask_words) {
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     WsLayout L;
+    memset(&L, 0, sizeof(L));
     size_t o = 0;
+    const size_t n = (size_t)(R > 0 ? R : 1);
     L.header = o; o += up(sizeof(WsHeader));
-    L.rays = o; o += up(sizeof(RayRec) * (size_t)(R > 0 ? R : 1));
-    L.rayout = o; o += up(sizeof(float4) * (size_t)(R > 0 ? R : 1));
-    size_t S = (size_t)(max_samples > 0 ? max_samples : 1);
-    L.pe = L.texit = 0;
+    L.rays = o; o += up(sizeof(RayRec) * n);
+    L.rayout = o; o += up(sizeof(float4) * n);
+    const size_t S = (size_t)(max_samples > 0 ? max_samples : 1);
     if (mode == DVGO_MODE_FINE) {
-        L.pe = o; o += up(sizeof(float) * kPeStride * (size_t)(R > 0 ? R : 1));
-        L.texit = o; o += up(sizeof(double) * (size_t)(R > 0 ? R : 1));
-        L.samp = o; o += up(sizeof(float4) * S);
+        L.pe = o; o += up(sizeof(float) * kPeStride * n);
+        L.texit = o; o += up(sizeof(double) * n);
+        L.rayk = o; o += up(sizeof(int2) * n);
+        L.stau = o; o += up(sizeof(float) * S);
+        L.kidx = o; o += up(sizeof(unsigned short) * S);
+        L.scol = o; o += up(sizeof(float4) * S);
         L.sgrad = o; o += up(sizeof(float4) * S);
         L.kept = o; o += up(sizeof(int2) * S);
-    } else {
-        L.samp = L.sgrad = L.kept = 0;
     }
     // last; counted in total, so the allocation-free forward's static scratch includes it even
     // though that forward (no auxiliary losses) never writes it
-    L.rtarget = o; o += up(sizeof(float4) * (size_t)(R > 0 ? R : 1));
-    L.xcache = 0;
+    L.rtarget = o; o += up(sizeof(float4) * n);
+    if (mask_words > 0 && mode == DVGO_MODE_FINE) { L.mask = o; o += up(sizeof(unsigned) * mask_words); }
     if (xcache && mode == DVGO_MODE_FINE) {   // 128 kept samples per tile, a 16 KiB panel each
         o = (o + 1023) & ~(size_t)1023;
         L.xcache = o;

@@ -1,6 +1,6 @@
 // touched.cu -- exact counts of the lattice points one fine-stage render reads: the density grid's
 // points at the corners of every sample outside the known free space that the density pass did
-// not terminate (a terminated sample's slot holds tau = +inf), and the feature grid's points at
+// not terminate (the density pass leaves the first terminated sample's index per ray), and the feature grid's points at
 // the corners of every kept sample (the sizes behind the minimum HBM bytes of a step).
 //
 // Runs after a forward on its workspace: the per-ray records give every sample's fixed-point
@@ -28,10 +28,10 @@ __global__ void __launch_bounds__(256) touched_density_kernel(RenderArgs A, uint
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int ray = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; ray < A.R; ray += nwarps) {
         const RayRec &rr = A.rays[ray];
-        for (int k = lane; k < rr.n; k += 32) {
+        const int kend = min(rr.n, A.rayk[ray].y);   // the first terminated sample: it and every later one are left out
+        for (int k = lane; k < kend; k += 32) {
             long long u[3];
             float dt;
-            if (isinf(A.samp[rr.off + k].x)) break;   // terminated: this and every later sample
             sample_fx(A, rr, ray, k, dt, u);
             if (A.fs_density && known_free(A, u)) continue;
             mark_cell(bm, cell_from_fx(u, A.nx, A.ny, A.nz), A.ny, A.nz);
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) touched_feat_kernel(RenderArgs A, uint32_
         const int2 kv = A.kept[e];
         const RayRec &rr = A.rays[kv.y];
         float dt;
-        mark_cell(bm, sample_cell(A, rr, kv.y, kv.x - rr.off, dt), A.ny, A.nz);
+        mark_cell(bm, sample_cell(A, rr, kv.y, kv.x >> 16, dt), A.ny, A.nz);
     }
 }
 
