@@ -146,7 +146,7 @@ typedef struct {
                             DVGO_MODE_FINE: colour = MLP(interp(x, V_feat), PE(d))
                             (Sec. 4.2 Eq. fine_queries)                                          */
     int rgb_act;         /* coarse: 0 = identity (the paper states no activation), 1 = sigmoid   */
-    int mlp_prec;        /* fine: DVGO_MLP_FP32 (SIMT FP32) or DVGO_MLP_BF16 (tensor cores,
+    int mlp_prec;        /* fine: DVGO_MLP_FP32 (FP32 arithmetic) or DVGO_MLP_BF16 (tensor cores,
                             BF16 operands, FP32 accumulation)                                    */
     int n_freq_dir;      /* fine: positional-encoding frequencies on d (Supp. A: k_d = 4)        */
     int hidden;          /* fine: MLP width; this build supports 128 (Supp. A)                   */
@@ -169,7 +169,8 @@ typedef struct {
     int n_freq_pos;      /* fine: positional-encoding frequencies on the query point x (Sec. 4.2
                             Eq. fine_queries_rgb, Supp. A: k_x = 5); 0 leaves x out of the MLP
                             input.  This build supports 0 and 5.                                 */
-    /* Failure detection of the tensor-core colour kernels (DVGO_MLP_BF16; not part of the method).
+    /* Failure detection of the tensor-core colour kernels (DVGO_MLP_BF16, and the forward of DVGO_MLP_FP32;
+     * not part of the method).
      * Every device-side wait of those kernels (an mbarrier phase: the producers' tile, the
      * consumers' release of a buffer, the completion of an MMA batch) gives up after
      * wait_limit_us microseconds (0: the default, 2 s); the kernel then stops its CTA's work, waits
@@ -177,7 +178,7 @@ typedef struct {
      * word (dvgo_workspace_status then returns DVGO_ERR_DEVICE until the next forward) and returns;
      * the gradients or colours of that call are incomplete.  Range 0 .. 60,000,000.
      * test_withhold_tile (testing aid, 0 in normal use): k > 0 makes one producer thread of the
-     * colour kernels withhold its arrival on tile k - 1, so that the consumers' wait for that tile
+     * DVGO_MLP_BF16 colour kernels withhold its arrival on tile k - 1, so that the consumers' wait for that tile
      * runs out -- the failure path above, taken on purpose. */
     int wait_limit_us;
     int test_withhold_tile;

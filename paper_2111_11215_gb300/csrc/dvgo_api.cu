@@ -10,7 +10,7 @@
 
 namespace dvgo {
 
-void launch_fine_colour_fwd_simt(const RenderArgs &A, cudaStream_t s);
+void launch_fine_colour_fwd_fp32(const RenderArgs &A, cudaStream_t s);
 void launch_fine_colour_bwd_simt(const RenderArgs &A, cudaStream_t s);
 int launch_fine_colour_fwd_tc(const RenderArgs &A, cudaStream_t s);
 int launch_fine_colour_bwd_tc(const RenderArgs &A, cudaStream_t s);
@@ -348,7 +348,7 @@ int dvgo_render_fwd(const dvgo_params *p, const dvgo_grid_desc *dd, const float 
         if (p->mlp_prec == DVGO_MLP_BF16) {
             if ((st = launch_fine_colour_fwd_tc(A, s))) return st;
         } else {
-            launch_fine_colour_fwd_simt(A, s);
+            launch_fine_colour_fwd_fp32(A, s);
         }
         launch_fine_composite_fwd(A, s);
     }

@@ -1,4 +1,5 @@
-// fine_simt.cu -- colour queries of the fine stage with the FP32 (SIMT) shallow MLP.
+// fine_simt.cu -- backward of the fine stage's colour queries with the FP32 (SIMT) shallow MLP (the
+// forward is fine_tc_fp32.cu).
 //
 // Sec. 4.2 Eq. fine_queries_rgb and Supp. A: c = MLP(interp(x, V_feat), PE(d)[, PE(x)]) with D = 12
 // feature channels, k_d = 4 direction frequencies, optionally k_x = 5 frequencies on the query
@@ -13,8 +14,7 @@
 // is read with 16-byte vector loads; W1/W2 rows have stride 132 (a multiple of 4 that is not a
 // multiple of 32) to spread the transposed reads of the backward over banks.
 //
-// Backward per tile: recompute gather + forward, then
-//   dout = dL/dc * c (1 - c)                        (sigmoid)
+// Per tile: recompute gather + hidden layers, then, with dout = dL/dc c (1 - c) from the compositing backward,
 //   dW3 += H2^T dout, db3 += sum dout
 //   dZ2 = (dout W3^T) * [Z2 > 0],  dW2 += H1^T dZ2,  db2 += sum dZ2
 //   dZ1 = (dZ2 W2^T) * [Z1 > 0],   dW1|b1 += X^T dZ1
@@ -221,41 +221,6 @@ __device__ __forceinline__ void gemm_fwd(const float *InT, const float *W, const
         int col = j < 4 ? c0 + j : c1 + j - 4;
         st4(OutT + col * LDA + s0, make_float4(fmaxf(acc[0][j], 0.0f), fmaxf(acc[1][j], 0.0f),
                                                fmaxf(acc[2][j], 0.0f), fmaxf(acc[3][j], 0.0f)));
-    }
-}
-
-// Output layer for sample s = tid & 63, channel ch = tid >> 6 (< 3): o = h2 . W3[:, ch] + b3.
-template <bool PEX>
-__device__ __forceinline__ float out_logit(const Smem<PEX> &S, int s, int ch) {
-    float o = S.b3[ch];
-#pragma unroll 8
-    for (int j = 0; j < HID; ++j) o = fmaf(S.h2[j * LDA + s], S.w3[j * 3 + ch], o);
-    return o;
-}
-
-template <typename FeatT, bool PEX, bool PK>
-__global__ void __launch_bounds__(NT, 1) fine_colour_fwd_kernel(RenderArgs A) {
-    constexpr int K1 = Dims<PEX>::K1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem<PEX> &S = *reinterpret_cast<Smem<PEX> *>(smem_raw);
-    load_weights(S, A);
-    const int n_kept = A.hdr->n_kept;
-    const int ntiles = (n_kept + TM - 1) / TM;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        __syncthreads();
-        gather_tile<FeatT, PEX, PK>(S, A, tile, n_kept);
-        __syncthreads();
-        gemm_fwd<K1>(S.xt, S.w1, nullptr, S.h1);
-        __syncthreads();
-        gemm_fwd<HID>(S.h1, S.w2, S.b2, S.h2);
-        __syncthreads();
-        int s = threadIdx.x & 63, ch = threadIdx.x >> 6;
-        if (ch < 3 && S.slot[s] >= 0) {
-            float c = sigmoidf_(out_logit(S, s, ch));
-            reinterpret_cast<float *>(A.scol + S.slot[s])[ch] = c;
-        } else if (ch == 3 && S.slot[s] >= 0) {
-            reinterpret_cast<float *>(A.scol + S.slot[s])[3] = A.stau[S.slot[s]];   // tau goes with the colour
-        }
     }
 }
 
@@ -479,34 +444,24 @@ void launch_persistent(void (*kernel)(RenderArgs), int kind, const RenderArgs &A
     kernel<<<num_sms(), NT, sizeof(Smem<PEX>), s>>>(A);
 }
 
-template <bool BWD, bool PEX, bool PK>
+template <bool PEX, bool PK>
 void launch_colour(const RenderArgs &A, cudaStream_t s) {
-    const int kind = BWD ? DVGO_K_FINE_COLOUR_BWD : DVGO_K_FINE_COLOUR_FWD;
-    if (A.cdtype == DVGO_DTYPE_BF16)
-        launch_persistent<PEX>(BWD ? fine_colour_bwd_kernel<__nv_bfloat16, PEX, PK>
-                                   : fine_colour_fwd_kernel<__nv_bfloat16, PEX, PK>,
-                               kind, A, s);
-    else
-        launch_persistent<PEX>(BWD ? fine_colour_bwd_kernel<float, PEX, PK> : fine_colour_fwd_kernel<float, PEX, PK>,
-                               kind, A, s);
-}
-
-template <bool BWD>
-void launch_colour_any(const RenderArgs &A, cudaStream_t s) {
-    const bool pex = A.nfreq_pos > 0;
-    if (A.packed) {
-        if (pex) launch_colour<BWD, true, true>(A, s);
-        else launch_colour<BWD, false, true>(A, s);
-    } else {
-        if (pex) launch_colour<BWD, true, false>(A, s);
-        else launch_colour<BWD, false, false>(A, s);
-    }
+    launch_persistent<PEX>(A.cdtype == DVGO_DTYPE_BF16 ? fine_colour_bwd_kernel<__nv_bfloat16, PEX, PK>
+                                                       : fine_colour_bwd_kernel<float, PEX, PK>,
+                           DVGO_K_FINE_COLOUR_BWD, A, s);
 }
 
 }  // namespace
 
-void launch_fine_colour_fwd_simt(const RenderArgs &A, cudaStream_t s) { launch_colour_any<false>(A, s); }
-
-void launch_fine_colour_bwd_simt(const RenderArgs &A, cudaStream_t s) { launch_colour_any<true>(A, s); }
+void launch_fine_colour_bwd_simt(const RenderArgs &A, cudaStream_t s) {
+    const bool pex = A.nfreq_pos > 0;
+    if (A.packed) {
+        if (pex) launch_colour<true, true>(A, s);
+        else launch_colour<false, true>(A, s);
+    } else {
+        if (pex) launch_colour<true, false>(A, s);
+        else launch_colour<false, false>(A, s);
+    }
+}
 
 }  // namespace dvgo

@@ -1,0 +1,380 @@
+// fine_tc_fp32.cu -- forward colour queries of the fine stage with the FP32 MLP, on the tensor cores.
+//
+// Same function as the FP32 contract asks (Sec. 4.2 Eq. fine_queries_rgb, Supp. A: 39 inputs, or 72 with
+// PE(x, 5); two hidden layers of 128 with ReLU, sigmoid output).  Every FP32 operand x is written as
+// three BF16 numbers x = hi + mid + lo, each the rounding to nearest of what the ones before leave (24
+// significand bits in all, so the sum is x exactly unless lo falls below the smallest BF16), and a
+// product of two operands as the six BF16 products hi hi, hi mid, mid hi, mid mid, hi lo, lo hi; the
+// three left out are below 2^-25 of it.  tcgen05 MMAs accumulate in FP32, cutting what falls below the
+// accumulator's last bit, so the small products go first, into an accumulator of their own size, and the
+// 128-wide contraction keeps two accumulators (64 inputs each) that are added with rounding.  Colours
+// and gradients are as close to FP64 as with the FP32 FMA chains (rgb 3.4e-8 relative either way).
+//
+// Bound: six MMAs for each FP32 one still leave the CUDA cores' FP32 rate (128 FMA a clock per SM, of
+// which the SIMT kernel before reached 45 %) far behind.  FWD_NUMBERS
+//
+// Persistent CTAs of 384 threads walk tiles of M = 128 kept samples, thread r (mod 128) of a warpgroup
+// owning row r (TMEM lane r).  Warps 8-11 gather the next tile's input rows and split them into shared
+// memory; warps 0-7 (two per row, 64 columns each) issue the MMAs (thread 0) and run the epilogues:
+//   Z1 = X W1 (bias in a constant-1 column) -> H1 = relu(Z1), split, to tensor memory (the next A operand)
+//   -> Z2 = H1 W2 -> o = relu(Z2 + b2) W3 + b3 on the CUDA cores -> c = sigmoid(o).
+// Layer 1 of the next tile runs while the last epilogue does.  Shared memory: W2 split 96 KB, W1 and X
+// split 48 KB each (64 KB with PE(x)) as 16-column blocks in 128-byte-swizzled panels (tc_helpers.cuh).
+// TMEM columns: Z1 [0, 128), then H1 hi / mid / lo [0, 192) over it; Z2 [192, 320) and [320, 448).
+
+#include "dvgo_internal.cuh"
+#include "fine_gather.cuh"
+#include "tc_helpers.cuh"
+
+namespace dvgo {
+
+namespace {
+
+using namespace tc;
+
+constexpr int TM = 128, NC = 256, NP = 128;
+constexpr int HID = 128, FEAT = 12, NFX = 5;
+constexpr int PX = FEAT + 3 + 6 * 4;   // 39: first input of the PE(x) block
+constexpr uint32_t COL_Z1 = 0, COL_H1 = 0, COL_Z2 = 192, NCOLS = 512;
+
+template <bool PEX>
+struct SplitDims {
+    static constexpr int IN = PX + (PEX ? 3 + 6 * NFX : 0);   // inputs; column IN is the constant 1 (bias)
+    static constexpr int KB = (IN + 1 + 15) / 16;             // 16-column blocks of a split: 3 or 5
+    static constexpr int PANELS = (3 * KB + 3) / 4;           // of the three splits, block s KB + kb in order
+    static constexpr int AUX = 3 * KB;                        // a block left over in the last panel: (W3, b2)
+    static_assert(AUX < 4 * PANELS, "a free block for the output layer");
+};
+
+struct SplitSmall {
+    float part[TM][3];   // the second half-row's share of the output layer
+    uint64_t full, empty, mma;
+    uint32_t tmem_base;
+    int abort;
+    float b3[4];
+};
+
+template <bool PEX>
+constexpr size_t split_smem() {
+    return (size_t)(6 + 2 * SplitDims<PEX>::PANELS) * kPanelBytes + sizeof(SplitSmall) + 1023;
+}
+static_assert(split_smem<true>() <= 232448, "one CTA per SM (227 KB of shared memory)");
+
+// Eight FP32 values as three BF16 chunks of 16 bytes: hi, mid, lo.
+__device__ __forceinline__ void split8(const float *v, uint4 (&q)[3]) {
+    uint32_t w[3][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float a = v[2 * i], b = v[2 * i + 1];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            w[s][i] = pack_bf16(a, b);
+            a = __fsub_rn(a, __uint_as_float(w[s][i] << 16));
+            b = __fsub_rn(b, __uint_as_float(w[s][i] & 0xffff0000u));
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) q[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+// Split s, columns [8 c, 8 c + 8) of row `row` of an operand of KB blocks a split.
+template <int KB>
+__device__ __forceinline__ uint4 *split_chunk(unsigned char *base, int s, int row, int c) {
+    const int q = s * KB + (c >> 1);
+    return reinterpret_cast<uint4 *>(base + (q >> 2) * kPanelBytes + panel_offset(row, (q & 3) * 16 + (c & 1) * 8));
+}
+
+__device__ __forceinline__ void arrive(uint64_t *mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
+}
+
+// Barrier among the 256 consumer threads.
+__device__ __forceinline__ void consumer_sync() {
+    fence_before();
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    fence_after();
+}
+
+template <typename FeatT, bool PEX, bool PK>
+__global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(RenderArgs A) {
+    using D = SplitDims<PEX>;
+    constexpr int KB = D::KB;
+    const int n_kept = A.hdr->n_kept;
+    const int ntiles = (n_kept + TM - 1) / TM;
+    if ((int)blockIdx.x >= ntiles) return;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *w2t = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *w1t = w2t + 6 * kPanelBytes, *xs = w1t + D::PANELS * kPanelBytes;
+    SplitSmall &S = *reinterpret_cast<SplitSmall *>(xs + D::PANELS * kPanelBytes);
+    const int tid = threadIdx.x, warp = tid >> 5;
+    if (tid == 0) {
+        mbar_init(&S.full, NP);
+        mbar_init(&S.empty, 1);
+        mbar_init(&S.mma, 1);
+        S.abort = 0;
+    }
+    if (warp == 0) tmem_alloc(&S.tmem_base, NCOLS);
+    // barriers initialised: the producers gather the first tile while the consumers stage the weights
+    fence_before();
+    __syncthreads();
+    fence_after();
+    bool ok = true;
+    uint32_t mphase = 0;
+
+    if (tid >= NC) {
+        // ------------------------------- producers -------------------------------
+        const int row = tid - NC;
+        auto kept_at = [&](int t) -> int2 {
+            const int e = t * TM + row;
+            return (t < ntiles && e < n_kept) ? A.kept[e] : make_int2(-1, -1);
+        };
+        int2 kv = kept_at(blockIdx.x);
+        RayPre rp = kv.y >= 0 ? ray_pre(A, kv.y) : RayPre{};
+        int i = 0;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
+            const int2 kv_next = kept_at(tile + gridDim.x);
+            float v[16 * KB];
+#pragma unroll
+            for (int k = 0; k < 16 * KB; ++k) v[k] = 0.0f;
+            if (kv.y >= 0) {
+                float dt;
+                const Cell c = cell_pre(A, rp, kv.y, kv.x >> 16, dt);
+                gather_features<FeatT, PK>(A, c, v);
+                const float4 *pe = reinterpret_cast<const float4 *>(A.pe + (size_t)kv.y * kPeStride);
+#pragma unroll
+                for (int k = 0; k < 7; ++k) {
+                    const float4 q4 = __ldg(pe + k);
+                    const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (4 * k + j < 27) v[FEAT + 4 * k + j] = q[j];
+                }
+                if constexpr (PEX) {
+                    // PE(x) of the world-space sample position: [x (3), sin(2^k x_c) (15), cos(2^k x_c) (15)]
+                    float xv[3];
+                    cell_world(A, c, xv);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        v[PX + a] = xv[a];
+                        pe_axis<NFX>(xv[a], v + PX + 3 + a * NFX, v + PX + 3 + 3 * NFX + a * NFX);
+                    }
+                }
+                v[D::IN] = 1.0f;
+            }
+            rp = kv_next.y >= 0 ? ray_pre(A, kv_next.y) : RayPre{};
+            kv = kv_next;
+            if (i >= 1 && !mbar_wait(&S.empty, (i - 1) & 1, A.wait_ns)) {
+                ok = false;
+                break;
+            }
+#pragma unroll
+            for (int c = 0; c < 2 * KB; ++c) {
+                uint4 q[3];
+                split8(v + 8 * c, q);
+#pragma unroll
+                for (int s = 0; s < 3; ++s) *split_chunk<KB>(xs, s, row, c) = q[s];
+            }
+            fence_async_smem();
+            arrive(&S.full);
+        }
+        if (!ok) atomicExch(&S.abort, 1);
+    } else {
+        // ------------------------------- consumers -------------------------------
+        // W1^T | b1 and W2^T split: (unit n, 8 input columns) per thread and turn
+        for (int t = tid; t < HID * (2 * KB + 16); t += NC) {
+            const int n = t & (HID - 1), c = t >> 7;
+            float v[8];
+            uint4 q[3];
+            if (c < 2 * KB) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = 8 * c + j;
+                    v[j] = k < D::IN ? A.w1[k * HID + n] : (k == D::IN ? A.b1[n] : 0.0f);
+                }
+                split8(v, q);
+#pragma unroll
+                for (int s = 0; s < 3; ++s) *split_chunk<KB>(w1t, s, n, c) = q[s];
+            } else {
+                const int c2 = c - 2 * KB;   // 0-15
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = A.w2[(8 * c2 + j) * HID + n];
+                split8(v, q);
+#pragma unroll
+                for (int s = 0; s < 3; ++s)
+                    *reinterpret_cast<uint4 *>(w2t + (2 * s + (c2 >> 3)) * kPanelBytes + panel_offset(n, (c2 & 7) * 8)) = q[s];
+            }
+        }
+        unsigned char *aux = w1t + (D::AUX >> 2) * kPanelBytes;   // per unit (W3 row, b2), 16 bytes in the free block
+        constexpr int aux_col = (D::AUX & 3) * 16;
+        if (tid < HID)
+            *reinterpret_cast<float4 *>(aux + panel_offset(tid, aux_col)) =
+                make_float4(A.w3[3 * tid], A.w3[3 * tid + 1], A.w3[3 * tid + 2], A.b2[tid]);
+        if (tid < 3) S.b3[tid] = A.b3[tid];
+        fence_async_smem();
+        consumer_sync();
+
+        const int r = tid & (TM - 1), hc = tid >> 7;
+        const uint32_t tb = S.tmem_base;
+        const uint32_t idesc = idesc_bf16(128, 128, 0, 0);
+        // the six products, smallest first: split of A, split of B
+        constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};
+        auto wait_mma = [&]() -> bool {
+            const bool w = mbar_wait(&S.mma, mphase, A.wait_ns);
+            mphase ^= 1;
+            fence_after();
+            return w;
+        };
+        auto issue_layer1 = [&]() {
+            uint32_t x_ = smem_u32(xs), w_ = smem_u32(w1t);
+            asm volatile("" : "+r"(x_), "+r"(w_));   // keeps the descriptors out of long-lived registers
+#pragma unroll
+            for (int p = 0; p < 6; ++p)
+#pragma unroll 1
+                for (int kk = 0; kk < KB; ++kk)
+                    mma(tb + COL_Z1, desc_kmajor(x_, PA[p] * KB + kk), desc_kmajor(w_, PB[p] * KB + kk), idesc,
+                        (p | kk) != 0);
+            commit(&S.mma);
+        };
+        int i = 0;
+        if (!mbar_wait(&S.full, 0, A.wait_ns)) ok = false;
+        fence_after();
+        if (ok && tid == 0) issue_layer1();
+        for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++i) {
+            // this row's sample slot and optical depth, needed at the end
+            const int e = tile * TM + r;
+            int slot = -1;
+            float tau = 0.0f;
+            if (hc == 0 && e < n_kept) {
+                const int2 kv = A.kept[e];
+                slot = kv.y * A.cap + (kv.x & 0xffff);
+                tau = __ldg(A.stau + slot);
+            }
+            if (!wait_mma()) { ok = false; break; }
+            if (tid == 0) arrive(&S.empty);   // X is free
+            // ---- epilogue 1: H1 = relu(Z1), split, over Z1 (read whole before any is overwritten) ----
+            {
+                float z[2][32];
+                tmem_ld32(taddr(tb, warp, COL_Z1 + 64 * hc), z[0]);
+                tmem_ld32(taddr(tb, warp, COL_Z1 + 64 * hc + 32), z[1]);
+                consumer_sync();
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    uint32_t w[3][16];
+#pragma unroll
+                    for (int k = 0; k < 32; k += 8) {
+                        float v[8];
+                        uint4 q[3];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) v[j] = fmaxf(z[g][k + j], 0.0f);
+                        split8(v, q);
+#pragma unroll
+                        for (int s = 0; s < 3; ++s) {
+                            w[s][k / 2] = q[s].x;
+                            w[s][k / 2 + 1] = q[s].y;
+                            w[s][k / 2 + 2] = q[s].z;
+                            w[s][k / 2 + 3] = q[s].w;
+                        }
+                    }
+#pragma unroll
+                    for (int s = 0; s < 3; ++s) tmem_st16(taddr(tb, warp, COL_H1 + 64 * s + 32 * hc + 16 * g), w[s]);
+                }
+                tmem_wait_st();
+                consumer_sync();
+            }
+            // ---- layer 2: Z2 = H1 W2, A = H1 from TMEM; inputs 0-63 and 64-127 in accumulators of their own ----
+            if (tid == 0) {
+                uint32_t w_ = smem_u32(w2t);
+                asm volatile("" : "+r"(w_));
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int p = 0; p < 6; ++p)
+#pragma unroll 1
+                        for (int kk = 4 * h; kk < 4 * h + 4; ++kk)
+                            mma_ts(tb + COL_Z2 + 128u * (uint32_t)h, tb + COL_H1 + 64u * PA[p] + 8u * (uint32_t)kk,
+                                   desc_kmajor(w_ + 2u * PB[p] * kPanelBytes, kk), idesc, p > 0 || kk > 4 * h);
+                commit(&S.mma);
+            }
+            if (!wait_mma()) { ok = false; break; }
+            // ---- layer 1 of the next tile, beside the last epilogue ----
+            if (tile + (int)gridDim.x < ntiles) {
+                if (!mbar_wait(&S.full, (i + 1) & 1, A.wait_ns)) { ok = false; break; }
+                fence_after();
+                if (tid == 0) issue_layer1();
+            }
+            // ---- epilogue 2: relu(Z2 + b2) W3, my 64 columns; the two halves of a row join ----
+            float o[3] = {0.0f, 0.0f, 0.0f};
+            if (hc == 0) {
+                o[0] = S.b3[0];
+                o[1] = S.b3[1];
+                o[2] = S.b3[2];
+            }
+#pragma unroll 1
+            for (int g = 0; g < 2; ++g) {
+                const int col = 64 * hc + 32 * g;
+                float za[32], zb[32];
+                tmem_ld32(taddr(tb, warp, COL_Z2 + col), za);
+                tmem_ld32(taddr(tb, warp, COL_Z2 + 128 + col), zb);
+#pragma unroll
+                for (int k = 0; k < 32; ++k) {
+                    const float4 w = *reinterpret_cast<const float4 *>(aux + panel_offset(col + k, aux_col));
+                    const float h = fmaxf(za[k] + zb[k] + w.w, 0.0f);
+                    o[0] = fmaf(h, w.x, o[0]);
+                    o[1] = fmaf(h, w.y, o[1]);
+                    o[2] = fmaf(h, w.z, o[2]);
+                }
+            }
+            if (hc == 1) {
+                S.part[r][0] = o[0];
+                S.part[r][1] = o[1];
+                S.part[r][2] = o[2];
+            }
+            consumer_sync();
+            if (slot >= 0)
+                A.scol[slot] = make_float4(sigmoidf_(o[0] + S.part[r][0]), sigmoidf_(o[1] + S.part[r][1]),
+                                           sigmoidf_(o[2] + S.part[r][2]), tau);
+        }
+        if (!ok) atomicExch(&S.abort, 1);
+    }
+
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (S.abort != 0) {
+        if (tid == 0) atomicOr(&A.hdr->flags, 2);
+        // an MMA batch whose completion timed out may still be running: wait (bounded) once more
+        if (tid < NC) mbar_wait(&S.mma, mphase ^ 1, A.wait_ns);
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) tmem_dealloc(S.tmem_base, NCOLS);
+}
+
+template <typename FeatT, bool PEX, bool PK>
+void launch_split(const RenderArgs &A, cudaStream_t s) {
+    auto kern = fine_colour_fwd_split_kernel<FeatT, PEX, PK>;
+    constexpr int bytes = (int)split_smem<PEX>();
+    ensure_smem(reinterpret_cast<const void *>(kern), bytes);
+    ProfScope ps_(DVGO_K_FINE_COLOUR_FWD, s);
+    kern<<<num_sms(), NC + NP, bytes, s>>>(A);
+}
+
+}  // namespace
+
+void launch_fine_colour_fwd_fp32(const RenderArgs &A, cudaStream_t s) {
+    const bool bf = A.cdtype == DVGO_DTYPE_BF16, pex = A.nfreq_pos > 0;
+    if (A.packed) {
+        if (bf && pex) launch_split<__nv_bfloat16, true, true>(A, s);
+        else if (bf) launch_split<__nv_bfloat16, false, true>(A, s);
+        else if (pex) launch_split<float, true, true>(A, s);
+        else launch_split<float, false, true>(A, s);
+    } else {
+        if (bf && pex) launch_split<__nv_bfloat16, true, false>(A, s);
+        else if (bf) launch_split<__nv_bfloat16, false, false>(A, s);
+        else if (pex) launch_split<float, true, false>(A, s);
+        else launch_split<float, false, false>(A, s);
+    }
+}
+
+}  // namespace dvgo
