@@ -22,14 +22,14 @@
 
 #include <math.h>
 
-#include "df64.cuh"
 #include "dvgo_internal.cuh"
+#include "proposal_rays.cuh"
 
 namespace dvgo {
 
 namespace {
 
-constexpr int NB = 64;             // bins
+constexpr int NB = kPropBins;      // bins
 constexpr int NFQ = 6;             // PE frequencies on the bin centre
 constexpr int PIN = 3 + 6 * NFQ;   // 39
 constexpr int PK0 = PIN + 1;       // 40 with the bias column
@@ -123,31 +123,33 @@ struct PropSmem {
     float b3[4];              // [0] used; 4 floats keep the following arrays 16-byte aligned
     float xt[PK0 * PLD];    // inputs, feature-major
     float h0[PW * PLD], h1[PW * PLD], h2[PW * PLD];
-    float logit[PTM], dlog[PTM];
-    double t0[2], t1[2], dn[2][3];
-    int hit[2];
+    alignas(16) float logit[PTM];
+    alignas(16) float dlog[PTM];
+    ClipDf clip[PTM];       // rays of the CTA's current 64 tiles
 };
 
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 
-// OutT[n][row] = act(sum_k InT[k][row] W[k][n] + bias[n]) for 128 rows x 64 outputs.
-// Thread: rows 4 (t >> 3) .. +3, outputs 8 (t & 7) .. +7.
+// acc[i][j] = sum_k InT[k][4 ty + i] W[k][col(j)] + bias for 128 rows x 64 outputs, one FMA chain over k
+// per value.  Thread (ty, tx) = (t >> 3, t & 7): rows 4 ty .. +3, outputs 4 tx .. +3 and 32 + 4 tx .. +3, so
+// that each 16-byte load of a warp is one pass over the banks.
+__device__ __forceinline__ int out_col(int tx, int j) { return j < 4 ? 4 * tx + j : 28 + 4 * tx + j; }
+
 template <int K>
-__device__ __forceinline__ void ptile_gemm(const float *InT, const float *W, const float *bias, float *OutT) {
+__device__ __forceinline__ void ptile_gemm(const float *InT, const float *W, const float *bias, float (&acc)[4][8]) {
     const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
-    const int r0 = 4 * ty, c0 = 8 * tx;
-    float acc[4][8];
+    const int r0 = 4 * ty;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const float b = bias ? bias[c0 + j] : 0.0f;
+        const float b = bias ? bias[out_col(tx, j)] : 0.0f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i][j] = b;
     }
-#pragma unroll 4
+#pragma unroll 8
     for (int k = 0; k < K; ++k) {
         const float4 a = ld4(InT + k * PLD + r0);
-        const float4 x0 = ld4(W + k * PW + c0), x1 = ld4(W + k * PW + c0 + 4);
+        const float4 x0 = ld4(W + k * PW + 4 * tx), x1 = ld4(W + k * PW + 32 + 4 * tx);
         const float av[4] = {a.x, a.y, a.z, a.w};
         const float bv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
@@ -155,24 +157,56 @@ __device__ __forceinline__ void ptile_gemm(const float *InT, const float *W, con
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        st4(OutT + (c0 + j) * PLD + r0, make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]));
 }
 
-__device__ __forceinline__ void relu_inplace(float *T, int nfeat) {
-    for (int i = threadIdx.x; i < nfeat * PTM; i += PNT) {
-        const int f = i / PTM, r = i % PTM;
-        T[f * PLD + r] = fmaxf(T[f * PLD + r], 0.0f);
+// OutT = relu(acc).
+__device__ __forceinline__ void store_relu(const float (&acc)[4][8], float *OutT) {
+    const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        st4(OutT + out_col(tx, j) * PLD + 4 * ty,
+            make_float4(fmaxf(acc[0][j], 0.0f), fmaxf(acc[1][j], 0.0f), fmaxf(acc[2][j], 0.0f), fmaxf(acc[3][j], 0.0f)));
+}
+
+// OutT = acc [H > 0].
+__device__ __forceinline__ void store_masked(const float (&acc)[4][8], const float *HT, float *OutT) {
+    const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int o = out_col(tx, j) * PLD + 4 * ty;
+        const float4 h = ld4(HT + o);
+        st4(OutT + o, make_float4(h.x > 0.0f ? acc[0][j] : 0.0f, h.y > 0.0f ? acc[1][j] : 0.0f,
+                                  h.z > 0.0f ? acc[2][j] : 0.0f, h.w > 0.0f ? acc[3][j] : 0.0f));
     }
 }
 
-// sin / cos of an FP64 argument: reduce by 2 pi in FP64, evaluate in FP32.
-__device__ __forceinline__ void sincos_reduced(double a, float *s, float *c) {
-    const double two_pi = 6.283185307179586;
-    const double n = rint(a / two_pi);
-    const double red = fma(-n, two_pi, a);
-    sincosf((float)red, s, c);
+// g[i][j] += sum_r HT[kq + 32 i][r] DT[nq + 8 j][r], thread (kq, nq) = (t >> 3, t & 7), and gb +=
+// sum_r DT[nq + 8 w][r] with w the warp (kept by its lanes kq % 4 == 0).  The strided outputs put the
+// eight rows a warp reads at once in different banks (with eight neighbouring rows per thread every
+// load was eight-way conflicted, and the weight gradients took most of the backward).
+__device__ __forceinline__ void weight_grad(const float *HT, const float *DT, float (&g)[2][8], float &gb) {
+    const int kq = threadIdx.x >> 3, nq = threadIdx.x & 7, warp = threadIdx.x >> 5;
+#pragma unroll 2
+    for (int r = 0; r < PTM; r += 4) {
+        const float4 a0 = ld4(HT + kq * PLD + r), a1 = ld4(HT + (kq + 32) * PLD + r);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float4 d = ld4(DT + (nq + 8 * j) * PLD + r);
+            g[0][j] = fmaf(a0.x, d.x, fmaf(a0.y, d.y, fmaf(a0.z, d.z, fmaf(a0.w, d.w, g[0][j]))));
+            g[1][j] = fmaf(a1.x, d.x, fmaf(a1.y, d.y, fmaf(a1.z, d.z, fmaf(a1.w, d.w, g[1][j]))));
+            if (j == warp) gb += (d.x + d.y) + (d.z + d.w);
+        }
+    }
+}
+
+// sin / cos of the double-float argument a (|a| below a few hundred), reduced by 2 pi in double-float
+// arithmetic (2 pi = 6.28318548... - 1.7484556e-7, to 2^-47) and evaluated in FP32.  The reduction in FP64,
+// 18 per row, had the FP64 pipe busy for 17 us a tile.
+__device__ __forceinline__ void sincos_reduced(Df a, float *s, float *c) {
+    const Df two_pi = {6.283185482025146484375f, -1.74845553146951715e-7f};
+    const float n = rintf(a.hi * 0.15915494f);
+    const Df red = df_add(a, df_neg(df_mul_f(two_pi, n)));
+    sincosf(red.hi, s, c);
 }
 
 template <bool BWD>
@@ -188,8 +222,10 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
         const int k = i / PW, j = i % PW;
         S.w1[i] = P.w1[i];
         S.w2[i] = P.w2[i];
-        S.w1t[j * PW + k] = P.w1[i];
-        S.w2t[j * PW + k] = P.w2[i];
+        if (BWD) {
+            S.w1t[j * PW + k] = P.w1[i];
+            S.w2t[j * PW + k] = P.w2[i];
+        }
     }
     if (tid < PW) {
         S.b1[tid] = P.b1[tid];
@@ -208,63 +244,64 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
     const float invR = 1.0f / (float)P.R;
 
     const int ntiles = (P.R + 1) / 2;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    int kt = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++kt) {
         __syncthreads();
-        if (tid < 2) {
-            const int r = 2 * tile + tid;
-            int hit = 0;
-            if (r < P.R) {
-                const Clip c = clip_ray(P.box, P.ro, P.rd, r);
-                hit = c.hi > c.lo;
-                S.t0[tid] = c.lo;
-                S.t1[tid] = c.hi;
-                for (int a = 0; a < 3; ++a) S.dn[tid][a] = c.dn[a];
-            }
-            S.hit[tid] = hit;
+        if (kt % 64 == 0) {
+            if (tid < PTM)
+                clip_tile_rays(P.R, P.ro, P.rd, P.box.mn, P.box.mx, P.box.t_near, P.box.t_far, kt, S.clip);
+            __syncthreads();
         }
-        __syncthreads();
         // encode the bin centres: 2 threads per row
         {
-            const int row = tid >> 1, part = tid & 1, rl = row >> 6, bin = row & 63, r = 2 * tile + rl;
-            double x[3] = {0.0, 0.0, 0.0};
-            if (S.hit[rl]) {
-                const double t0 = S.t0[rl], t1 = S.t1[rl];
-                const double tb = __dadd_rn(t0, __ddiv_rn(__dmul_rn((double)bin + 0.5, __dsub_rn(t1, t0)), (double)NB));
-                for (int a = 0; a < 3; ++a)
-                    x[a] = __dadd_rn((double)P.ro[3 * r + a], __dmul_rn(tb, S.dn[rl][a]));
+            const int row = tid >> 1, part = tid & 1;
+            const ClipDf &cl = S.clip[2 * (kt % 64) + (row >> 6)];
+            Df x[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+            if (cl.hit) {
+                const Df tb = bin_centre(cl, row & 63);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) x[a] = bin_position(cl, tb, a);
             }
             if (part == 0) {
-                for (int a = 0; a < 3; ++a) S.xt[a * PLD + row] = (float)x[a];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) S.xt[a * PLD + row] = x[a].hi;
                 S.xt[PIN * PLD + row] = 1.0f;
             }
             // part 0: k = 0..2, part 1: k = 3..5 for every axis
+#pragma unroll
             for (int a = 0; a < 3; ++a)
+#pragma unroll
                 for (int kk = 0; kk < 3; ++kk) {
                     const int k = 3 * part + kk;
+                    const float p2 = (float)(1 << k);
                     float sv, cv;
-                    sincos_reduced(ldexp(x[a], k), &sv, &cv);
+                    sincos_reduced(Df{x[a].hi * p2, x[a].lo * p2}, &sv, &cv);
                     S.xt[(3 + a * NFQ + k) * PLD + row] = sv;
                     S.xt[(3 + 3 * NFQ + a * NFQ + k) * PLD + row] = cv;
                 }
         }
         __syncthreads();
-        ptile_gemm<PK0>(S.xt, S.w0, nullptr, S.h0);
+        float acc[4][8];
+        ptile_gemm<PK0>(S.xt, S.w0, nullptr, acc);
+        store_relu(acc, S.h0);
         __syncthreads();
-        relu_inplace(S.h0, PW);
+        ptile_gemm<PW>(S.h0, S.w1, S.b1, acc);
+        store_relu(acc, S.h1);
         __syncthreads();
-        ptile_gemm<PW>(S.h0, S.w1, S.b1, S.h1);
-        __syncthreads();
-        relu_inplace(S.h1, PW);
-        __syncthreads();
-        ptile_gemm<PW>(S.h1, S.w2, S.b2, S.h2);
-        __syncthreads();
-        relu_inplace(S.h2, PW);
-        __syncthreads();
-        if (tid < PTM) {
-            float o = S.b3[0];
-#pragma unroll 8
-            for (int j = 0; j < PW; ++j) o = fmaf(S.h2[j * PLD + tid], S.w3[j], o);
-            S.logit[tid] = o;
+        ptile_gemm<PW>(S.h1, S.w2, S.b2, acc);
+        if (BWD) store_relu(acc, S.h2);
+        {   // output layer: each thread's eight columns, then the eight threads of a row group
+            const int ty = tid >> 3, tx = tid & 7;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float o = 0.0f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) o = fmaf(fmaxf(acc[i][j], 0.0f), S.w3[out_col(tx, j)], o);
+                o += __shfl_xor_sync(0xffffffffu, o, 1);
+                o += __shfl_xor_sync(0xffffffffu, o, 2);
+                o += __shfl_xor_sync(0xffffffffu, o, 4);
+                if (tx == i) S.logit[4 * ty + i] = o + S.b3[0];
+            }
         }
         __syncthreads();
         // softmax per ray (warp 0: ray 0, warp 1: ray 1), loss, dlogit
@@ -278,7 +315,7 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
                 const float e0 = expf(l0 - m), e1 = expf(l1 - m);
                 const float z = warp_sum(e0 + e1);
                 float p0 = e0 / z, p1 = e1 / z;
-                const bool hit = S.hit[rl] != 0;
+                const bool hit = S.clip[2 * (kt % 64) + rl].hit != 0;
                 if (!hit) p0 = p1 = 1.0f / NB;
                 if (!BWD && P.probs) {
                     P.probs[(size_t)r * NB + lane] = p0;
@@ -306,127 +343,31 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
         }
         if (!BWD) continue;
         __syncthreads();
-        // output layer: dW3, db3; dH2 = dlogit w3^T [H2 > 0] (in place over h2 is not possible: H2
-        // is needed for dW3 first)
-        if (tid < PW) {
+        // output layer: dW3 += H2^T dlogit, db3 += sum dlogit, and dZ2 = dlogit w3^T [H2 > 0] over H2: unit
+        // t >> 2, every fourth group of four rows
+        {
+            const int f = tid >> 2, part = tid & 3;
+            const float w3 = S.w3[f];
             float a = 0.0f;
-            for (int r = 0; r < PTM; r += 4) {
-                const float4 h = ld4(S.h2 + tid * PLD + r);
-                a = fmaf(h.x, S.dlog[r], fmaf(h.y, S.dlog[r + 1], fmaf(h.z, S.dlog[r + 2], fmaf(h.w, S.dlog[r + 3], a))));
+#pragma unroll
+            for (int r = 4 * part; r < PTM; r += 16) {
+                const float4 h = ld4(S.h2 + f * PLD + r), d = ld4(S.dlog + r);
+                a = fmaf(h.x, d.x, fmaf(h.y, d.y, fmaf(h.z, d.z, fmaf(h.w, d.w, a))));
+                if (f == 0) gb3 += (d.x + d.y) + (d.z + d.w);
+                st4(S.h2 + f * PLD + r, make_float4(h.x > 0.0f ? d.x * w3 : 0.0f, h.y > 0.0f ? d.y * w3 : 0.0f,
+                                                    h.z > 0.0f ? d.z * w3 : 0.0f, h.w > 0.0f ? d.w * w3 : 0.0f));
             }
             g3 += a;
         }
-        if (tid == PW) {
-            float a = 0.0f;
-            for (int r = 0; r < PTM; ++r) a += S.dlog[r];
-            gb3 += a;
-        }
         __syncthreads();
-        for (int i = tid; i < PW * PTM; i += PNT) {
-            const int f = i / PTM, r = i % PTM;
-            const float h = S.h2[f * PLD + r];
-            S.h2[f * PLD + r] = h > 0.0f ? S.dlog[r] * S.w3[f] : 0.0f;   // dZ2
-        }
+        weight_grad(S.h1, S.h2, g2, gb2);              // dW2 += H1^T dZ2, db2 += sum dZ2
+        ptile_gemm<PW>(S.h2, S.w2t, nullptr, acc);     // dH1 = dZ2 W2^T
+        __syncthreads();                               // all reads of H1 (dW2) and dZ2 done
+        store_masked(acc, S.h1, S.h1);                 // dZ1 over H1
         __syncthreads();
-        // dW2 += H1^T dZ2, db2 += sum dZ2 ; thread: inputs 2 kq, 2 kq + 1, outputs 8 nq .. +7
-        {
-            const int kq = tid >> 3, nq = tid & 7;
-            for (int r = 0; r < PTM; r += 4) {
-                const float4 a0 = ld4(S.h1 + (2 * kq) * PLD + r), a1 = ld4(S.h1 + (2 * kq + 1) * PLD + r);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float4 d = ld4(S.h2 + (8 * nq + j) * PLD + r);
-                    g2[0][j] = fmaf(a0.x, d.x, fmaf(a0.y, d.y, fmaf(a0.z, d.z, fmaf(a0.w, d.w, g2[0][j]))));
-                    g2[1][j] = fmaf(a1.x, d.x, fmaf(a1.y, d.y, fmaf(a1.z, d.z, fmaf(a1.w, d.w, g2[1][j]))));
-                }
-            }
-            if (tid < PW) {
-                float a = 0.0f;
-                for (int r = 0; r < PTM; r += 4) {
-                    const float4 d = ld4(S.h2 + tid * PLD + r);
-                    a += (d.x + d.y) + (d.z + d.w);
-                }
-                gb2 += a;
-            }
-        }
-        // dH1 = dZ2 W2^T -> xt is free: use h0's partner buffers carefully: write dZ1 into S.xt? No:
-        // xt is still needed for dW0.  dH1 goes to a register tile, then over h1 after a barrier.
-        {
-            const int ty = tid >> 3, tx = tid & 7, r0 = 4 * ty, c0 = 8 * tx;
-            float acc[4][8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-#pragma unroll 4
-            for (int k = 0; k < PW; ++k) {
-                const float4 a = ld4(S.h2 + k * PLD + r0);
-                const float4 x0 = ld4(S.w2t + k * PW + c0), x1 = ld4(S.w2t + k * PW + c0 + 4);
-                const float av[4] = {a.x, a.y, a.z, a.w};
-                const float bv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-            }
-            __syncthreads();   // all reads of h1 (dW2) and h2 done
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float4 h = ld4(S.h1 + (c0 + j) * PLD + r0);
-                st4(S.h1 + (c0 + j) * PLD + r0,
-                    make_float4(h.x > 0.0f ? acc[0][j] : 0.0f, h.y > 0.0f ? acc[1][j] : 0.0f,
-                                h.z > 0.0f ? acc[2][j] : 0.0f, h.w > 0.0f ? acc[3][j] : 0.0f));
-            }
-        }
-        __syncthreads();
-        // dW1 += H0^T dZ1, db1 += sum dZ1
-        {
-            const int kq = tid >> 3, nq = tid & 7;
-            for (int r = 0; r < PTM; r += 4) {
-                const float4 a0 = ld4(S.h0 + (2 * kq) * PLD + r), a1 = ld4(S.h0 + (2 * kq + 1) * PLD + r);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float4 d = ld4(S.h1 + (8 * nq + j) * PLD + r);
-                    g1[0][j] = fmaf(a0.x, d.x, fmaf(a0.y, d.y, fmaf(a0.z, d.z, fmaf(a0.w, d.w, g1[0][j]))));
-                    g1[1][j] = fmaf(a1.x, d.x, fmaf(a1.y, d.y, fmaf(a1.z, d.z, fmaf(a1.w, d.w, g1[1][j]))));
-                }
-            }
-            if (tid < PW) {
-                float a = 0.0f;
-                for (int r = 0; r < PTM; r += 4) {
-                    const float4 d = ld4(S.h1 + tid * PLD + r);
-                    a += (d.x + d.y) + (d.z + d.w);
-                }
-                gb1 += a;
-            }
-        }
-        // dZ0 = (dZ1 W1^T) [H0 > 0], over h2 (free now)
-        {
-            const int ty = tid >> 3, tx = tid & 7, r0 = 4 * ty, c0 = 8 * tx;
-            float acc[4][8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-#pragma unroll 4
-            for (int k = 0; k < PW; ++k) {
-                const float4 a = ld4(S.h1 + k * PLD + r0);
-                const float4 x0 = ld4(S.w1t + k * PW + c0), x1 = ld4(S.w1t + k * PW + c0 + 4);
-                const float av[4] = {a.x, a.y, a.z, a.w};
-                const float bv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float4 h = ld4(S.h0 + (c0 + j) * PLD + r0);
-                st4(S.h2 + (c0 + j) * PLD + r0,
-                    make_float4(h.x > 0.0f ? acc[0][j] : 0.0f, h.y > 0.0f ? acc[1][j] : 0.0f,
-                                h.z > 0.0f ? acc[2][j] : 0.0f, h.w > 0.0f ? acc[3][j] : 0.0f));
-            }
-        }
+        weight_grad(S.h0, S.h1, g1, gb1);              // dW1 += H0^T dZ1, db1 += sum dZ1
+        ptile_gemm<PW>(S.h1, S.w1t, nullptr, acc);
+        store_masked(acc, S.h0, S.h2);                 // dZ0 over h2 (free now)
         __syncthreads();
         // [dW0 | db0] += X^T dZ0 : thread: output n = t & 63, inputs 10 (t >> 6) .. +9
         {
@@ -446,14 +387,18 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
     float *G0 = P.grad, *GB0 = G0 + PIN * PW, *G1 = GB0 + PW, *GB1 = G1 + PW * PW, *G2 = GB1 + PW, *GB2 = G2 + PW * PW;
     float *G3 = GB2 + PW, *GB3 = G3 + PW;
     {
-        const int kq = tid >> 3, nq = tid & 7;
+        const int kq = tid >> 3, nq = tid & 7, warp = tid >> 5;
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                atomicAdd(G1 + (2 * kq + i) * PW + 8 * nq + j, g1[i][j]);
-                atomicAdd(G2 + (2 * kq + i) * PW + 8 * nq + j, g2[i][j]);
+                atomicAdd(G1 + (kq + 32 * i) * PW + nq + 8 * j, g1[i][j]);
+                atomicAdd(G2 + (kq + 32 * i) * PW + nq + 8 * j, g2[i][j]);
             }
+        if ((kq & 3) == 0) {
+            atomicAdd(GB1 + nq + 8 * warp, gb1);
+            atomicAdd(GB2 + nq + 8 * warp, gb2);
+        }
         const int n = tid & 63, k0 = 10 * (tid >> 6);
 #pragma unroll
         for (int i = 0; i < 10; ++i) {
@@ -462,12 +407,12 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
             else if (k == PIN) atomicAdd(GB0 + n, g0[i]);
         }
     }
-    if (tid < PW) {
-        atomicAdd(G3 + tid, g3);
-        atomicAdd(GB1 + tid, gb1);
-        atomicAdd(GB2 + tid, gb2);
-    }
-    if (tid == PW) atomicAdd(GB3, gb3);
+    g3 += __shfl_xor_sync(0xffffffffu, g3, 1);
+    g3 += __shfl_xor_sync(0xffffffffu, g3, 2);
+    gb3 += __shfl_xor_sync(0xffffffffu, gb3, 1);
+    gb3 += __shfl_xor_sync(0xffffffffu, gb3, 2);
+    if ((tid & 3) == 0) atomicAdd(G3 + (tid >> 2), g3);
+    if (tid == 0) atomicAdd(GB3, gb3);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -23,8 +23,8 @@
 
 #include <math.h>
 
-#include "df64.cuh"
 #include "dvgo_internal.cuh"
+#include "proposal_rays.cuh"
 #include "tc_helpers.cuh"
 
 namespace dvgo {
@@ -33,19 +33,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int NB = 64, NFQ = 6, PIN = 3 + 6 * NFQ, PW = 64, TT = 128;
+constexpr int NB = kPropBins, NFQ = 6, PIN = 3 + 6 * NFQ, PW = 64, TT = 128;
 // Forward TMEM: the three layers use one accumulator (64 columns at COL_Z) in turn; their A operand
 // (X, then H0, then H1, BF16 packed two per column: 32 columns at COL_A) is written there too.
 constexpr uint32_t COL_Z = 0, COL_A = 64, FWD_COLS = 128;
 constexpr int kFwdCtasPerSm = 4;   // 4 x 128 TMEM columns
-
-// Box clip of one ray as the encoding uses it: entry t0, bin width w = (t_exit - t_enter) / 64 and
-// direction as double-float values of the FP64 clip, the origin, and whether the ray hits the box.
-struct ClipDf {
-    Df t0, w, dn[3];
-    float o[3];
-    int hit;
-};
 
 constexpr int kClipTiles = TT / 2;   // tiles per clip pass: one ray per thread
 
@@ -118,32 +110,8 @@ __device__ __forceinline__ void load_weights(const PropTcArgs &P, unsigned char 
     if (tid == 0) b3[0] = P.b3[0];
 }
 
-// Box clips (FP64, as in the renderer) of the rays of the CTA's tiles k0 .. k0 + 63 (its k-th tile
-// is blockIdx.x + k gridDim.x, rays 2 tile and 2 tile + 1), one ray per thread.  Clipping per ray
-// instead of per tile keeps the FP64 work (1/64 of the FP32 rate on this GPU) off the tile loop.
 __device__ __forceinline__ void clip_pass(const PropTcArgs &P, int k0, ClipDf *cl) {
-    const int tid = threadIdx.x;
-    const long long tile = blockIdx.x + (long long)(k0 + (tid >> 1)) * gridDim.x, r = 2 * tile + (tid & 1);
-    ClipDf c;
-    c.t0 = c.w = c.dn[0] = c.dn[1] = c.dn[2] = Df{0.0f, 0.0f};
-    c.o[0] = c.o[1] = c.o[2] = 0.0f;
-    c.hit = 0;
-    if (r < P.R) {
-        const double o[3] = {(double)P.ro[3 * r], (double)P.ro[3 * r + 1], (double)P.ro[3 * r + 2]};
-        const double d[3] = {(double)P.rd[3 * r], (double)P.rd[3 * r + 1], (double)P.rd[3 * r + 2]};
-        const Clip q = slab_clip(o, d, P.mn, P.mx, P.t_near, P.t_far);
-        c.hit = q.hi > q.lo;
-        if (c.hit) {
-            c.t0 = df_from_double(q.lo);
-            c.w = df_from_double(__ddiv_rn(__dsub_rn(q.hi, q.lo), (double)NB));
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                c.dn[a] = df_from_double(q.dn[a]);
-                c.o[a] = P.ro[3 * r + a];
-            }
-        }
-    }
-    cl[tid] = c;
+    clip_tile_rays(P.R, P.ro, P.rd, P.mn, P.mx, P.t_near, P.t_far, k0, cl);
 }
 
 // Input row of this thread's bin centre (zeros for a ray that misses or does not exist).  The bin
@@ -154,10 +122,10 @@ __device__ __forceinline__ void encode_values(const ClipDf &c, float (&v)[64]) {
 #pragma unroll
     for (int k = 0; k < 64; ++k) v[k] = 0.0f;
     if (c.hit) {
-        const Df tb = df_add(c.t0, df_mul_f(c.w, (float)bin + 0.5f));
+        const Df tb = bin_centre(c, bin);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float xa = df_add(Df{c.o[a], 0.0f}, df_mul(tb, c.dn[a])).hi;
+            const float xa = bin_position(c, tb, a).hi;
             v[a] = xa;
             float sn, cs;
             sincosf(xa, &sn, &cs);
