@@ -11,7 +11,6 @@
 namespace dvgo {
 
 void launch_fine_colour_fwd_fp32(const RenderArgs &A, cudaStream_t s);
-void launch_fine_colour_bwd_simt(const RenderArgs &A, cudaStream_t s);
 int launch_fine_colour_fwd_tc(const RenderArgs &A, cudaStream_t s);
 int launch_fine_colour_bwd_tc(const RenderArgs &A, cudaStream_t s);
 
@@ -384,7 +383,7 @@ int dvgo_render_bwd(const dvgo_params *p, const dvgo_grid_desc *dd, const float 
         if (p->mlp_prec == DVGO_MLP_BF16) {
             if ((st = launch_fine_colour_bwd_tc(A, s))) return st;
         } else {
-            launch_fine_colour_bwd_simt(A, s);
+            launch_fine_colour_bwd_fp32(A, s);
         }
     }
     return launch_status();

@@ -1,5 +1,6 @@
 // fine_gather.cuh -- what the producers of the tensor-core colour kernels share: placing a kept sample
-// from its ray's record, and the trilinear gather of its 12 features (Sec. 4.2 Eq. fine_queries_rgb).
+// from its ray's record, the trilinear gather of its 12 features (Sec. 4.2 Eq. fine_queries_rgb), and the
+// scatter of a tile's feature gradients.
 #pragma once
 
 #include "dvgo_internal.cuh"
@@ -103,6 +104,56 @@ __device__ __forceinline__ void gather_features(const RenderArgs &A, const Cell 
                 v[4 * k + 3] += w0 * a1.y + w1 * b1.y;
             }
         }
+    }
+}
+
+// Producer: add a tile's feature gradients (de(row, k): channels 4 k .. 4 k + 3 of a row) to the grid.  Rows
+// are in kept order, so consecutive samples of a ray sit in consecutive rows; rows whose samples lie
+// in one lattice cell share all eight corners, and the last row of such a run adds the whole run's
+// weighted de with one set of reductions (the run's other rows add nothing).
+// slot (-1: padding row), cbase and frac: the tile's per-row tables.
+template <bool PK, typename De>
+__device__ __forceinline__ void scatter_row(const RenderArgs &A, const int *slot, const int *cbase,
+                                            const float (*frac)[3], De de, int row) {
+    constexpr int TM = 128, FEAT = 12;
+    if (slot[row] < 0) return;
+    const int cb = cbase[row];
+    if (row + 1 < TM && slot[row + 1] >= 0 && cbase[row + 1] == cb) return;
+    float4 acc[8][3];
+    {
+        const float4 e0 = de(row, 0), e1 = de(row, 1), e2 = de(row, 2);
+        const float fx = frac[row][0], fy = frac[row][1], fz = frac[row][2];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
+                            ((q & 1) ? fz : 1.0f - fz);
+            acc[q][0] = make_float4(w * e0.x, w * e0.y, w * e0.z, w * e0.w);
+            acc[q][1] = make_float4(w * e1.x, w * e1.y, w * e1.z, w * e1.w);
+            acc[q][2] = make_float4(w * e2.x, w * e2.y, w * e2.z, w * e2.w);
+        }
+    }
+    for (int j = row - 1; j >= 0 && slot[j] >= 0 && cbase[j] == cb; --j) {
+        const float4 e0 = de(j, 0), e1 = de(j, 1), e2 = de(j, 2);
+        const float fx = frac[j][0], fy = frac[j][1], fz = frac[j][2];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
+                            ((q & 1) ? fz : 1.0f - fz);
+            acc[q][0] = make_float4(fmaf(w, e0.x, acc[q][0].x), fmaf(w, e0.y, acc[q][0].y),
+                                    fmaf(w, e0.z, acc[q][0].z), fmaf(w, e0.w, acc[q][0].w));
+            acc[q][1] = make_float4(fmaf(w, e1.x, acc[q][1].x), fmaf(w, e1.y, acc[q][1].y),
+                                    fmaf(w, e1.z, acc[q][1].z), fmaf(w, e1.w, acc[q][1].w));
+            acc[q][2] = make_float4(fmaf(w, e2.x, acc[q][2].x), fmaf(w, e2.y, acc[q][2].y),
+                                    fmaf(w, e2.z, acc[q][2].z), fmaf(w, e2.w, acc[q][2].w));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const long long idx = corner_from_base(cb, (q >> 2) & 1, (q >> 1) & 1, q & 1, A.ny, A.nz, PK);
+        float4 *g = reinterpret_cast<float4 *>(A.grad_cgrid + idx * FEAT);
+        atomicAdd(g + 0, acc[q][0]);
+        atomicAdd(g + 1, acc[q][1]);
+        atomicAdd(g + 2, acc[q][2]);
     }
 }
 

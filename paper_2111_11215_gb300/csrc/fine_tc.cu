@@ -123,10 +123,6 @@ static_assert(offsetof(SmemTC, dout) == offsetof(SmemTC, h1) + 2 * kPanelBytes, 
 constexpr size_t smem_bytes(bool bwd) { return (bwd ? sizeof(SmemTC) : offsetof(SmemTC, dz2)) + 1024; }
 static_assert(smem_bytes(true) <= 232448, "the backward must fit one CTA per SM (227 KB of shared memory)");
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
-}
-
 // Barrier among the 256 consumer threads only (the producers run on their own schedule).
 __device__ __forceinline__ void consumer_sync() {
     fence_before();
@@ -143,55 +139,6 @@ __device__ __forceinline__ void consumer_publish() {
 // 16-byte chunk k (0-2) of the de[0:12] slot of X buffer b in row r of the dout panel.
 __device__ __forceinline__ float4 *de_slot(unsigned char *dout, int b, int r, int k) {
     return reinterpret_cast<float4 *>(dout + panel_offset(r, 8 * (2 + 3 * b + k)));
-}
-
-// Producer: add a tile's feature gradients (de rows staged in the dout panel) to the grid.  Rows
-// are in kept order, so consecutive samples of a ray sit in consecutive rows; rows whose samples lie
-// in one lattice cell share all eight corners, and the last row of such a run adds the whole run's
-// weighted de with one set of reductions (the run's other rows add nothing).
-template <bool PK>
-__device__ __forceinline__ void scatter_row(const RenderArgs &A, SmemTC &S, int b, int t, int row) {
-    const int slot = S.sm.slot[t][row];
-    if (slot < 0) return;
-    const int cb = S.sm.cbase[t][row];
-    if (row + 1 < TM && S.sm.slot[t][row + 1] >= 0 && S.sm.cbase[t][row + 1] == cb) return;
-    float4 acc[8][3];
-    {
-        const float4 e0 = *de_slot(S.dout, b, row, 0), e1 = *de_slot(S.dout, b, row, 1),
-                     e2 = *de_slot(S.dout, b, row, 2);
-        const float fx = S.sm.frac[t][row][0], fy = S.sm.frac[t][row][1], fz = S.sm.frac[t][row][2];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
-                            ((q & 1) ? fz : 1.0f - fz);
-            acc[q][0] = make_float4(w * e0.x, w * e0.y, w * e0.z, w * e0.w);
-            acc[q][1] = make_float4(w * e1.x, w * e1.y, w * e1.z, w * e1.w);
-            acc[q][2] = make_float4(w * e2.x, w * e2.y, w * e2.z, w * e2.w);
-        }
-    }
-    for (int j = row - 1; j >= 0 && S.sm.slot[t][j] >= 0 && S.sm.cbase[t][j] == cb; --j) {
-        const float4 e0 = *de_slot(S.dout, b, j, 0), e1 = *de_slot(S.dout, b, j, 1), e2 = *de_slot(S.dout, b, j, 2);
-        const float fx = S.sm.frac[t][j][0], fy = S.sm.frac[t][j][1], fz = S.sm.frac[t][j][2];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
-                            ((q & 1) ? fz : 1.0f - fz);
-            acc[q][0] = make_float4(fmaf(w, e0.x, acc[q][0].x), fmaf(w, e0.y, acc[q][0].y),
-                                    fmaf(w, e0.z, acc[q][0].z), fmaf(w, e0.w, acc[q][0].w));
-            acc[q][1] = make_float4(fmaf(w, e1.x, acc[q][1].x), fmaf(w, e1.y, acc[q][1].y),
-                                    fmaf(w, e1.z, acc[q][1].z), fmaf(w, e1.w, acc[q][1].w));
-            acc[q][2] = make_float4(fmaf(w, e2.x, acc[q][2].x), fmaf(w, e2.y, acc[q][2].y),
-                                    fmaf(w, e2.z, acc[q][2].z), fmaf(w, e2.w, acc[q][2].w));
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const long long idx = corner_from_base(cb, (q >> 2) & 1, (q >> 1) & 1, q & 1, A.ny, A.nz, PK);
-        float4 *g = reinterpret_cast<float4 *>(A.grad_cgrid + idx * FEAT);
-        atomicAdd(g + 0, acc[q][0]);
-        atomicAdd(g + 1, acc[q][1]);
-        atomicAdd(g + 2, acc[q][2]);
-    }
 }
 
 // Producer: gather sample row `row` of a tile (kept entry kv, kv.y < 0 for a padding row; its ray's
@@ -352,6 +299,10 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             const int e = t * TM + row;
             return (t < ntiles && e < n_kept) ? A.kept[e] : make_int2(-1, -1);
         };
+        auto scatter_tile = [&](int b, int t) {   // X buffer b, entry t of the table ring
+            scatter_row<PK>(A, S.sm.slot[t], S.sm.cbase[t], S.sm.frac[t],
+                            [&](int r, int k) { return *de_slot(S.dout, b, r, k); }, row);
+        };
         const int tile0 = (int)blockIdx.x + pset * (int)gridDim.x;
         int2 kv_cur = kept_at(tile0);
         RayPre rp_cur = kv_cur.y >= 0 ? ray_pre(A, kv_cur.y) : RayPre{};
@@ -371,7 +322,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
                 bulk_load(S.x[b], A.xcache + (size_t)tile * kPanelBytes, kPanelBytes, &S.sm.xl[b]);
                 ++nload[b];
             }
-            if (BWD && i >= 2) scatter_row<PK>(A, S, b, (i - 2) & 3, row);   // feature gradients of tile i - 2
+            if (BWD && i >= 2) scatter_tile(b, (i - 2) & 3);   // feature gradients of tile i - 2
             produce_row<FeatT, BWD, PEX, PK>(A, S, b, i & 3, kv_cur, rp_cur, row, cached);
             fence_async_smem();
             // (testing aid: one arrival withheld on a chosen tile makes the consumers' wait run out)
@@ -384,7 +335,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             // the last (up to) two tiles: wait until the consumers are done with them, then scatter
             for (int j = (i >= 2 ? i - 2 : 0); j < i && ok; ++j) {
                 if (!mbar_wait(&S.sm.empty[j & 1], (j >> 1) & 1, A.wait_ns)) ok = false;
-                else if (!*(volatile int *)&S.sm.abort) scatter_row<PK>(A, S, j & 1, j & 3, row);
+                else if (!*(volatile int *)&S.sm.abort) scatter_tile(j & 1, j & 3);
             }
         }
         // every bulk load issued has landed before the CTA can exit (bounded)

@@ -60,32 +60,11 @@ constexpr size_t split_smem() {
 }
 static_assert(split_smem<true>() <= 232448, "one CTA per SM (227 KB of shared memory)");
 
-// Eight FP32 values as three BF16 chunks of 16 bytes: hi, mid, lo.
-__device__ __forceinline__ void split8(const float *v, uint4 (&q)[3]) {
-    uint32_t w[3][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float a = v[2 * i], b = v[2 * i + 1];
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            w[s][i] = pack_bf16(a, b);
-            a = __fsub_rn(a, __uint_as_float(w[s][i] << 16));
-            b = __fsub_rn(b, __uint_as_float(w[s][i] & 0xffff0000u));
-        }
-    }
-#pragma unroll
-    for (int s = 0; s < 3; ++s) q[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-}
-
 // Split s, columns [8 c, 8 c + 8) of row `row` of an operand of KB blocks a split.
 template <int KB>
 __device__ __forceinline__ uint4 *split_chunk(unsigned char *base, int s, int row, int c) {
     const int q = s * KB + (c >> 1);
     return reinterpret_cast<uint4 *>(base + (q >> 2) * kPanelBytes + panel_offset(row, (q & 3) * 16 + (c & 1) * 8));
-}
-
-__device__ __forceinline__ void arrive(uint64_t *mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 // Barrier among the 256 consumer threads.
@@ -175,7 +154,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                 for (int s = 0; s < 3; ++s) *split_chunk<KB>(xs, s, row, c) = q[s];
             }
             fence_async_smem();
-            arrive(&S.full);
+            mbar_arrive(&S.full);
         }
         if (!ok) atomicExch(&S.abort, 1);
     } else {
@@ -250,7 +229,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                 tau = __ldg(A.stau + slot);
             }
             if (!wait_mma()) { ok = false; break; }
-            if (tid == 0) arrive(&S.empty);   // X is free
+            if (tid == 0) mbar_arrive(&S.empty);   // X is free
             // ---- epilogue 1: H1 = relu(Z1), split, over Z1 (read whole before any is overwritten) ----
             {
                 float z[2][32];

@@ -1,0 +1,718 @@
+// fine_tc_fp32_bwd.cu -- backward of the fine stage's colour queries with the FP32 MLP of 39 inputs, on the
+// tensor cores (the 72-input form is fine_simt.cu: its operands do not fit beside the weights).
+//
+// Arithmetic as in fine_tc_fp32.cu: every FP32 operand is the exact sum of three BF16 numbers, every
+// contraction the six products that matter with FP32 accumulation, the smallest first.  Weight
+// gradients leave their TMEM accumulator after every tile and are summed over the tiles in registers, with
+// rounding (an accumulator that lived through all tiles would lose a part in 10^4 to the tensor core's
+// truncation).  A ReLU unit within rounding of zero is decided by the plain FP32 FMA chain over its inputs
+// (exact_z1 / exact_z2, the order of the SIMT kernel), so the gradients do not hang on which
+// arithmetic recomputed the hidden layers.
+//
+// Bound: 1806 us-equivalents of FMA work left the SIMT kernel at 45 % of the CUDA cores' rate; BWD_NUMBERS
+//
+// Per tile of M = 128 kept samples, with dout = dL/do from the compositing backward; activations are kept
+// transposed (TMEM lane = hidden unit, column = sample), so that a thread owns a unit: the sums over the
+// samples of db2 and dW3 stay in its registers, and the activations are directly the A operand, from
+// tensor memory, of the weight gradients:
+//   Z1^T = W1^T X^T                 A = W1 (shared), B = X (shared)
+//   Z2^T = W2^T H1^T                A = W2 (shared), B = H1^T (shared, a third at a time)
+//   dZ2 = (dout W3^T) [Z2 > 0], dW3 += H2^T dout, db2 += sum dZ2      (CUDA cores)
+//   dW2 += H1^T dZ2                 A = H1^T (TMEM), B = dZ2^T (shared, a third at a time)
+//   dH1^T = W2 dZ2^T                A = W2 (shared, read MN-major), B = dZ2^T
+//   dZ1 = dH1 [Z1 > 0]
+//   de = dZ1 W1[0:12]^T             A = dZ1^T (shared, read MN-major), B = W1 (read MN-major)
+//   [dW1 | db1]^T += dZ1^T X        A = dZ1^T (TMEM), B = X (staged again)
+// Shared memory: W2 split 96 KB, W1 split 48 KB, and a pool of 64 KB that holds X (48 KB), then pairs of
+// 32 KB thirds of the activations, then X again.  Warps 0-7 consume (thread (n, half): unit n = t mod 128,
+// samples 64 half .. +63), warps 8-11 gather X, stage it twice and scatter the feature gradients of the
+// tile before.  TMEM columns: activations' split [0, 192), layer accumulator [192, 320), dW2 [320, 448),
+// dW1 [448, 496), de [496, 512).
+
+#include "dvgo_internal.cuh"
+#include "fine_gather.cuh"
+#include "tc_helpers.cuh"
+
+namespace dvgo {
+
+namespace {
+
+using namespace tc;
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int TM = 128, NC = 256, NP = 128;
+constexpr int HID = 128, FEAT = 12, IN = 39, XK = 40;   // column IN of X is the constant 1 (bias)
+constexpr int KB = 3;                                   // 16-column blocks of X and W1 per split
+constexpr uint32_t T_ACT = 0, T_Z = 192, T_DW2 = 320, T_DW1 = 448, T_DE = 496, NCOLS = 512;
+
+struct BwdSmall {
+    alignas(16) float dout[3][TM];   // dL/do
+    alignas(16) float xmax[TM];      // largest input magnitude of the row (0: padding row)
+    float4 de[TM][3];      // feature gradients of a tile
+    int slot[2][TM], cbase[2][TM];
+    float frac[2][TM][3];
+    uint64_t full, empty, mma_a, mma_b;
+    uint32_t tmem_base;
+    int abort;
+    int s1max;             // largest absolute row sum of W1^T | b1 (float bits)
+};
+
+constexpr int kPoolPanels = 4;
+constexpr size_t kBwdSmem = (size_t)(6 + 3 + kPoolPanels) * kPanelBytes + sizeof(BwdSmall) + 1023;
+static_assert(kBwdSmem <= 232448, "one CTA per SM (227 KB of shared memory)");
+
+__device__ __forceinline__ void consumer_sync() {
+    fence_before();
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    fence_after();
+}
+// Operands written by the consumers become visible to the tensor core, then the consumers sync.
+__device__ __forceinline__ void publish() {
+    fence_async_smem();
+    consumer_sync();
+}
+
+// The input row of kept sample e, bit for bit as the SIMT kernel forms it: lane l holds inputs l and 32 + l
+// (input 39: the constant 1).  All lanes of the warp take part.
+template <typename FeatT, bool PK>
+__device__ __noinline__ float2 exact_inputs(const RenderArgs &A, int e) {
+    const int lane = threadIdx.x & 31, q = lane & 3;
+    const int2 kv = A.kept[e];
+    float dt;
+    const Cell c = sample_cell(A, A.rays[kv.y], kv.y, kv.x >> 16, dt);
+    const FeatT *g0 = static_cast<const FeatT *>(A.cgrid) + corner_index(c, 2 * q, A.ny, A.nz, PK) * FEAT;
+    const FeatT *g1 = static_cast<const FeatT *>(A.cgrid) + corner_index(c, 2 * q + 1, A.ny, A.nz, PK) * FEAT;
+    const float w0 = corner_weight(c, 2 * q), w1 = corner_weight(c, 2 * q + 1);
+    float x0 = 0.0f;
+#pragma unroll
+    for (int ch = 0; ch < FEAT; ++ch) {
+        float f = fmaf(w0, (float)g0[ch], w1 * (float)g1[ch]);
+        f += __shfl_xor_sync(FULL, f, 1);
+        f += __shfl_xor_sync(FULL, f, 2);
+        if (lane == ch) x0 = f;
+    }
+    const float *pe = A.pe + (size_t)kv.y * kPeStride;
+    if (lane >= FEAT) x0 = pe[lane - FEAT];
+    return make_float2(x0, lane < 7 ? pe[20 + lane] : (lane == 7 ? 1.0f : 0.0f));
+}
+
+// z of a unit of layer 1 / layer 2 at kept sample e: FMA chains in input order (the bias last / first).
+template <typename FeatT, bool PK>
+__device__ __noinline__ float exact_z1(const RenderArgs &A, int e, int unit) {
+    const int lane = threadIdx.x & 31;
+    const float2 x = exact_inputs<FeatT, PK>(A, e);
+    const float w0 = A.w1[lane * HID + unit],
+                w1 = lane < 7 ? A.w1[(32 + lane) * HID + unit] : (lane == 7 ? A.b1[unit] : 0.0f);
+    float z = 0.0f;
+#pragma unroll 8
+    for (int k = 0; k < 32; ++k) z = fmaf(__shfl_sync(FULL, x.x, k), __shfl_sync(FULL, w0, k), z);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) z = fmaf(__shfl_sync(FULL, x.y, k), __shfl_sync(FULL, w1, k), z);
+    return z;
+}
+
+template <typename FeatT, bool PK>
+__device__ __noinline__ float exact_z2(const RenderArgs &A, int e, int unit) {
+    const int lane = threadIdx.x & 31;
+    const float2 x = exact_inputs<FeatT, PK>(A, e);
+    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, w[4];
+    for (int k0 = 0; k0 < XK; k0 += 8) {   // eight inputs' weights in flight
+        float r[8][4];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float *row = k0 + j < IN ? A.w1 + (k0 + j) * HID : A.b1;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) r[j][i] = row[lane + 32 * i];
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float xk = k0 < 32 ? __shfl_sync(FULL, x.x, k0 + j) : __shfl_sync(FULL, x.y, j);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) h[i] = fmaf(xk, r[j][i], h[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        h[i] = fmaxf(h[i], 0.0f);
+        w[i] = A.w2[(lane + 32 * i) * HID + unit];
+    }
+    float z = A.b2[unit];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll 8
+        for (int l = 0; l < 32; ++l) z = fmaf(__shfl_sync(FULL, h[i], l), __shfl_sync(FULL, w[i], l), z);
+    return z;
+}
+
+// The signs of the units within rounding of zero, decided by the FMA chains: amb marks this lane's among
+// samples e0 .. e0 + 15 (bit k), neg holds the sign bits (sample k in bit 15 - k) and is returned corrected.  A
+// unit counts as off unless z > 0.  All lanes of the warp take part.
+template <typename FeatT, bool PK, int kLayer>
+__device__ __noinline__ uint32_t resolve(const RenderArgs &A, int e0, int unit, uint32_t amb, uint32_t neg) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned any = __ballot_sync(FULL, amb != 0u); any; any = __ballot_sync(FULL, amb != 0u)) {
+        const int src = __ffs(any) - 1, k = __ffs(__shfl_sync(FULL, amb, src)) - 1, u = __shfl_sync(FULL, unit, src);
+        const float z = kLayer == 1 ? exact_z1<FeatT, PK>(A, e0 + k, u) : exact_z2<FeatT, PK>(A, e0 + k, u);
+        if (lane == src) {
+            amb &= amb - 1u;
+            const uint32_t bit = 0x8000u >> k;
+            neg = z > 0.0f ? neg & ~bit : neg | bit;
+        }
+    }
+    return neg;
+}
+__device__ __forceinline__ bool off(uint32_t neg, int k) { return (neg >> (15 - k)) & 1u; }
+
+// Splits 16 consecutive samples of this thread's unit (row n, samples 64 hc + 16 g ..): the three terms as
+// packed pairs (for TMEM) in w, and the chosen ones into the half panels lo / mid (row = unit).
+__device__ __forceinline__ void split16(const float *v, uint32_t (&w)[3][8]) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        uint4 q[3];
+        split8(v + 8 * c, q);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            w[s][4 * c] = q[s].x;
+            w[s][4 * c + 1] = q[s].y;
+            w[s][4 * c + 2] = q[s].z;
+            w[s][4 * c + 3] = q[s].w;
+        }
+    }
+}
+__device__ __forceinline__ void store16(unsigned char *half_panel, int n, int g, const uint32_t (&w)[8]) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+        *reinterpret_cast<uint4 *>(half_panel + panel_offset(n, 16 * g + 8 * c)) =
+            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+}
+
+// dL/do of four consecutive samples.
+__device__ __forceinline__ void load_dout(const BwdSmall &S, int s, float (&d)[3][4]) {
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) *reinterpret_cast<float4 *>(d[ch]) = *reinterpret_cast<const float4 *>(&S.dout[ch][s]);
+}
+
+template <typename FeatT, bool PK>
+__global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(RenderArgs A) {
+    const int n_kept = A.hdr->n_kept;
+    const int ntiles = (n_kept + TM - 1) / TM;
+    if ((int)blockIdx.x >= ntiles) return;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *w2t = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *w1t = w2t + 6 * kPanelBytes, *pool = w1t + 3 * kPanelBytes;
+    BwdSmall &S = *reinterpret_cast<BwdSmall *>(pool + kPoolPanels * kPanelBytes);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        mbar_init(&S.full, NP);
+        mbar_init(&S.empty, 1);
+        mbar_init(&S.mma_a, 1);
+        mbar_init(&S.mma_b, 1);
+        S.abort = 0;
+        S.s1max = 0;
+    }
+    if (warp == 0) tmem_alloc(&S.tmem_base, NCOLS);
+    fence_before();
+    __syncthreads();
+    fence_after();
+    bool ok = true;
+    uint32_t pa = 0, pb = 0;   // phases of mma_a and mma_b
+    bool b_out = false;        // a batch on mma_b not waited for yet
+
+    if (tid >= NC) {
+        // ------------------------------- producers -------------------------------
+        // 384 x 168 registers at launch = 256 x 192 + 128 x 120
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 120;");
+        const int row = tid - NC;
+        struct Row {
+            float v[XK];
+            float4 dout;
+            int slot, cbase;
+            float fx, fy, fz;
+        };
+        auto gather = [&](int t, Row &w) {
+            const int e = t * TM + row;
+#pragma unroll
+            for (int k = 0; k < XK; ++k) w.v[k] = 0.0f;
+            w.dout = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            w.slot = -1;
+            w.cbase = 0;
+            w.fx = w.fy = w.fz = 0.0f;
+            if (t >= ntiles || e >= n_kept) return;
+            const int2 kv = A.kept[e];
+            const RayPre rp = ray_pre(A, kv.y);
+            float dt;
+            const Cell c = cell_pre(A, rp, kv.y, kv.x >> 16, dt);
+            w.slot = rp.off + (kv.x & 0xffff);
+            w.cbase = cell_base(c, A.ny, A.nz, PK);
+            w.fx = c.fx;
+            w.fy = c.fy;
+            w.fz = c.fz;
+            const float4 g = A.sgrad[w.slot];
+            gather_features<FeatT, PK>(A, c, w.v);
+            const float4 *pe = reinterpret_cast<const float4 *>(A.pe + (size_t)kv.y * kPeStride);
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                const float4 q4 = __ldg(pe + k);
+                const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (4 * k + j < 27) w.v[FEAT + 4 * k + j] = q[j];
+            }
+            w.v[IN] = 1.0f;
+            float m = 1.0f;
+#pragma unroll
+            for (int k = 0; k < FEAT; ++k) m = fmaxf(m, fabsf(w.v[k]));
+            w.dout = make_float4(g.y, g.z, g.w, m);
+        };
+        auto stage = [&](const Row &w) {   // X: one panel per split, columns 0-47
+#pragma unroll
+            for (int c = 0; c < 2 * KB; ++c) {
+                uint4 q[3] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+                if (8 * c < XK) split8(w.v + 8 * c, q);
+#pragma unroll
+                for (int s = 0; s < 3; ++s)
+                    *reinterpret_cast<uint4 *>(pool + s * kPanelBytes + panel_offset(row, 8 * c)) = q[s];
+            }
+        };
+        auto scatter_tile = [&](int t) {
+            scatter_row<PK>(A, S.slot[t], S.cbase[t], S.frac[t], [&](int r, int k) { return S.de[r][k]; }, row);
+        };
+        Row cur;
+        gather(blockIdx.x, cur);
+        int i = 0;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
+            // the pool is free once the tile before is done (second release of a tile)
+            if (i > 0 && !mbar_wait(&S.empty, 1, A.wait_ns)) { ok = false; break; }
+            stage(cur);
+            const int t = i & 1;
+            S.slot[t][row] = cur.slot;
+            S.cbase[t][row] = cur.cbase;
+            S.frac[t][row][0] = cur.fx;
+            S.frac[t][row][1] = cur.fy;
+            S.frac[t][row][2] = cur.fz;
+            S.dout[0][row] = cur.dout.x;
+            S.dout[1][row] = cur.dout.y;
+            S.dout[2][row] = cur.dout.z;
+            S.xmax[row] = cur.dout.w;
+            fence_async_smem();
+            mbar_arrive(&S.full);
+            if (i > 0) {
+                // every producer's tables and de of the tile before are in place: they were written before
+                // the consumers' release that this thread has just waited for
+                scatter_tile(t ^ 1);
+            }
+            if (!mbar_wait(&S.empty, 0, A.wait_ns)) { ok = false; break; }
+            stage(cur);   // again, for dW1
+            fence_async_smem();
+            mbar_arrive(&S.full);
+            gather(tile + gridDim.x, cur);
+        }
+        if (ok && i > 0) {
+            if (!mbar_wait(&S.empty, 1, A.wait_ns)) ok = false;
+            else scatter_tile((i - 1) & 1);
+        }
+        if (!ok) atomicExch(&S.abort, 1);
+    } else {
+        // ------------------------------- consumers -------------------------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 192;");
+        const int n = tid & (HID - 1), hc = tid >> 7;
+        // W1^T | b1 and W2^T split: (unit, 8 input columns) per thread and turn
+        for (int t = tid; t < HID * (2 * KB + 16); t += NC) {
+            const int u = t & (HID - 1), c = t >> 7;
+            float v[8];
+            uint4 q[3];
+            if (c < 2 * KB) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int k = 8 * c + j;
+                    v[j] = k < IN ? A.w1[k * HID + u] : (k == IN ? A.b1[u] : 0.0f);
+                }
+                split8(v, q);
+#pragma unroll
+                for (int s = 0; s < 3; ++s)
+                    *reinterpret_cast<uint4 *>(w1t + s * kPanelBytes + panel_offset(u, 8 * c)) = q[s];
+            } else {
+                const int c2 = c - 2 * KB;   // 0-15
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = A.w2[(8 * c2 + j) * HID + u];
+                split8(v, q);
+#pragma unroll
+                for (int s = 0; s < 3; ++s)
+                    *reinterpret_cast<uint4 *>(w2t + (2 * s + (c2 >> 3)) * kPanelBytes + panel_offset(u, (c2 & 7) * 8)) = q[s];
+            }
+        }
+        const float w30 = A.w3[3 * n], w31 = A.w3[3 * n + 1], w32 = A.w3[3 * n + 2], b2 = A.b2[n];
+        // Where a unit's sign is looked at again: 2^-23 of a bound on the sum of magnitudes behind z (more than
+        // ten times the usual difference of the two arithmetics), for inputs of magnitude 1.
+        float s1 = fabsf(A.b1[n]), s2 = 0.0f;
+        for (int k = 0; k < IN; ++k) s1 += fabsf(A.w1[k * HID + n]);
+        for (int k = 0; k < HID; ++k) s2 += fabsf(A.w2[k * HID + n]);
+        atomicMax(&S.s1max, __float_as_int(s1));
+        publish();
+        const float eps1 = 0x1p-23f * s1, eps2 = 0x1p-23f * (0.25f * __int_as_float(S.s1max) * s2 + fabsf(b2));
+
+        const uint32_t tb = S.tmem_base;
+        const uint32_t w1_ = smem_u32(w1t), w2_ = smem_u32(w2t), pool_ = smem_u32(pool);
+        unsigned char *buf0 = pool + hc * kPanelBytes, *buf1 = pool + (2 + hc) * kPanelBytes;   // this thread's halves
+        const uint32_t b0_ = pool_, b1_ = pool_ + 2 * kPanelBytes;
+        const uint32_t id_z1 = idesc_bf16(128, 128, 0, 0), id_z2 = idesc_bf16(128, 128, 0, 1),
+                       id_dh = idesc_bf16(128, 128, 1, 1), id_de = idesc_bf16(128, 16, 1, 1),
+                       id_dw1 = idesc_bf16(128, 48, 0, 1);
+        constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};   // the six products, small first
+        auto wait_a = [&]() -> bool {
+            const bool w = mbar_wait(&S.mma_a, pa, A.wait_ns);
+            pa ^= 1;
+            fence_after();
+            return w;
+        };
+        auto wait_b = [&]() -> bool {
+            const bool w = mbar_wait(&S.mma_b, pb, A.wait_ns);
+            pb ^= 1;
+            b_out = false;
+            fence_after();
+            return w;
+        };
+        // MMA batches over a third of an activation held in the pool at b_ (thread 0).  Descriptors are a base
+        // and steps of the address field (16-byte units), so that an MMA costs the issuing thread two adds.
+        auto z2_batch = [&](uint32_t b_, int sa, bool first) {   // Z2^T (+)= W2[sa] H1^T
+            const uint64_t a = desc_kmajor(w2_ + 2u * sa * kPanelBytes, 0), b = desc_mnmajor(b_, 0);
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+                mma(tb + T_Z, a + kstep(kk), b + mnstep(kk), id_z2, !first || kk > 0);
+        };
+        auto dz2_batch = [&](uint32_t b_, int sa, bool first) {  // dW2 (+)= H1^T[sa] dZ2, dH1^T (+)= W2[sa] dZ2^T
+            const uint64_t a = desc_mnmajor(w2_ + 2u * sa * kPanelBytes, 0), b = desc_mnmajor(b_, 0), bk = desc_kmajor(b_, 0);
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) mma(tb + T_Z, a + mnstep(kk), b + mnstep(kk), id_dh, !first || kk > 0);
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+                mma_ts(tb + T_DW2, tb + T_ACT + 64u * sa + 8u * kk, bk + kstep(kk), id_z1, !first || kk > 0);
+        };
+        auto de_batch = [&](uint32_t b_, int sb, bool first) {   // de (+)= dZ1 W1[sb][0:16]^T
+            const uint64_t a = desc_mnmajor(b_, 0), b = desc_mnmajor(w1_ + sb * kPanelBytes, 0);
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)   // units 0-63 and 64-127 apart (the second where dW1 will be)
+                mma(tb + (kk < 4 ? T_DE : T_DW1), a + mnstep(kk), b + mnstep(kk), id_de, !first || (kk & 3) > 0);
+        };
+        // copies the hi third of the activations from TMEM into the pool's first buffer
+        auto stage_hi = [&]() {
+#pragma unroll 1
+            for (int g = 0; g < 2; ++g) {
+                float v[16];
+                tmem_ld16(taddr(tb, warp, T_ACT + 32 * hc + 16 * g), v);
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    *reinterpret_cast<uint4 *>(buf0 + panel_offset(n, 32 * g + 8 * c)) =
+                        make_uint4(__float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]), __float_as_uint(v[4 * c + 2]),
+                                   __float_as_uint(v[4 * c + 3]));
+            }
+        };
+
+        float acc2[64], acc1[32], a3[3] = {0.0f, 0.0f, 0.0f}, ab2 = 0.0f, ab3[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int j = 0; j < 64; ++j) acc2[j] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc1[j] = 0.0f;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+            if (!mbar_wait(&S.full, 0, A.wait_ns)) { ok = false; break; }
+            fence_after();
+            if (tid == 0) {
+                const uint64_t a = desc_kmajor(w1_, 0), b = desc_kmajor(pool_, 0);
+#pragma unroll
+                for (int p = 0; p < 6; ++p)
+#pragma unroll
+                    for (int kk = 0; kk < KB; ++kk)
+                        mma(tb + T_Z, a + PA[p] * kPanelStep + kstep(kk), b + PB[p] * kPanelStep + kstep(kk), id_z1, (p | kk) != 0);
+                commit(&S.mma_a);
+            }
+            if (hc == 0) {
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch) ab3[ch] += S.dout[ch][n];
+            }
+            if (!wait_a()) { ok = false; break; }
+            // ---- epilogue 1: H1 = relu(Z1), split: TMEM (A of dW2), lo and mid into the pool ----
+            uint32_t m1[4], m2[4];   // which units are off: 16 samples a word, sample k in bit 15 - k
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                float z[16];
+                tmem_ld16(taddr(tb, warp, T_Z + 64 * hc + 16 * g), z);
+                uint32_t neg = 0;   // sign bits, sample k in bit 15 - k
+                float near = 1.0f;  // below zero when a unit is within rounding of zero
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) {
+                    const float4 x4 = *reinterpret_cast<const float4 *>(&S.xmax[64 * hc + 16 * g + k]);
+                    const float xm[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        neg = __funnelshift_l(__float_as_uint(z[k + j]), neg, 1);
+                        near = fminf(near, fmaf(-eps1, xm[j], fabsf(z[k + j])));
+                    }
+                }
+                if (__any_sync(FULL, near < 0.0f)) {
+                    uint32_t amb = 0;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k)
+                        amb |= (fmaf(-eps1, S.xmax[64 * hc + 16 * g + k], fabsf(z[k])) < 0.0f ? 1u : 0u) << k;
+                    neg = resolve<FeatT, PK, 1>(A, tile * TM + 64 * hc + 16 * g, n, amb, neg);
+                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) z[k] = fmaxf(z[k], 0.0f);
+                m1[g] = neg;
+                uint32_t w[3][8];
+                split16(z, w);
+                store16(buf0, n, g, w[2]);
+                store16(buf1, n, g, w[1]);
+#pragma unroll
+                for (int s = 0; s < 3; ++s) tmem_st8(taddr(tb, warp, T_ACT + 64 * s + 32 * hc + 8 * g), w[s]);
+            }
+            tmem_wait_st();
+            publish();
+            // ---- layer 2 ----
+            if (tid == 0) {
+                z2_batch(b0_, 0, true);
+                commit(&S.mma_a);
+                z2_batch(b1_, 1, false);
+                z2_batch(b1_, 0, false);
+                commit(&S.mma_b);
+            }
+            b_out = true;
+            if (!wait_a()) { ok = false; break; }
+            stage_hi();
+            publish();
+            if (tid == 0) {
+                z2_batch(b0_, 2, false);
+                z2_batch(b0_, 1, false);
+                z2_batch(b0_, 0, false);
+                commit(&S.mma_a);
+            }
+            if (!wait_b() || !wait_a()) { ok = false; break; }
+            // ---- epilogue 2: dZ2, dW3, db2 (a tile's sums first, then the running ones) ----
+            float t3[3] = {0.0f, 0.0f, 0.0f}, tb2 = 0.0f;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                float z[16];
+                tmem_ld16(taddr(tb, warp, T_Z + 64 * hc + 16 * g), z);
+                uint32_t neg = 0;
+                float near = 1.0f;
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) {
+                    float d[3][4], xm[4];
+                    load_dout(S, 64 * hc + 16 * g + k, d);
+                    *reinterpret_cast<float4 *>(xm) = *reinterpret_cast<const float4 *>(&S.xmax[64 * hc + 16 * g + k]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float zz = z[k + j] + b2, h = fmaxf(zz, 0.0f);
+                        neg = __funnelshift_l(__float_as_uint(zz), neg, 1);
+                        near = fminf(near, fmaf(-eps2, xm[j], fabsf(zz)));
+                        t3[0] = fmaf(h, d[0][j], t3[0]);
+                        t3[1] = fmaf(h, d[1][j], t3[1]);
+                        t3[2] = fmaf(h, d[2][j], t3[2]);
+                    }
+                }
+                if (__any_sync(FULL, near < 0.0f)) {
+                    uint32_t amb = 0;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k)
+                        amb |= (fmaf(-eps2, S.xmax[64 * hc + 16 * g + k], fabsf(z[k] + b2)) < 0.0f ? 1u : 0u) << k;
+                    neg = resolve<FeatT, PK, 2>(A, tile * TM + 64 * hc + 16 * g, n, amb, neg);
+                }
+                m2[g] = neg;
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) {
+                    float d[3][4];
+                    load_dout(S, 64 * hc + 16 * g + k, d);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float v = fmaf(d[2][j], w32, fmaf(d[1][j], w31, d[0][j] * w30));
+                        z[k + j] = off(neg, k + j) ? 0.0f : v;
+                        tb2 += z[k + j];
+                    }
+                }
+                uint32_t w[3][8];
+                split16(z, w);
+                store16(buf0, n, g, w[2]);
+                store16(buf1, n, g, w[1]);
+            }
+            ab2 += tb2;
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) a3[ch] += t3[ch];
+            publish();
+            // ---- dW2 and dH1 ----
+            if (tid == 0) {
+                dz2_batch(b0_, 0, true);
+                commit(&S.mma_a);
+                dz2_batch(b1_, 1, false);
+                dz2_batch(b1_, 0, false);
+                commit(&S.mma_b);
+            }
+            b_out = true;
+            if (!wait_a()) { ok = false; break; }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {   // the hi third again from dout
+                uint32_t w[8];
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) {
+                    float d[3][4], v[4];
+                    load_dout(S, 64 * hc + 16 * g + k, d);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        v[j] = fmaf(d[2][j], w32, fmaf(d[1][j], w31, d[0][j] * w30));
+                        v[j] = off(m2[g], k + j) ? 0.0f : v[j];
+                    }
+                    w[k / 2] = pack_bf16(v[0], v[1]);
+                    w[k / 2 + 1] = pack_bf16(v[2], v[3]);
+                }
+                store16(buf0, n, g, w);
+            }
+            publish();
+            if (tid == 0) {
+                dz2_batch(b0_, 2, false);
+                dz2_batch(b0_, 1, false);
+                dz2_batch(b0_, 0, false);
+                commit(&S.mma_a);
+            }
+            if (!wait_b() || !wait_a()) { ok = false; break; }
+            // ---- epilogue 3: dZ1 = dH1 [Z1 > 0], split: TMEM (A of dW1), lo and mid into the pool; dW2 ----
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                float z[16];
+                tmem_ld16(taddr(tb, warp, T_Z + 64 * hc + 16 * g), z);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) z[k] = off(m1[g], k) ? 0.0f : z[k];
+                uint32_t w[3][8];
+                split16(z, w);
+                store16(buf0, n, g, w[2]);
+                store16(buf1, n, g, w[1]);
+#pragma unroll
+                for (int s = 0; s < 3; ++s) tmem_st8(taddr(tb, warp, T_ACT + 64 * s + 32 * hc + 8 * g), w[s]);
+            }
+            tmem_wait_st();
+            publish();
+            // ---- de ----
+            if (tid == 0) {
+                de_batch(b0_, 0, true);
+                commit(&S.mma_a);
+                de_batch(b1_, 1, false);
+                de_batch(b1_, 0, false);
+                commit(&S.mma_b);
+            }
+            b_out = true;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {   // this tile's dW2, beside the MMAs
+                float v[16];
+                tmem_ld16(taddr(tb, warp, T_DW2 + 64 * hc + 16 * g), v);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) acc2[16 * g + k] += v[k];
+            }
+            if (!wait_a()) { ok = false; break; }
+            stage_hi();
+            publish();
+            if (tid == 0) {
+                de_batch(b0_, 2, false);
+                de_batch(b0_, 1, false);
+                de_batch(b0_, 0, false);
+                commit(&S.mma_a);
+            }
+            if (!wait_b() || !wait_a()) { ok = false; break; }
+            if (tid == 0) mbar_arrive(&S.empty);   // the pool is free for X
+            float de[16], de2[16];
+            if (hc == 0) {   // lane = sample here
+                tmem_ld16(taddr(tb, warp, T_DE), de);
+                tmem_ld16(taddr(tb, warp, T_DW1), de2);
+            }
+            // (X staged again: the producers are also done with the de of the tile before)
+            if (!mbar_wait(&S.full, 1, A.wait_ns)) { ok = false; break; }
+            if (hc == 0) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    S.de[n][k] = make_float4(de[4 * k] + de2[4 * k], de[4 * k + 1] + de2[4 * k + 1], de[4 * k + 2] + de2[4 * k + 2],
+                                             de[4 * k + 3] + de2[4 * k + 3]);
+            }
+            consumer_sync();   // T_DW1 read
+            // ---- dW1 ----
+            if (tid == 0) {
+                const uint64_t b = desc_mnmajor(pool_, 0);
+#pragma unroll
+                for (int p = 0; p < 6; ++p)
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)
+                        mma_ts(tb + T_DW1, tb + T_ACT + 64u * PA[p] + 8u * kk, b + PB[p] * kPanelStep + mnstep(kk), id_dw1,
+                               (p | kk) != 0);
+                commit(&S.mma_a);
+            }
+            if (!wait_a()) { ok = false; break; }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {   // columns 0-31 / 32-47 of dW1
+                if (hc == 1 && g == 1) break;
+                float v[16];
+                tmem_ld16(taddr(tb, warp, T_DW1 + 32 * hc + 16 * g), v);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) acc1[16 * g + k] += v[k];
+            }
+            consumer_sync();   // de written, TMEM reads done
+            if (tid == 0) mbar_arrive(&S.empty);   // the tile is done
+        }
+        if (!ok) {
+            atomicExch(&S.abort, 1);
+        } else {
+            // grad_mlp = w1 | b1 | w2 | b2 | w3 | b3
+            float *gW1 = A.grad_mlp, *gB1 = gW1 + IN * HID, *gW2 = gB1 + HID, *gB2 = gW2 + HID * HID;
+            float *gW3 = gB2 + HID, *gB3 = gW3 + HID * 3;
+#pragma unroll
+            for (int j = 0; j < 64; ++j) atomicAdd(gW2 + n * HID + 64 * hc + j, acc2[j]);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const int c = 32 * hc + j;
+                if (c < IN) atomicAdd(gW1 + c * HID + n, acc1[j]);
+                else if (c == IN) atomicAdd(gB1 + n, acc1[j]);
+            }
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) {
+                atomicAdd(gW3 + 3 * n + ch, a3[ch]);
+                const float s = warp_sum(ab3[ch]);
+                if (hc == 0 && lane == 0) atomicAdd(gB3 + ch, s);
+            }
+            atomicAdd(gB2 + n, ab2);
+        }
+    }
+
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (S.abort != 0) {
+        if (tid == 0) atomicOr(&A.hdr->flags, 2);
+        // an MMA batch whose completion timed out may still be running: wait (bounded) once more
+        if (tid < NC) {
+            mbar_wait(&S.mma_a, pa ^ 1, A.wait_ns);
+            if (b_out) mbar_wait(&S.mma_b, pb, A.wait_ns);
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) tmem_dealloc(S.tmem_base, NCOLS);
+}
+
+template <typename FeatT, bool PK>
+void launch_split_bwd(const RenderArgs &A, cudaStream_t s) {
+    auto kern = fine_colour_bwd_split_kernel<FeatT, PK>;
+    ensure_smem(reinterpret_cast<const void *>(kern), (int)kBwdSmem);
+    ProfScope ps_(DVGO_K_FINE_COLOUR_BWD, s);
+    kern<<<num_sms(), NC + NP, kBwdSmem, s>>>(A);
+}
+
+}  // namespace
+
+void launch_fine_colour_bwd_fp32(const RenderArgs &A, cudaStream_t s) {
+    const bool bf = A.cdtype == DVGO_DTYPE_BF16;
+    if (A.nfreq_pos > 0) launch_fine_colour_bwd_simt(A, s);
+    else if (A.packed) {
+        if (bf) launch_split_bwd<__nv_bfloat16, true>(A, s);
+        else launch_split_bwd<float, true>(A, s);
+    } else {
+        if (bf) launch_split_bwd<__nv_bfloat16, false>(A, s);
+        else launch_split_bwd<float, false>(A, s);
+    }
+}
+
+}  // namespace dvgo

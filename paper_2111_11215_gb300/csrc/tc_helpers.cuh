@@ -54,6 +54,12 @@ __device__ __forceinline__ uint64_t desc_mnmajor(uint32_t base, int kk) {
     return sdesc(base + (uint32_t)kk * 2u * kGroupBytes, kPanelBytes, kGroupBytes);
 }
 
+// What to add to a descriptor of k-step 0 for k-step kk (the address field counts 16-byte units), and for
+// the next panel.
+constexpr uint64_t kPanelStep = kPanelBytes >> 4;
+__host__ __device__ constexpr uint64_t kstep(int kk) { return (uint64_t)(kk >> 2) * kPanelStep + (uint64_t)(kk & 3) * 2u; }
+__host__ __device__ constexpr uint64_t mnstep(int kk) { return (uint64_t)kk * (2u * kGroupBytes >> 4); }
+
 // Instruction descriptor, kind::f16: D = F32 (bits 4-5 = 1), A = B = BF16 (bits 7-9, 10-12 = 1),
 // A / B major-ness (bit 15 / 16: 1 = MN-major), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
 __device__ __forceinline__ uint32_t idesc_bf16(int M, int N, int a_mn, int b_mn) {
@@ -144,6 +150,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
         "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
         : "memory");
 }
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
+                 "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // TMEM address of (lane base of this warp, column).
@@ -180,6 +191,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity,
         if (done) return true;
         if (globaltimer() - t0 > limit_ns) return false;
     }
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 // Bulk copies (cp.async.bulk, 16-byte aligned addresses, size a multiple of 16).  Shared ->
@@ -221,6 +236,23 @@ __device__ __forceinline__ void panel_store8(unsigned char *panel, int row, int 
     q.z = pack_bf16(v[4], v[5]);
     q.w = pack_bf16(v[6], v[7]);
     *reinterpret_cast<uint4 *>(panel + panel_offset(row, col)) = q;
+}
+
+// Eight FP32 values as three BF16 chunks of 16 bytes: hi, mid, lo.
+__device__ __forceinline__ void split8(const float *v, uint4 (&q)[3]) {
+    uint32_t w[3][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float a = v[2 * i], b = v[2 * i + 1];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            w[s][i] = pack_bf16(a, b);
+            a = __fsub_rn(a, __uint_as_float(w[s][i] << 16));
+            b = __fsub_rn(b, __uint_as_float(w[s][i] & 0xffff0000u));
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) q[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
 }  // namespace tc
