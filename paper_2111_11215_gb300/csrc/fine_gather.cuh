@@ -112,48 +112,44 @@ __device__ __forceinline__ void gather_features(const RenderArgs &A, const Cell 
 // in one lattice cell share all eight corners, and the last row of such a run adds the whole run's
 // weighted de with one set of reductions (the run's other rows add nothing).
 // slot (-1: padding row), cbase and frac: the tile's per-row tables.
-template <bool PK, typename De>
+// kParts: the corners are taken in that many turns (two halve the 96 accumulator registers).
+template <bool PK, int kParts = 1, typename De>
 __device__ __forceinline__ void scatter_row(const RenderArgs &A, const int *slot, const int *cbase,
                                             const float (*frac)[3], De de, int row) {
-    constexpr int TM = 128, FEAT = 12;
+    constexpr int TM = 128, FEAT = 12, NQ = 8 / kParts;
     if (slot[row] < 0) return;
     const int cb = cbase[row];
     if (row + 1 < TM && slot[row + 1] >= 0 && cbase[row + 1] == cb) return;
-    float4 acc[8][3];
-    {
-        const float4 e0 = de(row, 0), e1 = de(row, 1), e2 = de(row, 2);
-        const float fx = frac[row][0], fy = frac[row][1], fz = frac[row][2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
-                            ((q & 1) ? fz : 1.0f - fz);
-            acc[q][0] = make_float4(w * e0.x, w * e0.y, w * e0.z, w * e0.w);
-            acc[q][1] = make_float4(w * e1.x, w * e1.y, w * e1.z, w * e1.w);
-            acc[q][2] = make_float4(w * e2.x, w * e2.y, w * e2.z, w * e2.w);
+    for (int part = 0; part < kParts; ++part) {
+        float4 acc[NQ][3];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) acc[q][0] = acc[q][1] = acc[q][2] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int j = row; j >= 0 && slot[j] >= 0 && cbase[j] == cb; --j) {
+            const float4 e0 = de(j, 0), e1 = de(j, 1), e2 = de(j, 2);
+            const float fx = frac[j][0], fy = frac[j][1], fz = frac[j][2];
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                const int q = part * NQ + i;
+                const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
+                                ((q & 1) ? fz : 1.0f - fz);
+                acc[i][0] = make_float4(fmaf(w, e0.x, acc[i][0].x), fmaf(w, e0.y, acc[i][0].y),
+                                        fmaf(w, e0.z, acc[i][0].z), fmaf(w, e0.w, acc[i][0].w));
+                acc[i][1] = make_float4(fmaf(w, e1.x, acc[i][1].x), fmaf(w, e1.y, acc[i][1].y),
+                                        fmaf(w, e1.z, acc[i][1].z), fmaf(w, e1.w, acc[i][1].w));
+                acc[i][2] = make_float4(fmaf(w, e2.x, acc[i][2].x), fmaf(w, e2.y, acc[i][2].y),
+                                        fmaf(w, e2.z, acc[i][2].z), fmaf(w, e2.w, acc[i][2].w));
+            }
         }
-    }
-    for (int j = row - 1; j >= 0 && slot[j] >= 0 && cbase[j] == cb; --j) {
-        const float4 e0 = de(j, 0), e1 = de(j, 1), e2 = de(j, 2);
-        const float fx = frac[j][0], fy = frac[j][1], fz = frac[j][2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float w = (((q >> 2) & 1) ? fx : 1.0f - fx) * (((q >> 1) & 1) ? fy : 1.0f - fy) *
-                            ((q & 1) ? fz : 1.0f - fz);
-            acc[q][0] = make_float4(fmaf(w, e0.x, acc[q][0].x), fmaf(w, e0.y, acc[q][0].y),
-                                    fmaf(w, e0.z, acc[q][0].z), fmaf(w, e0.w, acc[q][0].w));
-            acc[q][1] = make_float4(fmaf(w, e1.x, acc[q][1].x), fmaf(w, e1.y, acc[q][1].y),
-                                    fmaf(w, e1.z, acc[q][1].z), fmaf(w, e1.w, acc[q][1].w));
-            acc[q][2] = make_float4(fmaf(w, e2.x, acc[q][2].x), fmaf(w, e2.y, acc[q][2].y),
-                                    fmaf(w, e2.z, acc[q][2].z), fmaf(w, e2.w, acc[q][2].w));
+        for (int i = 0; i < NQ; ++i) {
+            const int q = part * NQ + i;
+            const long long idx = corner_from_base(cb, (q >> 2) & 1, (q >> 1) & 1, q & 1, A.ny, A.nz, PK);
+            float4 *g = reinterpret_cast<float4 *>(A.grad_cgrid + idx * FEAT);
+            atomicAdd(g + 0, acc[i][0]);
+            atomicAdd(g + 1, acc[i][1]);
+            atomicAdd(g + 2, acc[i][2]);
         }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const long long idx = corner_from_base(cb, (q >> 2) & 1, (q >> 1) & 1, q & 1, A.ny, A.nz, PK);
-        float4 *g = reinterpret_cast<float4 *>(A.grad_cgrid + idx * FEAT);
-        atomicAdd(g + 0, acc[q][0]);
-        atomicAdd(g + 1, acc[q][1]);
-        atomicAdd(g + 2, acc[q][2]);
     }
 }
 

@@ -60,13 +60,6 @@ constexpr size_t split_smem() {
 }
 static_assert(split_smem<true>() <= 232448, "one CTA per SM (227 KB of shared memory)");
 
-// Split s, columns [8 c, 8 c + 8) of row `row` of an operand of KB blocks a split.
-template <int KB>
-__device__ __forceinline__ uint4 *split_chunk(unsigned char *base, int s, int row, int c) {
-    const int q = s * KB + (c >> 1);
-    return reinterpret_cast<uint4 *>(base + (q >> 2) * kPanelBytes + panel_offset(row, (q & 3) * 16 + (c & 1) * 8));
-}
-
 // Barrier among the 256 consumer threads.
 __device__ __forceinline__ void consumer_sync() {
     fence_before();
@@ -204,14 +197,12 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
             return w;
         };
         auto issue_layer1 = [&]() {
-            uint32_t x_ = smem_u32(xs), w_ = smem_u32(w1t);
-            asm volatile("" : "+r"(x_), "+r"(w_));   // keeps the descriptors out of long-lived registers
+            const uint64_t x = desc_kmajor(smem_u32(xs), 0), w = desc_kmajor(smem_u32(w1t), 0);
 #pragma unroll
             for (int p = 0; p < 6; ++p)
-#pragma unroll 1
+#pragma unroll
                 for (int kk = 0; kk < KB; ++kk)
-                    mma(tb + COL_Z1, desc_kmajor(x_, PA[p] * KB + kk), desc_kmajor(w_, PB[p] * KB + kk), idesc,
-                        (p | kk) != 0);
+                    mma(tb + COL_Z1, x + kstep(PA[p] * KB + kk), w + kstep(PB[p] * KB + kk), idesc, (p | kk) != 0);
             commit(&S.mma);
         };
         int i = 0;
@@ -262,16 +253,15 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
             }
             // ---- layer 2: Z2 = H1 W2, A = H1 from TMEM; inputs 0-63 and 64-127 in accumulators of their own ----
             if (tid == 0) {
-                uint32_t w_ = smem_u32(w2t);
-                asm volatile("" : "+r"(w_));
-#pragma unroll 1
+                const uint64_t w = desc_kmajor(smem_u32(w2t), 0);
+#pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
                     for (int p = 0; p < 6; ++p)
-#pragma unroll 1
+#pragma unroll
                         for (int kk = 4 * h; kk < 4 * h + 4; ++kk)
-                            mma_ts(tb + COL_Z2 + 128u * (uint32_t)h, tb + COL_H1 + 64u * PA[p] + 8u * (uint32_t)kk,
-                                   desc_kmajor(w_ + 2u * PB[p] * kPanelBytes, kk), idesc, p > 0 || kk > 4 * h);
+                            mma_ts(tb + COL_Z2 + 128u * h, tb + COL_H1 + 64u * PA[p] + 8u * kk,
+                                   w + 2 * PB[p] * kPanelStep + kstep(kk), idesc, p > 0 || kk > 4 * h);
                 commit(&S.mma);
             }
             if (!wait_mma()) { ok = false; break; }

@@ -9,7 +9,10 @@
 // (exact_z1 / exact_z2, the order of the SIMT kernel), so the gradients do not hang on which
 // arithmetic recomputed the hidden layers.
 //
-// Bound: 1806 us-equivalents of FMA work left the SIMT kernel at 45 % of the CUDA cores' rate; BWD_NUMBERS
+// Bound: the serial chain of a tile -- seven MMA batches (12 k clocks of the tensor pipe at M = N = 128) and,
+// between them, three epilogues that split 16 k values each on two warps per scheduler; shared memory
+// (weights and 64 KB of activations) leaves no room for a second tile beside it.  160^3, 8,192 rays,
+// 1.38 M samples: 4610 us on the CUDA cores (45 % of their FP32 rate), 1500 us here, 44 k clocks a tile.
 //
 // Per tile of M = 128 kept samples, with dout = dL/do from the compositing backward; activations are kept
 // transposed (TMEM lane = hidden unit, column = sample), so that a thread owns a unit: the sums over the
@@ -22,12 +25,12 @@
 //   dH1^T = W2 dZ2^T                A = W2 (shared, read MN-major), B = dZ2^T
 //   dZ1 = dH1 [Z1 > 0]
 //   de = dZ1 W1[0:12]^T             A = dZ1^T (shared, read MN-major), B = W1 (read MN-major)
-//   [dW1 | db1]^T += dZ1^T X        A = dZ1^T (TMEM), B = X (staged again)
+//   [dW1 | db1]^T += dZ1^T X        A = dZ1^T (TMEM), B = X (staged again; its three terms side by side)
 // Shared memory: W2 split 96 KB, W1 split 48 KB, and a pool of 64 KB that holds X (48 KB), then pairs of
 // 32 KB thirds of the activations, then X again.  Warps 0-7 consume (thread (n, half): unit n = t mod 128,
 // samples 64 half .. +63), warps 8-11 gather X, stage it twice and scatter the feature gradients of the
-// tile before.  TMEM columns: activations' split [0, 192), layer accumulator [192, 320), dW2 [320, 448),
-// dW1 [448, 496), de [496, 512).
+// tile before.  TMEM columns: activations' split [0, 192); layer accumulator [192, 320); dW2, then the second
+// half of dH1 [320, 448); dW1 [192, 336) over both; de [448, 496).
 
 #include "dvgo_internal.cuh"
 #include "fine_gather.cuh"
@@ -43,7 +46,7 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int TM = 128, NC = 256, NP = 128;
 constexpr int HID = 128, FEAT = 12, IN = 39, XK = 40;   // column IN of X is the constant 1 (bias)
 constexpr int KB = 3;                                   // 16-column blocks of X and W1 per split
-constexpr uint32_t T_ACT = 0, T_Z = 192, T_DW2 = 320, T_DW1 = 448, T_DE = 496, NCOLS = 512;
+constexpr uint32_t T_ACT = 0, T_Z = 192, T_DW2 = 320, T_DW1 = 192, T_DE = 448, NCOLS = 512;
 
 struct BwdSmall {
     alignas(16) float dout[3][TM];   // dL/do
@@ -224,61 +227,77 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
         asm volatile("setmaxnreg.dec.sync.aligned.u32 120;");
         const int row = tid - NC;
         struct Row {
-            float v[XK];
-            float4 dout;
-            int slot, cbase;
-            float fx, fy, fz;
+            uint4 q[XK / 8][3];   // the input row's three terms, 8 columns a chunk
+            float d[3], xmax;
+            int slot, ray;        // slot < 0: padding row
+            Cell c;
         };
-        auto gather = [&](int t, Row &w) {
+        // Placing a sample takes two dependent loads (list, ray record); done while the consumers work on the
+        // tile before, with the corners' lines fetched towards the SM, it leaves one short load for the gather.
+        auto place = [&](int t, Row &w) {
             const int e = t * TM + row;
-#pragma unroll
-            for (int k = 0; k < XK; ++k) w.v[k] = 0.0f;
-            w.dout = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             w.slot = -1;
-            w.cbase = 0;
-            w.fx = w.fy = w.fz = 0.0f;
+            w.ray = 0;
+            w.c.i0 = w.c.j0 = w.c.k0 = 0;
+            w.c.fx = w.c.fy = w.c.fz = 0.0f;
             if (t >= ntiles || e >= n_kept) return;
             const int2 kv = A.kept[e];
             const RayPre rp = ray_pre(A, kv.y);
             float dt;
-            const Cell c = cell_pre(A, rp, kv.y, kv.x >> 16, dt);
+            w.c = cell_pre(A, rp, kv.y, kv.x >> 16, dt);
             w.slot = rp.off + (kv.x & 0xffff);
-            w.cbase = cell_base(c, A.ny, A.nz, PK);
-            w.fx = c.fx;
-            w.fy = c.fy;
-            w.fz = c.fz;
-            const float4 g = A.sgrad[w.slot];
-            gather_features<FeatT, PK>(A, c, w.v);
-            const float4 *pe = reinterpret_cast<const float4 *>(A.pe + (size_t)kv.y * kPeStride);
+            w.ray = kv.y;
 #pragma unroll
-            for (int k = 0; k < 7; ++k) {
-                const float4 q4 = __ldg(pe + k);
-                const float q[4] = {q4.x, q4.y, q4.z, q4.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (4 * k + j < 27) w.v[FEAT + 4 * k + j] = q[j];
+            for (int q = 0; q < 4; ++q) {
+                const FeatT *g = static_cast<const FeatT *>(A.cgrid) + corner_index(w.c, 2 * q, A.ny, A.nz, PK) * FEAT;
+                const FeatT *h = static_cast<const FeatT *>(A.cgrid) + corner_index(w.c, 2 * q + 1, A.ny, A.nz, PK) * FEAT;
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(g));
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(h + FEAT - 1));
             }
-            w.v[IN] = 1.0f;
-            float m = 1.0f;
-#pragma unroll
-            for (int k = 0; k < FEAT; ++k) m = fmaxf(m, fabsf(w.v[k]));
-            w.dout = make_float4(g.y, g.z, g.w, m);
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(A.sgrad + w.slot));
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(A.pe + (size_t)kv.y * kPeStride));
         };
-        auto stage = [&](const Row &w) {   // X: one panel per split, columns 0-47
+        auto gather = [&](Row &w) {
+            float v[XK];
 #pragma unroll
-            for (int c = 0; c < 2 * KB; ++c) {
-                uint4 q[3] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
-                if (8 * c < XK) split8(w.v + 8 * c, q);
+            for (int k = 0; k < XK; ++k) v[k] = 0.0f;
+            w.d[0] = w.d[1] = w.d[2] = w.xmax = 0.0f;
+            if (w.slot >= 0) {
+                const float4 g = A.sgrad[w.slot];
+                gather_features<FeatT, PK>(A, w.c, v);
+                const float4 *pe = reinterpret_cast<const float4 *>(A.pe + (size_t)w.ray * kPeStride);
+#pragma unroll
+                for (int k = 0; k < 7; ++k) {
+                    const float4 q4 = __ldg(pe + k);
+                    const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (4 * k + j < 27) v[FEAT + 4 * k + j] = q[j];
+                }
+                v[IN] = 1.0f;
+                w.xmax = 1.0f;
+#pragma unroll
+                for (int k = 0; k < FEAT; ++k) w.xmax = fmaxf(w.xmax, fabsf(v[k]));
+                w.d[0] = g.y;
+                w.d[1] = g.z;
+                w.d[2] = g.w;
+            }
+#pragma unroll
+            for (int c8 = 0; c8 < XK / 8; ++c8) split8(v + 8 * c8, w.q[c8]);
+        };
+        auto stage = [&](const Row &w) {
+#pragma unroll
+            for (int c = 0; c < 2 * KB; ++c)
 #pragma unroll
                 for (int s = 0; s < 3; ++s)
-                    *reinterpret_cast<uint4 *>(pool + s * kPanelBytes + panel_offset(row, 8 * c)) = q[s];
-            }
+                    *split_chunk<KB>(pool, s, row, c) = c < XK / 8 ? w.q[c][s] : make_uint4(0u, 0u, 0u, 0u);
         };
         auto scatter_tile = [&](int t) {
-            scatter_row<PK>(A, S.slot[t], S.cbase[t], S.frac[t], [&](int r, int k) { return S.de[r][k]; }, row);
+            scatter_row<PK, 2>(A, S.slot[t], S.cbase[t], S.frac[t], [&](int r, int k) { return S.de[r][k]; }, row);
         };
         Row cur;
-        gather(blockIdx.x, cur);
+        place(blockIdx.x, cur);
+        gather(cur);
         int i = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
             // the pool is free once the tile before is done (second release of a tile)
@@ -286,26 +305,25 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             stage(cur);
             const int t = i & 1;
             S.slot[t][row] = cur.slot;
-            S.cbase[t][row] = cur.cbase;
-            S.frac[t][row][0] = cur.fx;
-            S.frac[t][row][1] = cur.fy;
-            S.frac[t][row][2] = cur.fz;
-            S.dout[0][row] = cur.dout.x;
-            S.dout[1][row] = cur.dout.y;
-            S.dout[2][row] = cur.dout.z;
-            S.xmax[row] = cur.dout.w;
+            S.cbase[t][row] = cell_base(cur.c, A.ny, A.nz, PK);
+            S.frac[t][row][0] = cur.c.fx;
+            S.frac[t][row][1] = cur.c.fy;
+            S.frac[t][row][2] = cur.c.fz;
+            S.dout[0][row] = cur.d[0];
+            S.dout[1][row] = cur.d[1];
+            S.dout[2][row] = cur.d[2];
+            S.xmax[row] = cur.xmax;
             fence_async_smem();
             mbar_arrive(&S.full);
-            if (i > 0) {
-                // every producer's tables and de of the tile before are in place: they were written before
-                // the consumers' release that this thread has just waited for
-                scatter_tile(t ^ 1);
-            }
+            // every producer's tables and de of the tile before are in place: they were written before
+            // the consumers' release that this thread has just waited for
+            if (i > 0) scatter_tile(t ^ 1);
+            place(tile + gridDim.x, cur);
             if (!mbar_wait(&S.empty, 0, A.wait_ns)) { ok = false; break; }
             stage(cur);   // again, for dW1
             fence_async_smem();
             mbar_arrive(&S.full);
-            gather(tile + gridDim.x, cur);
+            gather(cur);
         }
         if (ok && i > 0) {
             if (!mbar_wait(&S.empty, 1, A.wait_ns)) ok = false;
@@ -330,7 +348,11 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 split8(v, q);
 #pragma unroll
                 for (int s = 0; s < 3; ++s)
-                    *reinterpret_cast<uint4 *>(w1t + s * kPanelBytes + panel_offset(u, 8 * c)) = q[s];
+                    *split_chunk<KB>(w1t, s, u, c) = q[s];
+                if (c < 2)   // the features' columns once more, their three terms side by side in the free blocks
+#pragma unroll
+                    for (int s = 0; s < 3; ++s)
+                        *reinterpret_cast<uint4 *>(w1t + 2 * kPanelBytes + panel_offset(u, 16 * (1 + s) + 8 * c)) = q[s];
             } else {
                 const int c2 = c - 2 * KB;   // 0-15
 #pragma unroll
@@ -356,8 +378,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
         unsigned char *buf0 = pool + hc * kPanelBytes, *buf1 = pool + (2 + hc) * kPanelBytes;   // this thread's halves
         const uint32_t b0_ = pool_, b1_ = pool_ + 2 * kPanelBytes;
         const uint32_t id_z1 = idesc_bf16(128, 128, 0, 0), id_z2 = idesc_bf16(128, 128, 0, 1),
-                       id_dh = idesc_bf16(128, 128, 1, 1), id_de = idesc_bf16(128, 16, 1, 1),
-                       id_dw1 = idesc_bf16(128, 48, 0, 1);
+                       id_dh = idesc_bf16(128, 128, 1, 1);
         constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};   // the six products, small first
         auto wait_a = [&]() -> bool {
             const bool w = mbar_wait(&S.mma_a, pa, A.wait_ns);
@@ -380,19 +401,24 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             for (int kk = 0; kk < 8; ++kk)
                 mma(tb + T_Z, a + kstep(kk), b + mnstep(kk), id_z2, !first || kk > 0);
         };
-        auto dz2_batch = [&](uint32_t b_, int sa, bool first) {  // dW2 (+)= H1^T[sa] dZ2, dH1^T (+)= W2[sa] dZ2^T
-            const uint64_t a = desc_mnmajor(w2_ + 2u * sa * kPanelBytes, 0), b = desc_mnmajor(b_, 0), bk = desc_kmajor(b_, 0);
+        auto dh_batch = [&](uint32_t b_, int sa, bool first) {   // dH1^T (+)= W2[sa] dZ2^T
+            const uint64_t a = desc_mnmajor(w2_ + 2u * sa * kPanelBytes, 0), b = desc_mnmajor(b_, 0);
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) mma(tb + T_Z, a + mnstep(kk), b + mnstep(kk), id_dh, !first || kk > 0);
+        };
+        auto dw2_batch = [&](uint32_t b_, int sa, bool first) {  // dW2 (+)= H1^T[sa] dZ2
+            const uint64_t b = desc_kmajor(b_, 0);
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-                mma_ts(tb + T_DW2, tb + T_ACT + 64u * sa + 8u * kk, bk + kstep(kk), id_z1, !first || kk > 0);
+                mma_ts(tb + T_DW2, tb + T_ACT + 64u * sa + 8u * kk, b + kstep(kk), id_z1, !first || kk > 0);
         };
-        auto de_batch = [&](uint32_t b_, int sb, bool first) {   // de (+)= dZ1 W1[sb][0:16]^T
-            const uint64_t a = desc_mnmajor(b_, 0), b = desc_mnmajor(w1_ + sb * kPanelBytes, 0);
+        // [de hi | de mid | de lo] (+)= dZ1 [W1 hi | W1 mid | W1 lo]^T, the first `terms` of W1 (16 columns each; an
+        // MMA this narrow costs the same for 16 columns as for 48).  The three parts join in FP32.
+        auto de_batch = [&](uint32_t b_, int terms, bool first) {
+            const uint64_t a = desc_mnmajor(b_, 0), b = desc_mnmajor(w1_ + 2 * kPanelBytes + 32u, 0);
+            const uint32_t id = idesc_bf16(128, 16 * terms, 1, 1);
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)   // units 0-63 and 64-127 apart (the second where dW1 will be)
-                mma(tb + (kk < 4 ? T_DE : T_DW1), a + mnstep(kk), b + mnstep(kk), id_de, !first || (kk & 3) > 0);
+            for (int kk = 0; kk < 8; ++kk) mma(tb + T_DE, a + mnstep(kk), b + mnstep(kk), id, !first || kk > 0);
         };
         // copies the hi third of the activations from TMEM into the pool's first buffer
         auto stage_hi = [&]() {
@@ -408,11 +434,11 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             }
         };
 
-        float acc2[64], acc1[32], a3[3] = {0.0f, 0.0f, 0.0f}, ab2 = 0.0f, ab3[3] = {0.0f, 0.0f, 0.0f};
+        float acc2[64], acc1[24], a3[3] = {0.0f, 0.0f, 0.0f}, ab2 = 0.0f, ab3[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int j = 0; j < 64; ++j) acc2[j] = 0.0f;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc1[j] = 0.0f;
+        for (int j = 0; j < 24; ++j) acc1[j] = 0.0f;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             if (!mbar_wait(&S.full, 0, A.wait_ns)) { ok = false; break; }
             fence_after();
@@ -422,7 +448,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 for (int p = 0; p < 6; ++p)
 #pragma unroll
                     for (int kk = 0; kk < KB; ++kk)
-                        mma(tb + T_Z, a + PA[p] * kPanelStep + kstep(kk), b + PB[p] * kPanelStep + kstep(kk), id_z1, (p | kk) != 0);
+                        mma(tb + T_Z, a + kstep(PA[p] * KB + kk), b + kstep(PB[p] * KB + kk), id_z1, (p | kk) != 0);
                 commit(&S.mma_a);
             }
             if (hc == 0) {
@@ -432,10 +458,13 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             if (!wait_a()) { ok = false; break; }
             // ---- epilogue 1: H1 = relu(Z1), split: TMEM (A of dW2), lo and mid into the pool ----
             uint32_t m1[4], m2[4];   // which units are off: 16 samples a word, sample k in bit 15 - k
+            float zz[32];
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
+                if ((g & 1) == 0) tmem_ld32(taddr(tb, warp, T_Z + 64 * hc + 16 * g), zz);
                 float z[16];
-                tmem_ld16(taddr(tb, warp, T_Z + 64 * hc + 16 * g), z);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) z[k] = zz[16 * (g & 1) + k];
                 uint32_t neg = 0;   // sign bits, sample k in bit 15 - k
                 float near = 1.0f;  // below zero when a unit is within rounding of zero
 #pragma unroll
@@ -490,8 +519,10 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             float t3[3] = {0.0f, 0.0f, 0.0f}, tb2 = 0.0f;
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
+                if ((g & 1) == 0) tmem_ld32(taddr(tb, warp, T_Z + 64 * hc + 16 * g), zz);
                 float z[16];
-                tmem_ld16(taddr(tb, warp, T_Z + 64 * hc + 16 * g), z);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) z[k] = zz[16 * (g & 1) + k];
                 uint32_t neg = 0;
                 float near = 1.0f;
 #pragma unroll
@@ -501,9 +532,9 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                     *reinterpret_cast<float4 *>(xm) = *reinterpret_cast<const float4 *>(&S.xmax[64 * hc + 16 * g + k]);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float zz = z[k + j] + b2, h = fmaxf(zz, 0.0f);
-                        neg = __funnelshift_l(__float_as_uint(zz), neg, 1);
-                        near = fminf(near, fmaf(-eps2, xm[j], fabsf(zz)));
+                        const float v = z[k + j] + b2, h = fmaxf(v, 0.0f);
+                        neg = __funnelshift_l(__float_as_uint(v), neg, 1);
+                        near = fminf(near, fmaf(-eps2, xm[j], fabsf(v)));
                         t3[0] = fmaf(h, d[0][j], t3[0]);
                         t3[1] = fmaf(h, d[1][j], t3[1]);
                         t3[2] = fmaf(h, d[2][j], t3[2]);
@@ -539,13 +570,14 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             publish();
             // ---- dW2 and dH1 ----
             if (tid == 0) {
-                dz2_batch(b0_, 0, true);
+                dw2_batch(b0_, 0, true);
+                dh_batch(b0_, 0, true);
                 commit(&S.mma_a);
-                dz2_batch(b1_, 1, false);
-                dz2_batch(b1_, 0, false);
-                commit(&S.mma_b);
+                dw2_batch(b1_, 1, false);
+                dw2_batch(b1_, 0, false);
+                dh_batch(b1_, 1, false);
+                dh_batch(b1_, 0, false);
             }
-            b_out = true;
             if (!wait_a()) { ok = false; break; }
 #pragma unroll
             for (int g = 0; g < 4; ++g) {   // the hi third again from dout
@@ -566,19 +598,41 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             }
             publish();
             if (tid == 0) {
-                dz2_batch(b0_, 2, false);
-                dz2_batch(b0_, 1, false);
-                dz2_batch(b0_, 0, false);
+                dw2_batch(b0_, 2, false);
+                dw2_batch(b0_, 1, false);
+                dw2_batch(b0_, 0, false);
+                commit(&S.mma_b);
+                dh_batch(b0_, 2, false);
+                dh_batch(b0_, 1, false);
+            }
+            b_out = true;
+            if (!wait_b()) { ok = false; break; }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {   // this tile's dW2, beside the MMAs of dH1
+                float v[16];
+                tmem_ld16(taddr(tb, warp, T_DW2 + 64 * hc + 16 * g), v);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) acc2[16 * g + k] += v[k];
+            }
+            consumer_sync();
+            if (tid == 0) {
+                // hi x hi last, units 0-63 on top of the small products, 64-127 in an accumulator of their own
+                // (dW2's, read by now)
+                const uint64_t a = desc_mnmajor(w2_, 0), b = desc_mnmajor(b0_, 0);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma(tb + (kk < 4 ? T_Z : T_DW2), a + mnstep(kk), b + mnstep(kk), id_dh, kk != 4);
                 commit(&S.mma_a);
             }
-            if (!wait_b() || !wait_a()) { ok = false; break; }
-            // ---- epilogue 3: dZ1 = dH1 [Z1 > 0], split: TMEM (A of dW1), lo and mid into the pool; dW2 ----
+            if (!wait_a()) { ok = false; break; }
+            // ---- epilogue 3: dZ1 = dH1 [Z1 > 0], split: TMEM (A of dW1), lo and mid into the pool ----
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
-                float z[16];
+                float z[16], z2[16];
                 tmem_ld16(taddr(tb, warp, T_Z + 64 * hc + 16 * g), z);
+                tmem_ld16(taddr(tb, warp, T_DW2 + 64 * hc + 16 * g), z2);
 #pragma unroll
-                for (int k = 0; k < 16; ++k) z[k] = off(m1[g], k) ? 0.0f : z[k];
+                for (int k = 0; k < 16; ++k) z[k] = off(m1[g], k) ? 0.0f : z[k] + z2[k];
                 uint32_t w[3][8];
                 split16(z, w);
                 store16(buf0, n, g, w[2]);
@@ -590,64 +644,57 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             publish();
             // ---- de ----
             if (tid == 0) {
-                de_batch(b0_, 0, true);
+                de_batch(b1_, 3, true);    // the mid term (with all of W1's, so that it starts all three parts)
+                de_batch(b0_, 1, false);   // lo
                 commit(&S.mma_a);
-                de_batch(b1_, 1, false);
-                de_batch(b1_, 0, false);
-                commit(&S.mma_b);
-            }
-            b_out = true;
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {   // this tile's dW2, beside the MMAs
-                float v[16];
-                tmem_ld16(taddr(tb, warp, T_DW2 + 64 * hc + 16 * g), v);
-#pragma unroll
-                for (int k = 0; k < 16; ++k) acc2[16 * g + k] += v[k];
             }
             if (!wait_a()) { ok = false; break; }
             stage_hi();
             publish();
             if (tid == 0) {
-                de_batch(b0_, 2, false);
-                de_batch(b0_, 1, false);
-                de_batch(b0_, 0, false);
-                commit(&S.mma_a);
-            }
-            if (!wait_b() || !wait_a()) { ok = false; break; }
-            if (tid == 0) mbar_arrive(&S.empty);   // the pool is free for X
-            float de[16], de2[16];
-            if (hc == 0) {   // lane = sample here
-                tmem_ld16(taddr(tb, warp, T_DE), de);
-                tmem_ld16(taddr(tb, warp, T_DW1), de2);
-            }
-            // (X staged again: the producers are also done with the de of the tile before)
-            if (!mbar_wait(&S.full, 1, A.wait_ns)) { ok = false; break; }
-            if (hc == 0) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-                    S.de[n][k] = make_float4(de[4 * k] + de2[4 * k], de[4 * k + 1] + de2[4 * k + 1], de[4 * k + 2] + de2[4 * k + 2],
-                                             de[4 * k + 3] + de2[4 * k + 3]);
-            }
-            consumer_sync();   // T_DW1 read
-            // ---- dW1 ----
-            if (tid == 0) {
-                const uint64_t b = desc_mnmajor(pool_, 0);
-#pragma unroll
-                for (int p = 0; p < 6; ++p)
-#pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_ts(tb + T_DW1, tb + T_ACT + 64u * PA[p] + 8u * kk, b + PB[p] * kPanelStep + mnstep(kk), id_dw1,
-                               (p | kk) != 0);
+                de_batch(b0_, 3, false);
                 commit(&S.mma_a);
             }
             if (!wait_a()) { ok = false; break; }
+            if (tid == 0) mbar_arrive(&S.empty);   // the pool is free for X
+            float de[16];
+            if (hc == 0) {   // lane = sample here
+                float d1[16], d2[16];
+                tmem_ld16(taddr(tb, warp, T_DE + 16), d1);
+                tmem_ld16(taddr(tb, warp, T_DE + 32), d2);
+                tmem_ld16(taddr(tb, warp, T_DE), de);
 #pragma unroll
-            for (int g = 0; g < 2; ++g) {   // columns 0-31 / 32-47 of dW1
-                if (hc == 1 && g == 1) break;
-                float v[16];
-                tmem_ld16(taddr(tb, warp, T_DW1 + 32 * hc + 16 * g), v);
+                for (int k = 0; k < FEAT; ++k) de[k] += d1[k] + d2[k];
+            }
+            // (X staged again: the producers are also done with the de of the tile before)
+            if (!mbar_wait(&S.full, 1, A.wait_ns)) { ok = false; break; }
+            fence_after();
+            // ---- dW1, its three parts by X's terms side by side ----
+            if (tid == 0) {
+                const uint64_t b = desc_mnmajor(pool_, 0);
+                const uint32_t id3 = idesc_bf16(128, 144, 0, 1), id1 = idesc_bf16(128, 48, 0, 1);
 #pragma unroll
-                for (int k = 0; k < 16; ++k) acc1[16 * g + k] += v[k];
+                for (int p = 0; p < 3; ++p) {   // dZ1's mid (starting all parts), lo, hi
+                    const int sa = p == 0 ? 1 : (p == 1 ? 2 : 0);
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)
+                        mma_ts(tb + T_DW1, tb + T_ACT + 64u * sa + 8u * kk, b + mnstep(kk), p == 1 ? id1 : id3, (p | kk) != 0);
+                }
+                commit(&S.mma_a);
+            }
+            if (hc == 0) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) S.de[n][k] = make_float4(de[4 * k], de[4 * k + 1], de[4 * k + 2], de[4 * k + 3]);
+            }
+            if (!wait_a()) { ok = false; break; }
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {   // columns 24 hc + 8 g .. of the three parts
+                float v0[8], v1[8], v2[8];
+                tmem_ld8(taddr(tb, warp, T_DW1 + 24 * hc + 8 * g), v0);
+                tmem_ld8(taddr(tb, warp, T_DW1 + 48 + 24 * hc + 8 * g), v1);
+                tmem_ld8(taddr(tb, warp, T_DW1 + 96 + 24 * hc + 8 * g), v2);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc1[8 * g + k] += v0[k] + (v1[k] + v2[k]);
             }
             consumer_sync();   // de written, TMEM reads done
             if (tid == 0) mbar_arrive(&S.empty);   // the tile is done
@@ -661,8 +708,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
             for (int j = 0; j < 64; ++j) atomicAdd(gW2 + n * HID + 64 * hc + j, acc2[j]);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int c = 32 * hc + j;
+            for (int j = 0; j < 24; ++j) {
+                const int c = 24 * hc + j;
                 if (c < IN) atomicAdd(gW1 + c * HID + n, acc1[j]);
                 else if (c == IN) atomicAdd(gB1 + n, acc1[j]);
             }

@@ -139,6 +139,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // 16 consecutive 32-bit columns of this thread's TMEM lane from registers; the stores are
 // complete (visible to a later MMA after a thread sync with the tcgen05 fences) once
 // tmem_wait_st() returns.
@@ -253,6 +263,14 @@ __device__ __forceinline__ void split8(const float *v, uint4 (&q)[3]) {
     }
 #pragma unroll
     for (int s = 0; s < 3; ++s) q[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+// A split operand of KB 16-column blocks a term: block (term s, kb) is number s KB + kb, four to a panel.
+// 16-byte chunk c (columns 8 c ..) of row `row`, and what to add to a K-major descriptor for a block.
+template <int KB>
+__device__ __forceinline__ uint4 *split_chunk(unsigned char *base, int s, int row, int c) {
+    const int q = s * KB + (c >> 1);
+    return reinterpret_cast<uint4 *>(base + (q >> 2) * kPanelBytes + panel_offset(row, (q & 3) * 16 + (c & 1) * 8));
 }
 
 }  // namespace tc
