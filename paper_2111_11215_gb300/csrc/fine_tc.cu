@@ -1,6 +1,6 @@
 // fine_tc.cu -- colour queries of the fine stage with the BF16 tensor-core MLP (tcgen05, sm_103a).
 //
-// Same function as fine_simt.cu (Sec. 4.2 Eq. fine_queries_rgb, Supp. A: 12 features + PE(d, 4)
+// Same function as fine_tc_fp32.cu and fine_tc_fp32_bwd.cu (Sec. 4.2 Eq. fine_queries_rgb, Supp. A: 12 features + PE(d, 4)
 // = 39 inputs, or 72 with PE(x, 5) appended; two hidden layers of 128 with ReLU, sigmoid output)
 // with the two 128-wide layers
 // and all weight-gradient contractions on the 5th-generation tensor cores: BF16 operands in
@@ -8,7 +8,7 @@
 // issued by one thread, completion signalled through mbarriers.  The 128 -> 3 output layer, the
 // sigmoid and the element-wise steps run on the CUDA cores in the epilogues.
 //
-// Persistent CTAs of 384 threads walk tiles of M = 128 kept samples.  Warps 8-11 (producers)
+// Persistent CTAs walk tiles of M = 128 kept samples.  Warps 8-11 (producers; 8-15 in the forward)
 // gather the next tile -- features at the 8 lattice corners, the ray's direction encoding, the
 // bias column -- into one of two X panels, and in the backward also scatter the feature gradients
 // of the tile that last used that panel.  The forward stores every finished X panel (16 KiB, as
@@ -16,9 +16,18 @@
 // with one bulk copy instead of gathering again (tile t holds the same kept samples in both: the
 // kept list is the forward's), so its producers only form the per-row tables, dL/dc and the PE(x)
 // tail.  Warps 0-7 (consumers)
-// issue the MMAs (thread 0) and run the epilogues: warp w reads TMEM lanes 32 (w % 4)..+31 and
-// handles columns 64 (w / 4)..+63 of those rows, so two warps share each row.  full[b] / empty[b]
-// mbarriers hand the X panels over; every wait is bounded.
+// run the epilogues and, in the forward, issue the MMAs.  full[b] / empty[b] mbarriers hand the X
+// panels over; every wait is bounded.
+//
+// The backward is a chain of MMA batches and epilogues.  Waiting for each batch as a whole, with one
+// thread of an epilogue issuing it, a tile took 11,700 clocks, of which the MMAs are 3,500.  So a warp of
+// its own (warp 12) issues them: what the next epilogue waits for first, the weight gradients behind it, and
+// the next tile's layer 1 before this tile's last batch; dZ1 goes over H2, not H1, so that its epilogue
+// need not wait for dW2, and the next tile's first epilogue runs during dW1.  The consumers hold no barrier
+// among themselves: a warp waits for MMA batches only and signals the issuing warp.  65,536 rays at 256^3
+// (284,928 tiles): 11.55 -> 7.33 ms, the scatter's new form (fine_gather.cuh) included; 310,320 samples: 121 -> 84 us.
+// What bounds it now: the producers (7,400 clocks a tile, 4,800 of them the scatter), the consumers' chain
+// close behind.
 //
 // Inputs beyond the 64 columns of the X panel (PE(x) entries 24-32 of the 72-input row) live in a
 // "tail panel" that also holds W3: columns 0-15 W3 (3 used), 16-31 / 32-47 the tail of X buffer 0 /
@@ -63,8 +72,9 @@ constexpr int NP = 128;        // producer threads of one set (one sample row ea
 #endif
 template <bool BWD>
 constexpr int kProdSets = BWD ? 1 : DVGO_FWD_PROD_SETS;
+// the backward has one more warp, which issues the MMAs
 template <bool BWD>
-constexpr int kThreads = NC + NP * kProdSets<BWD>;   // 384 / 512
+constexpr int kThreads = NC + NP * kProdSets<BWD> + (BWD ? 32 : 0);   // 416 / 512
 constexpr int HID = 128;
 constexpr int FEAT = 12;
 constexpr int NF = 4;
@@ -90,14 +100,21 @@ struct alignas(1024) SmallTC {
     float b2[HID];
     float b3[4];
     float db3[4];
-    // per-row tables of a tile, a ring of 4 (tile i in entry i % 4): the scatter of tile i - 2 reads
-    // other rows' entries while a producer that is done with it already fills tile i or i + 1
-    int slot[4][TM];          // sample slot per row, -1 for padding rows
-    int cbase[4][TM];         // flat index of the base lattice corner
-    float frac[4][TM][3];     // fractional offsets
+    // per-row tables of a tile.  Forward: the sample slot (-1 for padding rows), a ring of 4 (tile i in
+    // entry i % 4; a group may still read its entry when its X buffer is handed back).  Backward: what the
+    // scatter of tile i needs, which runs after tile i + 2 is placed
+    union {
+        int slot[4][TM];
+        float4 place[4][TM];
+    };
+    ScatterTab tab[NP / 32];  // backward
     float dc[2][TM][3];       // dL/dc (backward)
-    uint64_t full[2], empty[2], mma, mma1;   // mma1: the forward's second consumer group
-    uint64_t xl[2];           // backward: the bulk load of X panel b from the forward's copy
+    uint64_t full[2], empty[2];
+    uint64_t mma[2];          // forward: the MMAs of consumer group 0 / 1
+    // backward.  xl: the bulk load of X panel b from the forward's copy; z1, z2, dh, de: MMA batches
+    // complete; ev[e]: consumers have finished epilogue e; fin: every MMA of the launch complete; drained:
+    // the producers have scattered all tiles but the last two
+    uint64_t xl[2], z1, z2, dh, de, ev[4], fin, drained;
     uint32_t tmem_base;
     int abort;
 };
@@ -123,19 +140,6 @@ static_assert(offsetof(SmemTC, dout) == offsetof(SmemTC, h1) + 2 * kPanelBytes, 
 constexpr size_t smem_bytes(bool bwd) { return (bwd ? sizeof(SmemTC) : offsetof(SmemTC, dz2)) + 1024; }
 static_assert(smem_bytes(true) <= 232448, "the backward must fit one CTA per SM (227 KB of shared memory)");
 
-// Barrier among the 256 consumer threads only (the producers run on their own schedule).
-__device__ __forceinline__ void consumer_sync() {
-    fence_before();
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    fence_after();
-}
-
-// Operands written by the consumers become visible to the tensor core, then the consumers sync.
-__device__ __forceinline__ void consumer_publish() {
-    fence_async_smem();
-    consumer_sync();
-}
-
 // 16-byte chunk k (0-2) of the de[0:12] slot of X buffer b in row r of the dout panel.
 __device__ __forceinline__ float4 *de_slot(unsigned char *dout, int b, int r, int k) {
     return reinterpret_cast<float4 *>(dout + panel_offset(r, 8 * (2 + 3 * b + k)));
@@ -145,7 +149,7 @@ __device__ __forceinline__ float4 *de_slot(unsigned char *dout, int b, int r, in
 // prefetched data rp) into X panel b (and its tail) and the per-row tables.
 template <typename FeatT, bool BWD, bool PEX, bool PK>
 __device__ __forceinline__ void produce_row(const RenderArgs &A, SmemTC &S, int b, int t, int2 kv,
-                                            const RayPre &rp, int row, bool cached) {
+                                            const RayPre &rp, const float4 &gc, int row, bool cached) {
     // cached (backward): the X panel arrives by bulk copy; only the tables, dL/dc and the tail here
     using D = TcDims<PEX>;
     float v[64], tail[16];
@@ -153,19 +157,16 @@ __device__ __forceinline__ void produce_row(const RenderArgs &A, SmemTC &S, int 
     for (int i = 0; i < 64; ++i) v[i] = 0.0f;
 #pragma unroll
     for (int i = 0; i < 16; ++i) tail[i] = 0.0f;
-    int slot = -1, cbase = 0;
-    float fx = 0.0f, fy = 0.0f, fz = 0.0f, d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
+    int slot = -1;
+    float4 place = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));
+    float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
     if (kv.y >= 0) {
         float dt;
         const Cell c = cell_pre(A, rp, kv.y, kv.x >> 16, dt);
         slot = rp.off + (kv.x & 0xffff);
-        cbase = cell_base(c, A.ny, A.nz, PK);
-        fx = c.fx;
-        fy = c.fy;
-        fz = c.fz;
         if (BWD) {
+            place = row_place(A, c, true, PK);
             // dout = dL/dc c (1 - c), formed by the compositing backward with the forward's colour c
-            const float4 gc = A.sgrad[slot];
             d0 = gc.y;
             d1 = gc.z;
             d2 = gc.w;
@@ -204,12 +205,9 @@ __device__ __forceinline__ void produce_row(const RenderArgs &A, SmemTC &S, int 
         panel_store8(S.tp, row, 16 * (1 + b), tail);
         panel_store8(S.tp, row, 16 * (1 + b) + 8, tail + 8);
     }
-    S.sm.slot[t][row] = slot;
-    S.sm.cbase[t][row] = cbase;
-    S.sm.frac[t][row][0] = fx;
-    S.sm.frac[t][row][1] = fy;
-    S.sm.frac[t][row][2] = fz;
+    if (!BWD) S.sm.slot[t][row] = slot;
     if (BWD) {
+        S.sm.place[t][row] = place;
         S.sm.dc[b][row][0] = d0;
         S.sm.dc[b][row][1] = d1;
         S.sm.dc[b][row][2] = d2;
@@ -227,12 +225,21 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
     if (tid == 0) {
         mbar_init(&S.sm.full[0], NP);
         mbar_init(&S.sm.full[1], NP);
-        mbar_init(&S.sm.empty[0], 1);
-        mbar_init(&S.sm.empty[1], 1);
-        mbar_init(&S.sm.mma, 1);
-        mbar_init(&S.sm.mma1, 1);
-        mbar_init(&S.sm.xl[0], 1);
-        mbar_init(&S.sm.xl[1], 1);
+        mbar_init(&S.sm.empty[0], BWD ? 4 : 1);
+        mbar_init(&S.sm.empty[1], BWD ? 4 : 1);
+        mbar_init(&S.sm.mma[0], 1);
+        mbar_init(&S.sm.mma[1], 1);
+        if (BWD) {
+            mbar_init(&S.sm.xl[0], 1);
+            mbar_init(&S.sm.xl[1], 1);
+            mbar_init(&S.sm.z1, 1);
+            mbar_init(&S.sm.z2, 1);
+            mbar_init(&S.sm.dh, 1);
+            mbar_init(&S.sm.de, 1);
+            for (int e = 0; e < 4; ++e) mbar_init(&S.sm.ev[e], NC / 32);
+            mbar_init(&S.sm.fin, 1);
+            mbar_init(&S.sm.drained, NP);
+        }
         S.sm.abort = 0;
     }
     if (warp == 0) tmem_alloc(&S.sm.tmem_base, NCOLS);
@@ -276,7 +283,12 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         if (tid < 3) S.sm.b3[tid] = A.b3[tid];
         if (tid < 4) S.sm.db3[tid] = 0.0f;
     }
-    if (tid < NC) consumer_publish();
+    if (tid < NC || tid >= NC + NP * kProdSets<BWD>) {   // weights staged: all that issue MMAs may use them
+        fence_async_smem();
+        fence_before();
+        asm volatile("bar.sync 1, %0;" ::"n"(NC + (BWD ? 32 : 0)) : "memory");
+        fence_after();
+    }
 
     const int n_kept = A.hdr->n_kept;
     const int ntiles = (n_kept + TM - 1) / TM;
@@ -286,7 +298,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
     bool ok = true;
     int ntile_mine = 0;
 
-    if (tid >= NC) {
+    if (tid >= NC && tid < NC + NP * kProdSets<BWD>) {
         // ------------------------------- producers -------------------------------
         // Set pset takes the CTA's tiles i = pset, pset + nsets, ... (X buffer i & 1).  Software-
         // pipelined a tile deep: while producing a tile, a producer already has its set's next tile's
@@ -299,13 +311,17 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             const int e = t * TM + row;
             return (t < ntiles && e < n_kept) ? A.kept[e] : make_int2(-1, -1);
         };
-        auto scatter_tile = [&](int b, int t) {   // X buffer b, entry t of the table ring
-            scatter_row<PK>(A, S.sm.slot[t], S.sm.cbase[t], S.sm.frac[t],
-                            [&](int r, int k) { return *de_slot(S.dout, b, r, k); }, row);
+        auto scatter_tile = [&](int j) {   // the CTA's tile j
+            scatter_rows<PK>(A, S.sm.place[j & 3], [&](int r, int k) { return de_slot(S.dout, j & 1, r, k); },
+                             S.sm.tab[row >> 5], row);
+        };
+        auto dldo_at = [&](const int2 &kv, const RayPre &rp) -> float4 {
+            return (BWD && kv.y >= 0) ? A.sgrad[rp.off + (kv.x & 0xffff)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         };
         const int tile0 = (int)blockIdx.x + pset * (int)gridDim.x;
         int2 kv_cur = kept_at(tile0);
         RayPre rp_cur = kv_cur.y >= 0 ? ray_pre(A, kv_cur.y) : RayPre{};
+        float4 gc_cur = dldo_at(kv_cur, rp_cur);
         int2 kv_next = kept_at(tile0 + stride);
         int nload[2] = {0, 0};   // row 0, backward: bulk loads issued into X panel 0 / 1
         int i = pset;
@@ -313,29 +329,33 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             const int b = i & 1;
             const RayPre rp_next = kv_next.y >= 0 ? ray_pre(A, kv_next.y) : RayPre{};
             const int2 kv_after = kept_at(tile + 2 * stride);
-            if (i >= 2 && !mbar_wait(&S.sm.empty[b], ((i >> 1) - 1) & 1, A.wait_ns)) {
+            if (i >= 2) ok = mbar_wait(&S.sm.empty[b], ((i >> 1) - 1) & 1, A.wait_ns);
+            // (the warp leaves as one: the scatter is a warp's work)
+            if (__any_sync(0xffffffffu, !ok)) {
                 ok = false;
                 break;
             }
-            if (*(volatile int *)&S.sm.abort) break;
+            if (__any_sync(0xffffffffu, *(volatile int *)&S.sm.abort != 0)) break;
             if (cached && row == 0) {   // X panel b is free: the forward's copy of this tile's panel
                 bulk_load(S.x[b], A.xcache + (size_t)tile * kPanelBytes, kPanelBytes, &S.sm.xl[b]);
                 ++nload[b];
             }
-            if (BWD && i >= 2) scatter_tile(b, (i - 2) & 3);   // feature gradients of tile i - 2
-            produce_row<FeatT, BWD, PEX, PK>(A, S, b, i & 3, kv_cur, rp_cur, row, cached);
+            produce_row<FeatT, BWD, PEX, PK>(A, S, b, i & 3, kv_cur, rp_cur, gc_cur, row, cached);
             fence_async_smem();
             // (testing aid: one arrival withheld on a chosen tile makes the consumers' wait run out)
             if (!(row == 0 && tile + 1 == A.withhold_tile)) mbar_arrive(&S.sm.full[b]);
+            if (BWD && i >= 2) scatter_tile(i - 2);   // its de stays until tile i + 1 is full
+            gc_cur = dldo_at(kv_next, rp_next);
             kv_cur = kv_next;
             rp_cur = rp_next;
             kv_next = kv_after;
         }
+        if (BWD) mbar_arrive(&S.sm.drained);
         if (BWD && ok) {
             // the last (up to) two tiles: wait until the consumers are done with them, then scatter
             for (int j = (i >= 2 ? i - 2 : 0); j < i && ok; ++j) {
-                if (!mbar_wait(&S.sm.empty[j & 1], (j >> 1) & 1, A.wait_ns)) ok = false;
-                else if (!*(volatile int *)&S.sm.abort) scatter_tile(j & 1, j & 3);
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.sm.empty[j & 1], (j >> 1) & 1, A.wait_ns));
+                if (ok && !__any_sync(0xffffffffu, *(volatile int *)&S.sm.abort != 0)) scatter_tile(j);
             }
         }
         // every bulk load issued has landed before the CTA can exit (bounded)
@@ -355,7 +375,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         constexpr uint32_t F_H1 = 0, F_H2 = 64, F_Z2 = 128, F_O = 128;
         const int grp = warp >> 2, r = tid & (TM - 1);
         const uint32_t tb = S.sm.tmem_base + 256u * (uint32_t)grp;
-        uint64_t *mbar = grp ? &S.sm.mma1 : &S.sm.mma;
+        uint64_t *mbar = &S.sm.mma[grp];
         uint32_t mphase = 0;
         auto wait_mma = [&]() -> bool {
             bool w = mbar_wait(mbar, mphase, A.wait_ns);
@@ -399,20 +419,20 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             }
             // ---- epilogue 1: H1 = relu(Z1), all 128 columns of my row, as BF16 into TMEM (32-column
             //      chunk g of Z1 becomes columns 16 g .. 16 g + 15, which chunks before g held) ----
-#pragma unroll 1
+#pragma unroll
             for (int g = 0; g < 4; ++g) {
                 float z[32];
                 tmem_ld32(taddr(tb, warp, COL_Z1 + 32 * g), z);
                 uint32_t h[16];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) h[k] = pack_bf16(fmaxf(z[2 * k], 0.0f), fmaxf(z[2 * k + 1], 0.0f));
+                for (int k = 0; k < 16; ++k) h[k] = relu_bf16(pack_bf16(z[2 * k], z[2 * k + 1]));
                 tmem_st16(taddr(tb, warp, F_H1 + 16 * g), h);
             }
             tmem_wait_st();
             group_sync();
             // ---- layer 2: Z2 = H1 W2, A = H1 from TMEM ----
             if (r == 0) {
-#pragma unroll 1
+#pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     mma_ts(tb + F_Z2, tb + F_H1 + 8u * (uint32_t)kk, desc_kmajor(w2t_, kk), idesc_bf16(128, 128, 0, 0),
                            kk > 0);
@@ -420,7 +440,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             }
             if (!wait_mma()) { ok = false; break; }
             // ---- epilogue 2: H2 = relu(Z2 + b2), as BF16 into TMEM ----
-#pragma unroll 1
+#pragma unroll
             for (int g = 0; g < 4; ++g) {
                 float z[32];
                 tmem_ld32(taddr(tb, warp, F_Z2 + 32 * g), z);
@@ -428,8 +448,8 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
 #pragma unroll
                 for (int k = 0; k < 32; k += 4) {
                     const float4 bb = *reinterpret_cast<const float4 *>(&S.sm.b2[32 * g + k]);
-                    h[k / 2] = pack_bf16(fmaxf(z[k] + bb.x, 0.0f), fmaxf(z[k + 1] + bb.y, 0.0f));
-                    h[k / 2 + 1] = pack_bf16(fmaxf(z[k + 2] + bb.z, 0.0f), fmaxf(z[k + 3] + bb.w, 0.0f));
+                    h[k / 2] = relu_bf16(pack_bf16(z[k] + bb.x, z[k + 1] + bb.y));
+                    h[k / 2 + 1] = relu_bf16(pack_bf16(z[k + 2] + bb.z, z[k + 3] + bb.w));
                 }
                 tmem_st16(taddr(tb, warp, F_H2 + 16 * g), h);
             }
@@ -437,7 +457,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             group_sync();
             // ---- layer 3: O = H2 W3 (N = 16, columns 0-2 used), A = H2 from TMEM ----
             if (r == 0) {
-#pragma unroll 1
+#pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     mma_ts(tb + F_O, tb + F_H2 + 8u * (uint32_t)kk, desc_mnmajor(w3p_, kk), idesc_bf16(128, 16, 0, 1),
                            kk > 0);
@@ -453,68 +473,159 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         }
         if (r == 0 && A.xcache) bulk_wait_all();   // the copies are complete before the kernel ends
         if (!ok) atomicExch(&S.sm.abort, 1);
+    } else if (warp == NC / 32 + NP / 32) {
+        // ------------------------------- MMA issue (backward) -------------------------------
+        // One thread issues a tile's batches as their operands become ready, and the next tile's layer 1 as
+        // soon as its X panel is there, so that it is complete when the consumers come to it:
+        //   Z1(0) | Z2, dH2 | dW3 | dH1 | dW2, then Z1 of the next tile | de, dW1
+        if ((tid & 31) == 0) {
+            const uint32_t tb = S.sm.tmem_base;
+            auto wait = [&](uint64_t *bar, uint32_t par) -> bool {
+                ok = ok && mbar_wait(bar, par, A.wait_ns);
+                fence_after();
+                return ok;
+            };
+            // descriptors of k-step 0; the steps are constants added to them, so that a batch is issued
+            // faster than the tensor core takes it
+            const uint64_t x_k = desc_kmajor(smem_u32(S.x[0]), 0), x_m = desc_mnmajor(smem_u32(S.x[0]), 0);
+            const uint64_t w1_k = desc_kmajor(smem_u32(S.w1t), 0), w1_m = desc_mnmajor(smem_u32(S.w1t), 0);
+            const uint64_t w2_k = desc_kmajor(smem_u32(S.w2t), 0), w2_m = desc_mnmajor(smem_u32(S.w2t), 0);
+            const uint64_t h1_k = desc_kmajor(smem_u32(S.h1), 0), h1_m = desc_mnmajor(smem_u32(S.h1), 0);
+            const uint64_t h2_k = desc_kmajor(smem_u32(S.h2), 0), h2_m = desc_mnmajor(smem_u32(S.h2), 0);
+            const uint64_t dz2_k = desc_kmajor(smem_u32(S.dz2), 0), dz2_m = desc_mnmajor(smem_u32(S.dz2), 0);
+            const uint64_t do_k = desc_kmajor(smem_u32(S.dout), 0), do_m = desc_mnmajor(smem_u32(S.dout), 0);
+            const uint64_t tp_k = desc_kmajor(smem_u32(S.tp), 0), tp_m = desc_mnmajor(smem_u32(S.tp), 0);
+            auto layer1 = [&](int b) {   // Z1 = X W1; the X tail (k-step 1 + b of the tail panel) against the W1 tail
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    mma(tb + COL_Z1, x_k + (b ? kPanelStep : 0) + kstep(kk), w1_k + kstep(kk), idesc_bf16(128, 128, 0, 0), kk > 0);
+                if (PEX)
+                    mma(tb + COL_Z1, tp_k + (b ? kstep(2) : kstep(1)), tp_k + kstep(3), idesc_bf16(128, 128, 0, 0), 1u);
+                commit(&S.sm.z1);
+            };
+            bool early = false;   // this tile's layer 1 has been issued
+            int i = 0;
+            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
+                const int b = i & 1;
+                const uint32_t par = i & 1, xpar = (i >> 1) & 1;
+                const uint32_t acc_w = i > 0 ? 1u : 0u;   // first tile of this CTA initialises the accumulators
+                if (!early) {
+                    if (!wait(&S.sm.full[b], xpar) || (cached && !wait(&S.sm.xl[b], xpar))) break;
+                    layer1(b);
+                }
+                // ---- layer 2: Z2 = H1 W2; and dH2 = dout W3^T (K = 16: dout's columns [dL/do, 1, 0 ...]
+                //      against the tail panel's [W3, 0 ...]) into Z1's columns, which epilogue 1 has read ----
+                if (!wait(&S.sm.ev[0], par)) break;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma(tb + COL_Z2, h1_k + kstep(kk), w2_k + kstep(kk), idesc_bf16(128, 128, 0, 0), kk > 0);
+                mma(tb + COL_Z1, do_k, tp_k, idesc_bf16(128, 128, 0, 0), 0u);
+                commit(&S.sm.z2);
+                // ---- dW3, while the consumers form dZ2 ----
+                if (!wait(&S.sm.ev[1], par)) break;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma(tb + COL_DW3, h2_m + mnstep(kk), do_m + mnstep(kk), idesc_bf16(128, 16, 1, 1),
+                        acc_w | (kk > 0));
+                // ---- dH1; then, while the consumers form dZ1 (over H2, which dW3 has read), dW2 ----
+                if (!wait(&S.sm.ev[2], par)) break;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma(tb + COL_Z2, dz2_k + kstep(kk), w2_m + mnstep(kk), idesc_bf16(128, 128, 0, 1), kk > 0);
+                commit(&S.sm.dh);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma(tb + COL_DW2T, dz2_m + mnstep(kk), h1_m + mnstep(kk), idesc_bf16(128, 144, 1, 1),
+                        acc_w | (kk > 0));   // [dW2^T | db2]: B = [H1 | dout]
+                // ---- the next tile's layer 1 (its columns were read with dH2), if its X panel comes first ----
+                early = false;
+                const bool more = tile + (int)gridDim.x < ntiles;
+                const uint32_t npar = ((i + 1) >> 1) & 1;
+                const uint64_t t0 = globaltimer();
+                for (;;) {
+                    if (more && !early && mbar_test(&S.sm.full[b ^ 1], npar) &&
+                        (!cached || mbar_test(&S.sm.xl[b ^ 1], npar))) {
+                        fence_after();
+                        layer1(b ^ 1);
+                        early = true;
+                    }
+                    if (mbar_test(&S.sm.ev[3], par)) break;
+                    if (globaltimer() - t0 > A.wait_ns) {
+                        ok = false;
+                        break;
+                    }
+                }
+                fence_after();
+                if (!ok) break;
+                // ---- de = dZ1 W1[0:16]^T and dW1 ----
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    mma(tb + COL_DE, h2_k + kstep(kk), w1_m + mnstep(kk), idesc_bf16(128, 16, 0, 1), kk > 0);
+                    mma(tb + COL_DW1, h2_m + mnstep(kk), x_m + (b ? kPanelStep : 0) + mnstep(kk), idesc_bf16(128, 64, 1, 1),
+                        acc_w | (kk > 0));
+                    if (PEX)
+                        mma(tb + COL_DW1T, h2_m + mnstep(kk), tp_m + (b ? 4u : 2u) + mnstep(kk),
+                            idesc_bf16(128, 16, 1, 1), acc_w | (kk > 0));
+                }
+                commit(&S.sm.de);
+            }
+            if (!ok) atomicExch(&S.sm.abort, 1);
+            commit(&S.sm.fin);   // every MMA is complete before the CTA goes on (bounded)
+            mbar_wait(&S.sm.fin, 0, A.wait_ns);
+        }
+        __syncwarp();
     } else {
         // ------------------------------- consumers -------------------------------
-        // thread: row r = 32 (warp % 4) + lane (its TMEM lane), column half hc = warp / 4
+        // thread: row r = 32 (warp % 4) + lane (its TMEM lane), column half hc = warp / 4.  A warp only ever
+        // overwrites what the MMA batches it has waited for were the last to read, so the consumers need
+        // no barrier among themselves.
         const int r = tid & (TM - 1), hc = tid >> 7;
         const uint32_t tb = S.sm.tmem_base;
-        uint32_t mphase = 0;
         float db3_part[3] = {0.0f, 0.0f, 0.0f};
         int i = 0;
-        // waits for the current MMA batch; on a timeout every consumer leaves the loop
-        auto wait_mma = [&]() -> bool {
-            bool w = mbar_wait(&S.sm.mma, mphase, A.wait_ns);
-            mphase ^= 1;
+        auto wait = [&](uint64_t *bar, uint32_t par) -> bool {
+            ok = __all_sync(0xffffffffu, mbar_wait(bar, par, A.wait_ns));
             fence_after();
-            return w;
+            return ok;
+        };
+        auto signal = [&](uint64_t *bar) {   // my warp's operands are written and its accumulators read
+            fence_async_smem();
+            fence_before();
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(bar);
+        };
+        // de[0:12] of tile j for the producers' scatter; X[j & 1] and de's slot are theirs again
+        auto stage_de = [&](int j) {
+            float de[16];
+            tmem_ld16(taddr(tb, warp, COL_DE), de);
+            *de_slot(S.dout, j & 1, r, 0) = make_float4(de[0], de[1], de[2], de[3]);
+            *de_slot(S.dout, j & 1, r, 1) = make_float4(de[4], de[5], de[6], de[7]);
+            *de_slot(S.dout, j & 1, r, 2) = make_float4(de[8], de[9], de[10], de[11]);
+            fence_before();
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(&S.sm.empty[j & 1]);
         };
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
             const int b = i & 1;
-            const uint32_t acc_w = i > 0 ? 1u : 0u;   // first tile of this CTA initialises the accumulators
-            // opaque copies: keeps the compiler from hoisting every MMA descriptor out of the loop
-            uint32_t x_ = smem_u32(S.x[b]), w1t_ = smem_u32(S.w1t), w2t_ = smem_u32(S.w2t), w3p_ = smem_u32(S.tp);
-            uint32_t h1_ = smem_u32(S.h1), h2_ = smem_u32(S.h2), dz2_ = smem_u32(S.dz2), dout_ = smem_u32(S.dout);
-            asm volatile("" : "+r"(x_), "+r"(w1t_), "+r"(w2t_), "+r"(w3p_), "+r"(h1_), "+r"(h2_), "+r"(dz2_), "+r"(dout_));
-            // (no abort-flag test: consumers reading it on either side of its setting would part at
-            // their named barrier; a failed producer leaves this wait unsatisfied for all of them)
-            if (!mbar_wait(&S.sm.full[b], (i >> 1) & 1, A.wait_ns)) ok = false;
-            else if (cached && !mbar_wait(&S.sm.xl[b], (i >> 1) & 1, A.wait_ns)) ok = false;
-            fence_after();
-            if (!ok) break;
-            // per-row tables of buffer b, read before the buffer is handed back to the producers
-            const int slot = S.sm.slot[i & 3][r];
-            const float d0 = BWD ? S.sm.dc[b][r][0] : 0.0f, d1 = BWD ? S.sm.dc[b][r][1] : 0.0f,
-                        d2 = BWD ? S.sm.dc[b][r][2] : 0.0f;
-            // ---- layer 1: Z1 = X W1 ----
-            if (tid == 0) {
-#pragma unroll 1
-                for (int kk = 0; kk < 4; ++kk)
-                    mma(tb + COL_Z1, desc_kmajor(x_, kk), desc_kmajor(w1t_, kk), idesc_bf16(128, 128, 0, 0), kk > 0);
-                if (PEX)   // the X tail (k-step 1 + b of the tail panel) against the W1 tail (k-step 3)
-                    mma(tb + COL_Z1, desc_kmajor(w3p_, 1 + b), desc_kmajor(w3p_, 3), idesc_bf16(128, 128, 0, 0), 1u);
-                commit(&S.sm.mma);
-            }
-            if (!wait_mma()) { ok = false; break; }
+            const uint32_t par = i & 1;
+            // (no abort-flag test: a failed producer leaves these waits unsatisfied for every thread)
+            if (!wait(&S.sm.full[b], (i >> 1) & 1) || !wait(&S.sm.z1, par)) break;
             // ---- epilogue 1: H1 = relu(Z1), my 64 columns ----
-            uint32_t m1lo = 0u, m1hi = 0u;   // ReLU masks of my 64 columns
-#pragma unroll 1
+            // (The epilogues are bound by the ALU pipe.  So the ReLU is taken, and its derivative looked up,
+            // two values at a time on the BF16 operand: 5 ALU instructions a hidden unit and sample in
+            // all, against 12 with FP32 compares, selects and a bit mask.  z > 0 and bf16(z) > 0 differ
+            // only below 2^-134.)
+#pragma unroll
             for (int g = 0; g < 2; ++g) {
                 float z[32];
                 tmem_ld32(taddr(tb, warp, COL_Z1 + 64 * hc + 32 * g), z);
-                uint32_t bits = 0;
 #pragma unroll
-                for (int k = 0; k < 32; ++k) {
-                    bits |= (z[k] > 0.0f ? 1u : 0u) << k;
-                    z[k] = fmaxf(z[k], 0.0f);
-                }
-                if (g == 0) m1lo = bits;
-                else m1hi = bits;
-#pragma unroll
-                for (int k = 0; k < 32; k += 8) panel_store8(S.h1 + hc * kPanelBytes, r, 32 * g + k, z + k);
+                for (int k = 0; k < 32; k += 8) *panel_chunk(S.h1 + hc * kPanelBytes, r, 32 * g + k) = pack8_relu(z + k);
             }
             // dout = dL/dc c (1 - c), formed by the producers, into the dout panel: the operand of
             // dH2 (issued with layer 2), of dW3 and, through its constant-1 column, of db2
-            if (BWD && hc == 0) {
+            if (hc == 0) {
+                const float d0 = S.sm.dc[b][r][0], d1 = S.sm.dc[b][r][1], d2 = S.sm.dc[b][r][2];
                 db3_part[0] += d0;
                 db3_part[1] += d1;
                 db3_part[2] += d2;
@@ -523,105 +634,63 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
                 q.y = pack_bf16(d2, 1.0f);
                 *reinterpret_cast<uint2 *>(S.dout + panel_offset(r, 0)) = q;
             }
-            consumer_publish();
-            // ---- layer 2: Z2 = H1 W2; in the backward also dH2 = dout W3^T (K = 16: dout's columns
-            //      [dL/do, 1, 0 ...] against the tail panel's [W3, 0 ...]) into Z1's columns, which
-            //      epilogue 1 has read ----
-            if (tid == 0) {
-#pragma unroll 1
-                for (int kk = 0; kk < 8; ++kk)
-                    mma(tb + COL_Z2, desc_kmajor(h1_, kk), desc_kmajor(w2t_, kk), idesc_bf16(128, 128, 0, 0), kk > 0);
-                if (BWD)
-                    mma(tb + COL_Z1, desc_kmajor(dout_, 0), desc_kmajor(w3p_, 0), idesc_bf16(128, 128, 0, 0), 0u);
-                commit(&S.sm.mma);
+            signal(&S.sm.ev[0]);
+            // ---- the tile before: its de, while layer 2 runs (the scatter of the tile three back, which
+            //      had this slot, was done when this tile was full) ----
+            if (i > 0 && hc == 1) {
+                if (!wait(&S.sm.de, par ^ 1)) break;
+                stage_de(i - 1);
             }
-            if (!wait_mma()) { ok = false; break; }
-            // ---- epilogue 2: H2 = relu(Z2 + b2), my 64 columns; in the backward also
-            //      dZ2 = dH2 [Z2 + b2 > 0] ----
-#pragma unroll 1
+            // ---- epilogue 2: H2 = relu(Z2 + b2), then dZ2 = dH2 [Z2 + b2 > 0], my 64 columns ----
+            if (!wait(&S.sm.z2, par)) break;
+            uint4 hw[8];   // my row of H2, then of H1, for the ReLU's derivative
+#pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const int col = 64 * hc + 32 * g;
-                float z[32], dz[32];
+                float z[32];
                 tmem_ld32(taddr(tb, warp, COL_Z2 + col), z);
-                if (BWD) tmem_ld32(taddr(tb, warp, COL_Z1 + col), dz);
 #pragma unroll
                 for (int k = 0; k < 32; k += 4) {
                     const float4 bb = *reinterpret_cast<const float4 *>(&S.sm.b2[col + k]);
-                    const float hb[4] = {bb.x, bb.y, bb.z, bb.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float h = z[k + j] + hb[j];
-                        z[k + j] = fmaxf(h, 0.0f);
-                        if (BWD) dz[k + j] = h > 0.0f ? dz[k + j] : 0.0f;
-                    }
+                    z[k] += bb.x;
+                    z[k + 1] += bb.y;
+                    z[k + 2] += bb.z;
+                    z[k + 3] += bb.w;
                 }
 #pragma unroll
-                for (int k = 0; k < 32; k += 8) panel_store8(S.h2 + hc * kPanelBytes, r, 32 * g + k, z + k);
-                if (BWD) {
+                for (int k = 0; k < 32; k += 8) {
+                    hw[4 * g + k / 8] = pack8_relu(z + k);
+                    *panel_chunk(S.h2 + hc * kPanelBytes, r, 32 * g + k) = hw[4 * g + k / 8];
+                }
+            }
+            signal(&S.sm.ev[1]);
+            auto masked = [&](uint32_t col, unsigned char *dz) {   // dz = dh where h > 0
 #pragma unroll
-                    for (int k = 0; k < 32; k += 8) panel_store8(S.dz2 + hc * kPanelBytes, r, 32 * g + k, dz + k);
-                }
-            }
-            // ---- backward: H2 and dZ2 published for batch A ----
-            consumer_publish();
-            if (tid == 0) {
-#pragma unroll 1
-                for (int kk = 0; kk < 8; ++kk) {
-                    mma(tb + COL_Z2, desc_kmajor(dz2_, kk), desc_mnmajor(w2t_, kk), idesc_bf16(128, 128, 0, 1), kk > 0);  // dH1
-                    mma(tb + COL_DW2T, desc_mnmajor(dz2_, kk), desc_mnmajor(h1_, kk), idesc_bf16(128, 144, 1, 1),
-                        acc_w | (kk > 0));   // [dW2^T | db2]: B = [H1 | dout]
-                    mma(tb + COL_DW3, desc_mnmajor(h2_, kk), desc_mnmajor(dout_, kk), idesc_bf16(128, 16, 1, 1),
-                        acc_w | (kk > 0));
-                }
-                commit(&S.sm.mma);
-            }
-            if (!wait_mma()) { ok = false; break; }
-            // ---- dZ1 = dH1 [Z1 > 0], over H1 ----
-#pragma unroll 1
-            for (int g = 0; g < 2; ++g) {
-                const uint32_t bits = g == 0 ? m1lo : m1hi;
-                float z[32];
-                tmem_ld32(taddr(tb, warp, COL_Z2 + 64 * hc + 32 * g), z);
+                for (int g = 0; g < 2; ++g) {
+                    float z[32];
+                    tmem_ld32(taddr(tb, warp, col + 64 * hc + 32 * g), z);
 #pragma unroll
-                for (int k = 0; k < 32; ++k) z[k] = ((bits >> k) & 1u) ? z[k] : 0.0f;
+                    for (int k = 0; k < 32; k += 8)
+                        *panel_chunk(dz + hc * kPanelBytes, r, 32 * g + k) = pack8_where(hw[4 * g + k / 8], z + k);
+                }
+            };
+            masked(COL_Z1, S.dz2);
+            signal(&S.sm.ev[2]);
+            // ---- dZ1 = dH1 [Z1 > 0], over H2 ----
 #pragma unroll
-                for (int k = 0; k < 32; k += 8) panel_store8(S.h1 + hc * kPanelBytes, r, 32 * g + k, z + k);
-            }
-            consumer_publish();
-            if (tid == 0) {
-#pragma unroll 1
-                for (int kk = 0; kk < 8; ++kk) {
-                    mma(tb + COL_DE, desc_kmajor(h1_, kk), desc_mnmajor(w1t_, kk), idesc_bf16(128, 16, 0, 1), kk > 0);
-                    mma(tb + COL_DW1, desc_mnmajor(h1_, kk), desc_mnmajor(x_, kk), idesc_bf16(128, 64, 1, 1),
-                        acc_w | (kk > 0));
-                    if (PEX)
-                        mma(tb + COL_DW1T, desc_mnmajor(h1_, kk), desc_mnmajor(w3p_ + 32u * (1 + b), kk),
-                            idesc_bf16(128, 16, 1, 1), acc_w | (kk > 0));
-                }
-                commit(&S.sm.mma);
-            }
-            if (!wait_mma()) { ok = false; break; }
-            // ---- stage de[0:12] for the producers' scatter, then release X[b] ----
-            {
-                float de[16];
-                tmem_ld16(taddr(tb, warp, COL_DE), de);
-                if (hc == 0) {
-                    *de_slot(S.dout, b, r, 0) = make_float4(de[0], de[1], de[2], de[3]);
-                    *de_slot(S.dout, b, r, 1) = make_float4(de[4], de[5], de[6], de[7]);
-                    *de_slot(S.dout, b, r, 2) = make_float4(de[8], de[9], de[10], de[11]);
-                }
-            }
-            consumer_sync();
-            if (tid == 0) mbar_arrive(&S.sm.empty[b]);   // X[b] consumed, de staged
+            for (int c = 0; c < 8; ++c) hw[c] = *panel_chunk(S.h1 + hc * kPanelBytes, r, 8 * c);
+            if (!wait(&S.sm.dh, par)) break;
+            masked(COL_Z2, S.h2);
+            signal(&S.sm.ev[3]);
         }
+        // the last tile's de, once the scatter that had its slot is done
+        if (ok && i > 0 && wait(&S.sm.de, (i - 1) & 1) && hc == 1 && wait(&S.sm.drained, 0)) stage_de(i - 1);
         ntile_mine = i;
         if (!ok) atomicExch(&S.sm.abort, 1);
-        if (BWD) {
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) {
-                const float sum = warp_sum(db3_part[ch]);
-                if ((tid & 31) == 0) atomicAdd(&S.sm.db3[ch], sum);
-            }
+        for (int ch = 0; ch < 3; ++ch) {
+            const float sum = warp_sum(db3_part[ch]);
+            if ((tid & 31) == 0) atomicAdd(&S.sm.db3[ch], sum);
         }
     }
 
@@ -632,7 +701,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
     if (failed) {
         if (tid == 0) atomicOr(&A.hdr->flags, 2);
         // an MMA batch whose completion timed out may still be running: wait (bounded) once more
-        if (tid < NC) mbar_wait((!BWD && tid >= TM) ? &S.sm.mma1 : &S.sm.mma, 0, A.wait_ns);
+        if (!BWD && tid < NC) mbar_wait(&S.sm.mma[tid / TM], 0, A.wait_ns);
     }
     if (BWD && !failed && tid < NC && ntile_mine > 0) {
         const uint32_t tb = S.sm.tmem_base;

@@ -52,8 +52,8 @@ struct BwdSmall {
     alignas(16) float dout[3][TM];   // dL/do
     alignas(16) float xmax[TM];      // largest input magnitude of the row (0: padding row)
     float4 de[TM][3];      // feature gradients of a tile
-    int slot[2][TM], cbase[2][TM];
-    float frac[2][TM][3];
+    float4 place[2][TM];
+    ScatterTab tab[NP / 32];
     uint64_t full, empty, mma_a, mma_b;
     uint32_t tmem_base;
     int abort;
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                     *split_chunk<KB>(pool, s, row, c) = c < XK / 8 ? w.q[c][s] : make_uint4(0u, 0u, 0u, 0u);
         };
         auto scatter_tile = [&](int t) {
-            scatter_row<PK, 2>(A, S.slot[t], S.cbase[t], S.frac[t], [&](int r, int k) { return S.de[r][k]; }, row);
+            scatter_rows<PK>(A, S.place[t], [&](int r, int k) { return &S.de[r][k]; }, S.tab[row >> 5], row);
         };
         Row cur;
         place(blockIdx.x, cur);
@@ -301,33 +301,32 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
         int i = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
             // the pool is free once the tile before is done (second release of a tile)
-            if (i > 0 && !mbar_wait(&S.empty, 1, A.wait_ns)) { ok = false; break; }
+            // (the warp leaves as one: the scatter is a warp's work)
+            if (i > 0) ok = __all_sync(0xffffffffu, mbar_wait(&S.empty, 1, A.wait_ns));
+            if (!ok) break;
             stage(cur);
             const int t = i & 1;
-            S.slot[t][row] = cur.slot;
-            S.cbase[t][row] = cell_base(cur.c, A.ny, A.nz, PK);
-            S.frac[t][row][0] = cur.c.fx;
-            S.frac[t][row][1] = cur.c.fy;
-            S.frac[t][row][2] = cur.c.fz;
+            S.place[t][row] = row_place(A, cur.c, cur.slot >= 0, PK);
             S.dout[0][row] = cur.d[0];
             S.dout[1][row] = cur.d[1];
             S.dout[2][row] = cur.d[2];
             S.xmax[row] = cur.xmax;
             fence_async_smem();
             mbar_arrive(&S.full);
-            // every producer's tables and de of the tile before are in place: they were written before
-            // the consumers' release that this thread has just waited for
+            // de of the tile before is in place: written before the consumers' release that this thread
+            // has just waited for
             if (i > 0) scatter_tile(t ^ 1);
             place(tile + gridDim.x, cur);
-            if (!mbar_wait(&S.empty, 0, A.wait_ns)) { ok = false; break; }
+            ok = __all_sync(0xffffffffu, mbar_wait(&S.empty, 0, A.wait_ns));
+            if (!ok) break;
             stage(cur);   // again, for dW1
             fence_async_smem();
             mbar_arrive(&S.full);
             gather(cur);
         }
         if (ok && i > 0) {
-            if (!mbar_wait(&S.empty, 1, A.wait_ns)) ok = false;
-            else scatter_tile((i - 1) & 1);
+            ok = __all_sync(0xffffffffu, mbar_wait(&S.empty, 1, A.wait_ns));
+            if (ok) scatter_tile((i - 1) & 1);
         }
         if (!ok) atomicExch(&S.abort, 1);
     } else {

@@ -203,6 +203,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity,
     }
 }
 
+// Has the phase with the given parity completed?
+__device__ __forceinline__ bool mbar_test(uint64_t *mbar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(smem_u32(mbar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
@@ -246,6 +259,34 @@ __device__ __forceinline__ void panel_store8(unsigned char *panel, int row, int 
     q.z = pack_bf16(v[4], v[5]);
     q.w = pack_bf16(v[6], v[7]);
     *reinterpret_cast<uint4 *>(panel + panel_offset(row, col)) = q;
+}
+
+// max(., 0) of two BF16 values (0 for a NaN, as fmaxf gives).
+__device__ __forceinline__ uint32_t relu_bf16(uint32_t h) {
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0u));
+    return r;
+}
+
+// 16-byte chunk of a panel: row, columns [col, col + 8).
+__device__ __forceinline__ uint4 *panel_chunk(unsigned char *panel, int row, int col) {
+    return reinterpret_cast<uint4 *>(panel + panel_offset(row, col));
+}
+
+// Eight values as BF16: max(v, 0); and v where h, a chunk of such values, is above 0, 0 elsewhere.
+__device__ __forceinline__ uint4 pack8_relu(const float *v) {
+    return make_uint4(relu_bf16(pack_bf16(v[0], v[1])), relu_bf16(pack_bf16(v[2], v[3])),
+                      relu_bf16(pack_bf16(v[4], v[5])), relu_bf16(pack_bf16(v[6], v[7])));
+}
+__device__ __forceinline__ uint4 pack8_where(const uint4 &h, const float *v) {
+    // h holds no negative values: adding 0x7fff sets the top bit of every half that is not 0, and the byte
+    // permutation spreads it over the half
+    auto where = [](uint32_t hw, float a, float b) {
+        uint32_t m;
+        asm("prmt.b32 %0, %1, 0, 0xbb99;" : "=r"(m) : "r"(hw + 0x7fff7fffu));
+        return pack_bf16(a, b) & m;
+    };
+    return make_uint4(where(h.x, v[0], v[1]), where(h.y, v[2], v[3]), where(h.z, v[4], v[5]), where(h.w, v[6], v[7]));
 }
 
 // Eight FP32 values as three BF16 chunks of 16 bytes: hi, mid, lo.
