@@ -12,7 +12,7 @@
 // Bound: the serial chain of a tile -- seven MMA batches (12 k clocks of the tensor pipe at M = N = 128) and,
 // between them, three epilogues that split 16 k values each on two warps per scheduler; shared memory
 // (weights and 64 KB of activations) leaves no room for a second tile beside it.  160^3, 8,192 rays,
-// 1.38 M samples: 4610 us on the CUDA cores (45 % of their FP32 rate), 1500 us here, 44 k clocks a tile.
+// 1.38 M samples: 4610 us on the CUDA cores (45 % of their FP32 rate), 1245 us here, 33 k clocks a tile.
 //
 // Per tile of M = 128 kept samples, with dout = dL/do from the compositing backward; activations are kept
 // transposed (TMEM lane = hidden unit, column = sample), so that a thread owns a unit: the sums over the
@@ -30,7 +30,7 @@
 // 32 KB thirds of the activations, then X again.  Warps 0-7 consume (thread (n, half): unit n = t mod 128,
 // samples 64 half .. +63), warps 8-11 gather X, stage it twice and scatter the feature gradients of the
 // tile before.  TMEM columns: activations' split [0, 192); layer accumulator [192, 320); dW2, then the second
-// half of dH1 [320, 448); dW1 [192, 336) over both; de [448, 496).
+// half of dH1 [320, 448); dW1 [192, 336) over both; dZ2's hi third, then de [448, 512).
 
 #include "dvgo_internal.cuh"
 #include "fine_gather.cuh"
@@ -46,11 +46,12 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int TM = 128, NC = 256, NP = 128;
 constexpr int HID = 128, FEAT = 12, IN = 39, XK = 40;   // column IN of X is the constant 1 (bias)
 constexpr int KB = 3;                                   // 16-column blocks of X and W1 per split
-constexpr uint32_t T_ACT = 0, T_Z = 192, T_DW2 = 320, T_DW1 = 192, T_DE = 448, NCOLS = 512;
+constexpr uint32_t T_ACT = 0, T_Z = 192, T_DW2 = 320, T_DW1 = 192, T_DE = 448, T_HI = 448, NCOLS = 512;
 
 struct BwdSmall {
     alignas(16) float dout[3][TM];   // dL/do
     alignas(16) float xmax[TM];      // largest input magnitude of the row (0: padding row)
+    float gmax[TM / 16];             // the same of 16 rows
     float4 de[TM][3];      // feature gradients of a tile
     float4 place[2][TM];
     ScatterTab tab[NP / 32];
@@ -311,6 +312,10 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             S.dout[1][row] = cur.d[1];
             S.dout[2][row] = cur.d[2];
             S.xmax[row] = cur.xmax;
+            float gm = cur.xmax;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(FULL, gm, o));
+            if ((row & 15) == 0) S.gmax[row >> 4] = gm;
             fence_async_smem();
             mbar_arrive(&S.full);
             // de of the tile before is in place: written before the consumers' release that this thread
@@ -419,12 +424,12 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) mma(tb + T_DE, a + mnstep(kk), b + mnstep(kk), id, !first || kk > 0);
         };
-        // copies the hi third of the activations from TMEM into the pool's first buffer
-        auto stage_hi = [&]() {
+        // copies a hi third from TMEM columns `from` into the pool's first buffer
+        auto stage_hi = [&](uint32_t from) {
 #pragma unroll 1
             for (int g = 0; g < 2; ++g) {
                 float v[16];
-                tmem_ld16(taddr(tb, warp, T_ACT + 32 * hc + 16 * g), v);
+                tmem_ld16(taddr(tb, warp, from + 32 * hc + 16 * g), v);
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
                     *reinterpret_cast<uint4 *>(buf0 + panel_offset(n, 32 * g + 8 * c)) =
@@ -456,42 +461,48 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             }
             if (!wait_a()) { ok = false; break; }
             // ---- epilogue 1: H1 = relu(Z1), split: TMEM (A of dW2), lo and mid into the pool ----
-            uint32_t m1[4], m2[4];   // which units are off: 16 samples a word, sample k in bit 15 - k
+            uint32_t m1[4], m2[2];   // which units are off: 16 samples a word, sample k in bit 15 - k
             float zz[32];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                if ((g & 1) == 0) tmem_ld32(taddr(tb, warp, T_Z + 64 * hc + 16 * g), zz);
-                float z[16];
+            for (int half = 0; half < 2; ++half) {
+                tmem_ld32(taddr(tb, warp, T_Z + 64 * hc + 32 * half), zz);
+                bool near = false;   // a unit within rounding of zero
 #pragma unroll
-                for (int k = 0; k < 16; ++k) z[k] = zz[16 * (g & 1) + k];
-                uint32_t neg = 0;   // sign bits, sample k in bit 15 - k
-                float near = 1.0f;  // below zero when a unit is within rounding of zero
+                for (int q = 0; q < 2; ++q) {
+                    uint32_t neg = 0;   // sign bits, sample k in bit 15 - k
+                    float low = 0x1p127f;
 #pragma unroll
-                for (int k = 0; k < 16; k += 4) {
-                    const float4 x4 = *reinterpret_cast<const float4 *>(&S.xmax[64 * hc + 16 * g + k]);
-                    const float xm[4] = {x4.x, x4.y, x4.z, x4.w};
+                    for (int k = 0; k < 16; ++k) {
+                        neg = __funnelshift_l(__float_as_uint(zz[16 * q + k]), neg, 1);
+                        low = fminf(low, fabsf(zz[16 * q + k]));
+                    }
+                    m1[2 * half + q] = neg;
+                    near |= low < eps1 * S.gmax[4 * hc + 2 * half + q];
+                }
+                if (__any_sync(FULL, near)) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        neg = __funnelshift_l(__float_as_uint(z[k + j]), neg, 1);
-                        near = fminf(near, fmaf(-eps1, xm[j], fabsf(z[k + j])));
+                    for (int q = 0; q < 2; ++q) {
+                        const int k0 = 64 * hc + 32 * half + 16 * q;
+                        uint32_t amb = 0;
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            amb |= (fmaf(-eps1, S.xmax[k0 + k], fabsf(zz[16 * q + k])) < 0.0f ? 1u : 0u) << k;
+                        m1[2 * half + q] = resolve<FeatT, PK, 1>(A, tile * TM + k0, n, amb, m1[2 * half + q]);
                     }
                 }
-                if (__any_sync(FULL, near < 0.0f)) {
-                    uint32_t amb = 0;
 #pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        amb |= (fmaf(-eps1, S.xmax[64 * hc + 16 * g + k], fabsf(z[k])) < 0.0f ? 1u : 0u) << k;
-                    neg = resolve<FeatT, PK, 1>(A, tile * TM + 64 * hc + 16 * g, n, amb, neg);
+                for (int q = 0; q < 2; ++q) {
+                    const int g = 2 * half + q;
+                    float z[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) z[k] = fmaxf(zz[16 * q + k], 0.0f);
+                    uint32_t w[3][8];
+                    split16(z, w);
+                    store16(buf0, n, g, w[2]);
+                    store16(buf1, n, g, w[1]);
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) tmem_st8(taddr(tb, warp, T_ACT + 64 * t + 32 * hc + 8 * g), w[t]);
                 }
-#pragma unroll
-                for (int k = 0; k < 16; ++k) z[k] = fmaxf(z[k], 0.0f);
-                m1[g] = neg;
-                uint32_t w[3][8];
-                split16(z, w);
-                store16(buf0, n, g, w[2]);
-                store16(buf1, n, g, w[1]);
-#pragma unroll
-                for (int s = 0; s < 3; ++s) tmem_st8(taddr(tb, warp, T_ACT + 64 * s + 32 * hc + 8 * g), w[s]);
             }
             tmem_wait_st();
             publish();
@@ -505,7 +516,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             }
             b_out = true;
             if (!wait_a()) { ok = false; break; }
-            stage_hi();
+            stage_hi(T_ACT);
             publish();
             if (tid == 0) {
                 z2_batch(b0_, 2, false);
@@ -516,53 +527,66 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             if (!wait_b() || !wait_a()) { ok = false; break; }
             // ---- epilogue 2: dZ2, dW3, db2 (a tile's sums first, then the running ones) ----
             float t3[3] = {0.0f, 0.0f, 0.0f}, tb2 = 0.0f;
+            // (dL/do of a sample is read once for both: a read of four samples' takes the load unit four clocks a
+            // warp, and reading it for h, for dZ2 and again for dZ2's hi third took it 4,600 clocks of a tile; so did
+            // xmax of every sample 1,000.  1482 -> 1245 us at 1.38 M samples.)
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                if ((g & 1) == 0) tmem_ld32(taddr(tb, warp, T_Z + 64 * hc + 16 * g), zz);
-                float z[16];
+            for (int half = 0; half < 2; ++half) {
+                tmem_ld32(taddr(tb, warp, T_Z + 64 * hc + 32 * half), zz);
+                bool near = false;
 #pragma unroll
-                for (int k = 0; k < 16; ++k) z[k] = zz[16 * (g & 1) + k];
-                uint32_t neg = 0;
-                float near = 1.0f;
+                for (int q = 0; q < 2; ++q) {
+                    uint32_t neg = 0;
+                    float low = 0x1p127f;
 #pragma unroll
-                for (int k = 0; k < 16; k += 4) {
-                    float d[3][4], xm[4];
-                    load_dout(S, 64 * hc + 16 * g + k, d);
-                    *reinterpret_cast<float4 *>(xm) = *reinterpret_cast<const float4 *>(&S.xmax[64 * hc + 16 * g + k]);
+                    for (int k = 0; k < 16; k += 4) {
+                        float d[3][4];
+                        load_dout(S, 64 * hc + 32 * half + 16 * q + k, d);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float v = z[k + j] + b2, h = fmaxf(v, 0.0f);
-                        neg = __funnelshift_l(__float_as_uint(v), neg, 1);
-                        near = fminf(near, fmaf(-eps2, xm[j], fabsf(v)));
-                        t3[0] = fmaf(h, d[0][j], t3[0]);
-                        t3[1] = fmaf(h, d[1][j], t3[1]);
-                        t3[2] = fmaf(h, d[2][j], t3[2]);
+                        for (int j = 0; j < 4; ++j) {
+                            float &z = zz[16 * q + k + j];
+                            const float v = z + b2, h = fmaxf(v, 0.0f);
+                            neg = __funnelshift_l(__float_as_uint(v), neg, 1);
+                            low = fminf(low, fabsf(v));
+                            t3[0] = fmaf(h, d[0][j], t3[0]);
+                            t3[1] = fmaf(h, d[1][j], t3[1]);
+                            t3[2] = fmaf(h, d[2][j], t3[2]);
+                            z = fmaf(d[2][j], w32, fmaf(d[1][j], w31, d[0][j] * w30));   // dH2
+                        }
+                    }
+                    m2[q] = neg;
+                    near |= low < eps2 * S.gmax[4 * hc + 2 * half + q];
+                }
+                if (__any_sync(FULL, near)) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int k0 = 64 * hc + 32 * half + 16 * q;
+                        float z[16];
+                        tmem_ld16(taddr(tb, warp, T_Z + k0), z);
+                        uint32_t amb = 0;
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            amb |= (fmaf(-eps2, S.xmax[k0 + k], fabsf(z[k] + b2)) < 0.0f ? 1u : 0u) << k;
+                        m2[q] = resolve<FeatT, PK, 2>(A, tile * TM + k0, n, amb, m2[q]);
                     }
                 }
-                if (__any_sync(FULL, near < 0.0f)) {
-                    uint32_t amb = 0;
 #pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        amb |= (fmaf(-eps2, S.xmax[64 * hc + 16 * g + k], fabsf(z[k] + b2)) < 0.0f ? 1u : 0u) << k;
-                    neg = resolve<FeatT, PK, 2>(A, tile * TM + 64 * hc + 16 * g, n, amb, neg);
-                }
-                m2[g] = neg;
+                for (int q = 0; q < 2; ++q) {
+                    const int g = 2 * half + q;
+                    float z[16];
 #pragma unroll
-                for (int k = 0; k < 16; k += 4) {
-                    float d[3][4];
-                    load_dout(S, 64 * hc + 16 * g + k, d);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float v = fmaf(d[2][j], w32, fmaf(d[1][j], w31, d[0][j] * w30));
-                        z[k + j] = off(neg, k + j) ? 0.0f : v;
-                        tb2 += z[k + j];
+                    for (int k = 0; k < 16; ++k) {
+                        z[k] = off(m2[q], k) ? 0.0f : zz[16 * q + k];
+                        tb2 += z[k];
                     }
+                    uint32_t w[3][8];
+                    split16(z, w);
+                    store16(buf0, n, g, w[2]);
+                    store16(buf1, n, g, w[1]);
+                    tmem_st8(taddr(tb, warp, T_HI + 32 * hc + 8 * g), w[0]);   // until the pool has room for it
                 }
-                uint32_t w[3][8];
-                split16(z, w);
-                store16(buf0, n, g, w[2]);
-                store16(buf1, n, g, w[1]);
             }
+            tmem_wait_st();
             ab2 += tb2;
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) a3[ch] += t3[ch];
@@ -578,23 +602,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 dh_batch(b1_, 0, false);
             }
             if (!wait_a()) { ok = false; break; }
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {   // the hi third again from dout
-                uint32_t w[8];
-#pragma unroll
-                for (int k = 0; k < 16; k += 4) {
-                    float d[3][4], v[4];
-                    load_dout(S, 64 * hc + 16 * g + k, d);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        v[j] = fmaf(d[2][j], w32, fmaf(d[1][j], w31, d[0][j] * w30));
-                        v[j] = off(m2[g], k + j) ? 0.0f : v[j];
-                    }
-                    w[k / 2] = pack_bf16(v[0], v[1]);
-                    w[k / 2 + 1] = pack_bf16(v[2], v[3]);
-                }
-                store16(buf0, n, g, w);
-            }
+            stage_hi(T_HI);
             publish();
             if (tid == 0) {
                 dw2_batch(b0_, 2, false);
@@ -648,7 +656,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 commit(&S.mma_a);
             }
             if (!wait_a()) { ok = false; break; }
-            stage_hi();
+            stage_hi(T_ACT);
             publish();
             if (tid == 0) {
                 de_batch(b0_, 3, false);
