@@ -143,9 +143,9 @@ __device__ __forceinline__ bool cells_adjacent(int cb, int cbn, int ny, int nz, 
     return abs(dz) <= 1;
 }
 
-// A warp's table of 16 rows: by corner parity (x, y, z), the weight and the grid index of the corner.  (The
+// A warp's table of 8 rows: by corner parity (x, y, z), the weight and the grid index of the corner.  (The
 // ninth column keeps the rows' writes off each other's banks.)
-constexpr int kScatterRows = 16;
+constexpr int kScatterRows = 8;
 struct ScatterTab {
     float2 at[kScatterRows][9];
 };
@@ -201,18 +201,17 @@ __device__ __forceinline__ void scatter_rows(const RenderArgs &A, const float4 *
     for (int j0 = 0; j0 < n; j0 += kScatterRows) {
         __syncwarp();
         {
-            // two lanes a row, one for each z parity
-            const int j = j0 + (lane & 15);
+            // four lanes a row, one for each pair of (y, z) parities
+            const int j = j0 + (lane & 7), by = ((lane >> 4) ^ (odd_y >> j)) & 1, bz = ((lane >> 3) ^ (odd_z >> j)) & 1;
             const float4 f = place[r0 + j];
-            const int cb = __float_as_int(f.w);
-            const int ix = (odd_x >> j) & 1, iy = (odd_y >> j) & 1, bz = (lane >> 4) ^ (int)((odd_z >> j) & 1);
-            const float wz = bz ? f.z : 1.0f - f.z;
+            const int cb = __float_as_int(f.w), ix = (odd_x >> j) & 1;
+            const float wy = by ? f.y : 1.0f - f.y, wz = bz ? f.z : 1.0f - f.z;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int bx = (q >> 1) ^ ix, by = (q & 1) ^ iy;
-                const float w = (bx ? f.x : 1.0f - f.x) * (by ? f.y : 1.0f - f.y) * wz;
+            for (int q = 0; q < 2; ++q) {
+                const int bx = q ^ ix;
+                const float w = (bx ? f.x : 1.0f - f.x) * wy * wz;
                 const unsigned idx = (unsigned)corner_from_base(cb, bx, by, bz, A.ny, A.nz, PK);
-                tab.at[lane & 15][2 * q + (lane >> 4)] = make_float2(w, __uint_as_float(idx));
+                tab.at[lane & 7][4 * q + (lane >> 3)] = make_float2(w, __uint_as_float(idx));
             }
         }
         __syncwarp();

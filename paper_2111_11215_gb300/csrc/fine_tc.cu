@@ -8,7 +8,7 @@
 // issued by one thread, completion signalled through mbarriers.  The 128 -> 3 output layer, the
 // sigmoid and the element-wise steps run on the CUDA cores in the epilogues.
 //
-// Persistent CTAs walk tiles of M = 128 kept samples.  Warps 8-11 (producers; 8-15 in the forward)
+// Persistent CTAs walk tiles of M = 128 kept samples.  Warps 8-15 (producers, two sets)
 // gather the next tile -- features at the 8 lattice corners, the ray's direction encoding, the
 // bias column -- into one of two X panels, and in the backward also scatter the feature gradients
 // of the tile that last used that panel.  The forward stores every finished X panel (16 KiB, as
@@ -21,13 +21,13 @@
 //
 // The backward is a chain of MMA batches and epilogues.  Waiting for each batch as a whole, with one
 // thread of an epilogue issuing it, a tile took 11,700 clocks, of which the MMAs are 3,500.  So a warp of
-// its own (warp 12) issues them: what the next epilogue waits for first, the weight gradients behind it, and
+// its own (warp 16) issues them: what the next epilogue waits for first, the weight gradients behind it, and
 // the next tile's layer 1 before this tile's last batch; dZ1 goes over H2, not H1, so that its epilogue
 // need not wait for dW2, and the next tile's first epilogue runs during dW1.  The consumers hold no barrier
 // among themselves: a warp waits for MMA batches only and signals the issuing warp.  65,536 rays at 256^3
-// (284,928 tiles): 11.55 -> 7.33 ms, the scatter's new form (fine_gather.cuh) included; 310,320 samples: 121 -> 84 us.
-// What bounds it now: the producers (7,400 clocks a tile, 4,800 of them the scatter), the consumers' chain
-// close behind.
+// (284,928 tiles): 11.55 -> 7.33 ms, the scatter's new form (fine_gather.cuh) included, 6.87 ms with two producer
+// sets (the scatter was 4,800 of a producer's 7,400 clocks a tile); 310,320 samples: 121 -> 84 -> 77 us.  What
+// bounds it now: the consumers' chain of three epilogues and three MMA batches, 7,000 clocks a tile.
 //
 // Inputs beyond the 64 columns of the X panel (PE(x) entries 24-32 of the 72-input row) live in a
 // "tail panel" that also holds W3: columns 0-15 W3 (3 used), 16-31 / 32-47 the tail of X buffer 0 /
@@ -65,16 +65,12 @@ using namespace tc;
 constexpr int TM = 128;
 constexpr int NC = 256;        // consumer threads: warp w owns TMEM lanes 32 (w % 4).., columns 64 (w / 4)..
 constexpr int NP = 128;        // producer threads of one set (one sample row each)
-// producer sets: the backward has one (its consumers are the bound); the forward two, set p filling
-// X buffer p for consumer group p, so that two tiles are gathered at once
-#ifndef DVGO_FWD_PROD_SETS
-#define DVGO_FWD_PROD_SETS 2
-#endif
-template <bool BWD>
-constexpr int kProdSets = BWD ? 1 : DVGO_FWD_PROD_SETS;
+// producer sets: set p fills X buffer p with every other tile, so that two tiles are gathered (in the backward
+// also scattered) at once
+constexpr int kProdSets = 2;
 // the backward has one more warp, which issues the MMAs
 template <bool BWD>
-constexpr int kThreads = NC + NP * kProdSets<BWD> + (BWD ? 32 : 0);   // 416 / 512
+constexpr int kThreads = NC + NP * kProdSets + (BWD ? 32 : 0);   // 544 / 512
 constexpr int HID = 128;
 constexpr int FEAT = 12;
 constexpr int NF = 4;
@@ -107,14 +103,14 @@ struct alignas(1024) SmallTC {
         int slot[4][TM];
         float4 place[4][TM];
     };
-    ScatterTab tab[NP / 32];  // backward
+    ScatterTab tab[kProdSets * NP / 32];   // backward
     float dc[2][TM][3];       // dL/dc (backward)
     uint64_t full[2], empty[2];
     uint64_t mma[2];          // forward: the MMAs of consumer group 0 / 1
     // backward.  xl: the bulk load of X panel b from the forward's copy; z1, z2, dh, de: MMA batches
-    // complete; ev[e]: consumers have finished epilogue e; fin: every MMA of the launch complete; drained:
-    // the producers have scattered all tiles but the last two
-    uint64_t xl[2], z1, z2, dh, de, ev[4], fin, drained;
+    // complete; ev[e]: consumers have finished epilogue e; fin: every MMA of the launch complete; sc: the
+    // de of a tile of X buffer b has been scattered
+    uint64_t xl[2], z1, z2, dh, de, ev[4], fin, sc[2];
     uint32_t tmem_base;
     int abort;
 };
@@ -238,7 +234,8 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             mbar_init(&S.sm.de, 1);
             for (int e = 0; e < 4; ++e) mbar_init(&S.sm.ev[e], NC / 32);
             mbar_init(&S.sm.fin, 1);
-            mbar_init(&S.sm.drained, NP);
+            mbar_init(&S.sm.sc[0], NP);
+            mbar_init(&S.sm.sc[1], NP);
         }
         S.sm.abort = 0;
     }
@@ -283,7 +280,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         if (tid < 3) S.sm.b3[tid] = A.b3[tid];
         if (tid < 4) S.sm.db3[tid] = 0.0f;
     }
-    if (tid < NC || tid >= NC + NP * kProdSets<BWD>) {   // weights staged: all that issue MMAs may use them
+    if (tid < NC || tid >= NC + NP * kProdSets) {   // weights staged: all that issue MMAs may use them
         fence_async_smem();
         fence_before();
         asm volatile("bar.sync 1, %0;" ::"n"(NC + (BWD ? 32 : 0)) : "memory");
@@ -298,13 +295,13 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
     bool ok = true;
     int ntile_mine = 0;
 
-    if (tid >= NC && tid < NC + NP * kProdSets<BWD>) {
+    if (tid >= NC && tid < NC + NP * kProdSets) {
         // ------------------------------- producers -------------------------------
         // Set pset takes the CTA's tiles i = pset, pset + nsets, ... (X buffer i & 1).  Software-
         // pipelined a tile deep: while producing a tile, a producer already has its set's next tile's
         // kept entry and fetches that tile's ray data and the kept entry of the tile after, so that
         // only the corner-feature loads of a tile wait on memory when it is produced.
-        constexpr int nsets = kProdSets<BWD>;
+        constexpr int nsets = kProdSets;
         const int row = (tid - NC) & (NP - 1), pset = (tid - NC) / NP;
         const int stride = nsets * (int)gridDim.x;
         auto kept_at = [&](int t) -> int2 {
@@ -313,7 +310,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         };
         auto scatter_tile = [&](int j) {   // the CTA's tile j
             scatter_rows<PK>(A, S.sm.place[j & 3], [&](int r, int k) { return de_slot(S.dout, j & 1, r, k); },
-                             S.sm.tab[row >> 5], row);
+                             S.sm.tab[warp - NC / 32], row);
         };
         auto dldo_at = [&](const int2 &kv, const RayPre &rp) -> float4 {
             return (BWD && kv.y >= 0) ? A.sgrad[rp.off + (kv.x & 0xffff)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -344,16 +341,18 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             fence_async_smem();
             // (testing aid: one arrival withheld on a chosen tile makes the consumers' wait run out)
             if (!(row == 0 && tile + 1 == A.withhold_tile)) mbar_arrive(&S.sm.full[b]);
-            if (BWD && i >= 2) scatter_tile(i - 2);   // its de stays until tile i + 1 is full
+            if (BWD && i >= 2) {
+                scatter_tile(i - 2);
+                mbar_arrive(&S.sm.sc[b]);
+            }
             gc_cur = dldo_at(kv_next, rp_next);
             kv_cur = kv_next;
             rp_cur = rp_next;
             kv_next = kv_after;
         }
-        if (BWD) mbar_arrive(&S.sm.drained);
         if (BWD && ok) {
-            // the last (up to) two tiles: wait until the consumers are done with them, then scatter
-            for (int j = (i >= 2 ? i - 2 : 0); j < i && ok; ++j) {
+            // the last tile: wait until the consumers are done with it, then scatter
+            for (int j = i - nsets; j >= 0 && j < i && ok; j += nsets) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&S.sm.empty[j & 1], (j >> 1) & 1, A.wait_ns));
                 if (ok && !__any_sync(0xffffffffu, *(volatile int *)&S.sm.abort != 0)) scatter_tile(j);
             }
@@ -473,7 +472,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         }
         if (r == 0 && A.xcache) bulk_wait_all();   // the copies are complete before the kernel ends
         if (!ok) atomicExch(&S.sm.abort, 1);
-    } else if (warp == NC / 32 + NP / 32) {
+    } else if (warp == (NC + NP * kProdSets) / 32) {
         // ------------------------------- MMA issue (backward) -------------------------------
         // One thread issues a tile's batches as their operands become ready, and the next tile's layer 1 as
         // soon as its X panel is there, so that it is complete when the consumers come to it:
@@ -594,8 +593,10 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             __syncwarp();
             if ((tid & 31) == 0) mbar_arrive(bar);
         };
-        // de[0:12] of tile j for the producers' scatter; X[j & 1] and de's slot are theirs again
-        auto stage_de = [&](int j) {
+        // de[0:12] of tile j for the producers' scatter, when the tile that had the slot is scattered; X[j & 1] is
+        // the producers' again
+        auto stage_de = [&](int j) -> bool {
+            if (!wait(&S.sm.de, j & 1) || (j >= 2 && !wait(&S.sm.sc[j & 1], ((j >> 1) - 1) & 1))) return false;
             float de[16];
             tmem_ld16(taddr(tb, warp, COL_DE), de);
             *de_slot(S.dout, j & 1, r, 0) = make_float4(de[0], de[1], de[2], de[3]);
@@ -604,6 +605,7 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             fence_before();
             __syncwarp();
             if ((tid & 31) == 0) mbar_arrive(&S.sm.empty[j & 1]);
+            return true;
         };
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
             const int b = i & 1;
@@ -635,12 +637,8 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
                 *reinterpret_cast<uint2 *>(S.dout + panel_offset(r, 0)) = q;
             }
             signal(&S.sm.ev[0]);
-            // ---- the tile before: its de, while layer 2 runs (the scatter of the tile three back, which
-            //      had this slot, was done when this tile was full) ----
-            if (i > 0 && hc == 1) {
-                if (!wait(&S.sm.de, par ^ 1)) break;
-                stage_de(i - 1);
-            }
+            // ---- the tile before: its de, while layer 2 runs ----
+            if (i > 0 && hc == 1 && !stage_de(i - 1)) break;
             // ---- epilogue 2: H2 = relu(Z2 + b2), then dZ2 = dH2 [Z2 + b2 > 0], my 64 columns ----
             if (!wait(&S.sm.z2, par)) break;
             uint4 hw[8];   // my row of H2, then of H1, for the ReLU's derivative
@@ -683,8 +681,10 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             masked(COL_Z2, S.h2);
             signal(&S.sm.ev[3]);
         }
-        // the last tile's de, once the scatter that had its slot is done
-        if (ok && i > 0 && wait(&S.sm.de, (i - 1) & 1) && hc == 1 && wait(&S.sm.drained, 0)) stage_de(i - 1);
+        if (ok && i > 0) {   // the last tile's de; all wait for the last MMAs
+            if (hc == 1) stage_de(i - 1);
+            else wait(&S.sm.de, (i - 1) & 1);
+        }
         ntile_mine = i;
         if (!ok) atomicExch(&S.sm.abort, 1);
 #pragma unroll
