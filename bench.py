@@ -8,7 +8,7 @@ rays drawn from 100 inward-facing 800x800 views (radius 4, focal 1111).  One ste
 + MSE + backward + Adam on every parameter (density, features, MLP).
 
 Forms (both are timed by default; `value` is the chosen form):
-  plain  = uniform 0.5-voxel steps, FP32 feature grid, FP32 SIMT MLP;
+  plain  = uniform 0.5-voxel steps, FP32 feature grid, FP32 MLP;
   chosen = learned proposal (64-bin PDF from a BF16 tensor-core proposal MLP trained by its BF16
            tensor-core backward; 48 inverse-CDF samples per ray from the PDF mixed 0.05 with the
            uniform one; every 4th step is a full uniform step whose forward also labels 1024 rays
@@ -355,7 +355,7 @@ def measure_form(name, args, dev, dens, feat, mlp, batches, dvgo, torch, world, 
     n_prop_train = (form.trainer.n_uniform - n_prop_train0) if form.trainer is not None else 0
     # chosen form: the same number of steps again, each waiting for the previous step's feature-grid
     # Adam before it starts, so that nothing runs beside any kernel: each kernel's own time (the
-    # sampling, ray set-up, scan and density pass otherwise share the GPU with that Adam)
+    # sampling, ray set-up and density pass otherwise share the GPU with that Adam)
     per_kind_alone = None
     if form.trainer is not None:
         dvgo.dvgo_profile_enable(True)
@@ -971,7 +971,7 @@ def run_trace(args):
             "data": "synthetic", "config": workload_config(args, "chosen"),
             "launches": [[k, round(a, 4), round(b, 4)] for k, a, b in tr],
             "note": "the feature-grid Adam (kind adam, ~0.25 ms) runs on a side stream beside the next step's "
-                    "sampling, ray set-up, scan and density pass; every other launch is on the main stream"}
+                    "sampling, ray set-up and density pass; every other launch is on the main stream"}
     print(json.dumps(line), flush=True)
 
 

@@ -169,8 +169,8 @@ typedef struct {
     int n_freq_pos;      /* fine: positional-encoding frequencies on the query point x (Sec. 4.2
                             Eq. fine_queries_rgb, Supp. A: k_x = 5); 0 leaves x out of the MLP
                             input.  This build supports 0 and 5.                                 */
-    /* Failure detection of the tensor-core colour kernels (DVGO_MLP_BF16, and the forward of DVGO_MLP_FP32;
-     * not part of the method).
+    /* Failure detection of the tensor-core colour kernels (DVGO_MLP_BF16; of DVGO_MLP_FP32 the forward and the
+     * backward of 39 inputs; not part of the method).
      * Every device-side wait of those kernels (an mbarrier phase: the producers' tile, the
      * consumers' release of a buffer, the completion of an MMA batch) gives up after
      * wait_limit_us microseconds (0: the default, 2 s); the kernel then stops its CTA's work, waits
@@ -185,7 +185,7 @@ typedef struct {
     /* cgrid_ready: NULL, or a cudaEvent_t (of the calling device) that dvgo_render_fwd and
      * dvgo_render_bwd make their stream wait on right before their first kernel that reads the
      * colour / feature grid -- for a producer of that grid on another stream (an optimiser step):
-     * the ray set-up, the sample scan and the density pass before it are not held back.  Not
+     * the ray set-up and the density pass before it are not held back.  Not
      * validated; an event that was never recorded is complete.  Other calls ignore it. */
     void *cgrid_ready;
     /* forward_only: non-zero when no dvgo_render_bwd follows the forward (test-time rendering).
@@ -195,8 +195,8 @@ typedef struct {
     int forward_only;
     /* density_ready: NULL, or a cudaEvent_t (of the calling device) that dvgo_render_fwd and
      * dvgo_render_bwd make their stream wait on right before their first kernel that reads the
-     * density grid -- for a producer of that grid on another stream: the ray set-up and the sample
-     * scan before it are not held back.  Not validated; an event that was never recorded is
+     * density grid -- for a producer of that grid on another stream: the ray set-up before it
+     * is not held back.  Not validated; an event that was never recorded is
      * complete.  Other calls ignore it. */
     void *density_ready;
 } dvgo_params;
@@ -436,7 +436,7 @@ typedef struct {
     int n_bins;          /* bins per ray; this build supports 64                                 */
     int n_freq;          /* PE frequencies on the bin centre x_b; this build supports 6            */
     int width;           /* MLP width; this build supports 64                                     */
-    int precision;       /* arithmetic of the forward and the backward: DVGO_MLP_FP32 (SIMT) or
+    int precision;       /* arithmetic of the forward and the backward: DVGO_MLP_FP32 (CUDA cores) or
                             DVGO_MLP_BF16 (tcgen05 tensor cores: BF16 operands -- inputs,
                             activations, weights, dlogit and the dZ of each layer -- with FP32
                             accumulation; the encoding and the softmax in FP32)                   */

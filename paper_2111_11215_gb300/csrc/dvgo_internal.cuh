@@ -456,12 +456,10 @@ void launch_coarse_fwd(const RenderArgs &A, cudaStream_t s);
 void launch_coarse_bwd(const RenderArgs &A, cudaStream_t s);
 void launch_empty_cells(const RenderArgs &A, cudaStream_t s);
 void launch_fine_density(const RenderArgs &A, cudaStream_t s);
-void launch_fine_colour_fwd(const RenderArgs &A, cudaStream_t s);
 void launch_fine_composite_fwd(const RenderArgs &A, cudaStream_t s);
 void launch_fine_composite_bwd(const RenderArgs &A, cudaStream_t s);
 void launch_fine_colour_bwd_simt(const RenderArgs &A, cudaStream_t s);
 void launch_fine_colour_bwd_fp32(const RenderArgs &A, cudaStream_t s);
-void launch_fine_colour_bwd(const RenderArgs &A, cudaStream_t s);
 void launch_adam(float *param, float *grad, float *m, float *v, size_t n, const dvgo_adam_hparams &h,
                  const float *lr_scale, uint16_t *bf16_out, int zero_grad, cudaStream_t s);
 void launch_adam_multi(const dvgo_adam_tensor *t, int nt, cudaStream_t s);

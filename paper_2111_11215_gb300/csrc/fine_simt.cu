@@ -1,12 +1,11 @@
-// fine_simt.cu -- backward of the fine stage's colour queries with the FP32 (SIMT) shallow MLP (the
-// forward is fine_tc_fp32.cu).
+// fine_simt.cu -- backward of the fine stage's colour queries with the FP32 shallow MLP of 72 inputs, on the
+// CUDA cores (39 inputs: fine_tc_fp32_bwd.cu; the forward of both: fine_tc_fp32.cu).
 //
-// Sec. 4.2 Eq. fine_queries_rgb and Supp. A: c = MLP(interp(x, V_feat), PE(d)[, PE(x)]) with D = 12
-// feature channels, k_d = 4 direction frequencies, optionally k_x = 5 frequencies on the query
-// point, two hidden layers of 128 and ReLU, sigmoid output.  Input row e = [feat (12), d (3),
-// sin(2^k d_c) (12, c-major), cos(2^k d_c) (12)] (39 inputs), with PE(x) [x (3), sin(2^k x_c)
-// (15), cos(2^k x_c) (15)] appended (72 inputs), and a constant 1 in the next column that carries
-// the first-layer bias (W1 row IN = b1).
+// Sec. 4.2 Eq. fine_queries_rgb and Supp. A: c = MLP(interp(x, V_feat), PE(d), PE(x)) with D = 12
+// feature channels, k_d = 4 direction frequencies, k_x = 5 frequencies on the query point, two hidden
+// layers of 128 and ReLU, sigmoid output.  Input row e = [feat (12), d (3), sin(2^k d_c) (12, c-major),
+// cos(2^k d_c) (12), x (3), sin(2^k x_c) (15), cos(2^k x_c) (15)] and a constant 1 in the next column
+// that carries the first-layer bias (W1 row IN = b1).
 //
 // Persistent CTAs (one per SM, 256 threads) walk tiles of 64 kept samples from the compact
 // list.  Weights stay in shared memory for the whole launch.  Activations are stored
@@ -38,18 +37,16 @@ constexpr int LDA = TM + 4;             // 68: activation row stride
 constexpr int LDW = HID + 4;            // 132: weight row stride
 constexpr int PX = FEAT + 3 + 6 * NF;   // 39: first input of the PE(x) block
 
-// Input widths: 39 (features + PE(d)) or 72 (+ PE(x)); K1 adds the bias column; the backward
-// splits the K1 (padded to 2 KH) rows of dW1|b1 between two thread halves.
-template <bool PEX>
+// 72 inputs (features, PE(d), PE(x)); K1 adds the bias column; the K1 (padded to 2 KH) rows of dW1|b1 are
+// split between two thread halves.
 struct Dims {
-    static constexpr int IN = PX + (PEX ? 3 + 6 * NFX : 0);
+    static constexpr int IN = PX + 3 + 6 * NFX;
     static constexpr int K1 = IN + 1;
     static constexpr int KH = (K1 + 1) / 2;
 };
 
-template <bool PEX>
 struct Smem {
-    static constexpr int K1 = Dims<PEX>::K1, KP = 2 * Dims<PEX>::KH;
+    static constexpr int K1 = Dims::K1, KP = 2 * Dims::KH;
     float w1[K1 * LDW];
     float w2[HID * LDW];
     float b2[HID];
@@ -69,10 +66,9 @@ __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast
 __device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 
 // Load weights into shared memory (FP32 master weights, row-major [in][out]).
-template <bool PEX>
-__device__ void load_weights(Smem<PEX> &S, const RenderArgs &A) {
-    constexpr int IN = Dims<PEX>::IN, K1 = Dims<PEX>::K1;
-    for (int i = threadIdx.x; i < (Smem<PEX>::KP - K1) * LDA; i += NT) S.xt[K1 * LDA + i] = 0.0f;
+__device__ void load_weights(Smem &S, const RenderArgs &A) {
+    constexpr int IN = Dims::IN, K1 = Dims::K1;
+    for (int i = threadIdx.x; i < (Smem::KP - K1) * LDA; i += NT) S.xt[K1 * LDA + i] = 0.0f;
     for (int i = threadIdx.x; i < K1 * HID; i += NT) {
         int k = i / HID, j = i % HID;
         S.w1[k * LDW + j] = (k < IN) ? A.w1[k * HID + j] : A.b1[j];
@@ -85,9 +81,9 @@ __device__ void load_weights(Smem<PEX> &S, const RenderArgs &A) {
 
 // Gather the input rows of one tile: 4 threads per sample, thread q handles the corner pair
 // (x bit, y bit) = (q >> 1, q & 1) with z = 0, 1 (adjacent in memory).
-template <typename FeatT, bool PEX, bool PK>
-__device__ void gather_tile(Smem<PEX> &S, const RenderArgs &A, int tile, int n_kept) {
-    constexpr int IN = Dims<PEX>::IN;
+template <typename FeatT, bool PK>
+__device__ void gather_tile(Smem &S, const RenderArgs &A, int tile, int n_kept) {
+    constexpr int IN = Dims::IN;
     int tid = threadIdx.x;
     int i = tid >> 2, q = tid & 3;
     int e = tile * TM + i;
@@ -107,7 +103,7 @@ __device__ void gather_tile(Smem<PEX> &S, const RenderArgs &A, int tile, int n_k
         const int k = kv.x >> 16;
         float dt;
         Cell c = sample_cell(A, rr, ray, k, dt);
-        if (PEX && q > 0) {
+        if (q > 0) {
             float xv[3];
             cell_world(A, c, xv);
             xw = xv[q - 1];
@@ -179,7 +175,7 @@ __device__ void gather_tile(Smem<PEX> &S, const RenderArgs &A, int tile, int n_k
             S.xt[(FEAT + 3 + a * NF + k) * LDA + i] = s;
             S.xt[(FEAT + 3 + 3 * NF + a * NF + k) * LDA + i] = cs;
         }
-        if constexpr (PEX) {
+        {
             float sx[NFX], cx[NFX];
             pe_axis<NFX>(xw, sx, cx);
             S.xt[(PX + a) * LDA + i] = xw;
@@ -224,11 +220,11 @@ __device__ __forceinline__ void gemm_fwd(const float *InT, const float *W, const
     }
 }
 
-template <typename FeatT, bool PEX, bool PK>
+template <typename FeatT, bool PK>
 __global__ void __launch_bounds__(NT, 1) fine_colour_bwd_kernel(RenderArgs A) {
-    constexpr int IN = Dims<PEX>::IN, K1 = Dims<PEX>::K1, KH = Dims<PEX>::KH;
+    constexpr int IN = Dims::IN, K1 = Dims::K1, KH = Dims::KH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem<PEX> &S = *reinterpret_cast<Smem<PEX> *>(smem_raw);
+    Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     load_weights(S, A);
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
@@ -250,7 +246,7 @@ __global__ void __launch_bounds__(NT, 1) fine_colour_bwd_kernel(RenderArgs A) {
 
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         __syncthreads();
-        gather_tile<FeatT, PEX, PK>(S, A, tile, n_kept);
+        gather_tile<FeatT, PK>(S, A, tile, n_kept);
         __syncthreads();
         gemm_fwd<K1>(S.xt, S.w1, nullptr, S.h1);
         __syncthreads();
@@ -437,31 +433,20 @@ __global__ void __launch_bounds__(NT, 1) fine_colour_bwd_kernel(RenderArgs A) {
     if (tid < 3) atomicAdd(gB3 + tid, gb3);
 }
 
-template <bool PEX>
-void launch_persistent(void (*kernel)(RenderArgs), int kind, const RenderArgs &A, cudaStream_t s) {
-    ensure_smem(reinterpret_cast<const void *>(kernel), (int)sizeof(Smem<PEX>));
-    ProfScope ps_(kind, s);
-    kernel<<<num_sms(), NT, sizeof(Smem<PEX>), s>>>(A);
-}
-
-template <bool PEX, bool PK>
+template <bool PK>
 void launch_colour(const RenderArgs &A, cudaStream_t s) {
-    launch_persistent<PEX>(A.cdtype == DVGO_DTYPE_BF16 ? fine_colour_bwd_kernel<__nv_bfloat16, PEX, PK>
-                                                       : fine_colour_bwd_kernel<float, PEX, PK>,
-                           DVGO_K_FINE_COLOUR_BWD, A, s);
+    void (*kernel)(RenderArgs) = A.cdtype == DVGO_DTYPE_BF16 ? fine_colour_bwd_kernel<__nv_bfloat16, PK>
+                                                             : fine_colour_bwd_kernel<float, PK>;
+    ensure_smem(reinterpret_cast<const void *>(kernel), (int)sizeof(Smem));
+    ProfScope ps_(DVGO_K_FINE_COLOUR_BWD, s);
+    kernel<<<num_sms(), NT, sizeof(Smem), s>>>(A);
 }
 
 }  // namespace
 
 void launch_fine_colour_bwd_simt(const RenderArgs &A, cudaStream_t s) {
-    const bool pex = A.nfreq_pos > 0;
-    if (A.packed) {
-        if (pex) launch_colour<true, true>(A, s);
-        else launch_colour<false, true>(A, s);
-    } else {
-        if (pex) launch_colour<true, false>(A, s);
-        else launch_colour<false, false>(A, s);
-    }
+    if (A.packed) launch_colour<true>(A, s);
+    else launch_colour<false>(A, s);
 }
 
 }  // namespace dvgo

@@ -87,7 +87,7 @@ struct TcDims {
     static constexpr int NTAIL = IN - NMAIN;                  // 0 or 9
 };
 
-constexpr uint32_t COL_Z1 = 0, COL_O = 0, COL_Z2 = 128, COL_DW2T = 256, COL_DW1 = 400, COL_DW3 = 464,
+constexpr uint32_t COL_Z1 = 0, COL_Z2 = 128, COL_DW2T = 256, COL_DW1 = 400, COL_DW3 = 464,
                    COL_DE = 480, COL_DW1T = 496;
 
 // Small per-CTA state, padded to a multiple of 1024 bytes so that the panels after it stay

@@ -45,8 +45,8 @@ class Renderer:
     def forward(self, density, cgrid, mlp, rays_o, rays_d, jitter=None, samples=None, target=None,
                 rgb=None, tfinal=None, loss=None, dloss=None, stream=None, cgrid_ready=None, density_ready=None):
         """cgrid_ready: an event (torch.cuda.Event) whose completion the colour kernels wait for;
-        the kernels before them (ray set-up, sample scan, density pass) do not.  density_ready: the
-        same for the density pass (the ray set-up and the sample scan do not wait)."""
+        the kernels before them (ray set-up, density pass) do not.  density_ready: the
+        same for the density pass (the ray set-up does not wait)."""
         R = rays_o.shape[0]
         dev = rays_o.device
         rgb = torch.empty((R, 3), device=dev) if rgb is None else rgb
