@@ -493,6 +493,13 @@ def roofline(kind, total_ms, launches, fwd_units, bwd_units, chosen, peaks, adam
                     "frac": achieved / peak, "traffic": traffic_from_profiles(kind, chosen), "units_per_launch": units,
                     "flop_per_launch": flop, "ms_per_launch": avg_ms, "launches": launches,
                     "peak_source": "measured bf16 sustained" if "bf16_tflops_sustained" in peaks else "fallback"}
+        if kind == "fine_colour_fwd" or n_freq_pos() == 0:   # six BF16 products for each FP32 one
+            peak = peaks.get("bf16_tflops_sustained", 1700.0) / 6
+            return {"bound": "tensor", "kernel": kind, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                    "frac": achieved / peak, "traffic": traffic_from_profiles(kind, chosen), "units_per_launch": units,
+                    "flop_per_launch": flop, "ms_per_launch": avg_ms, "launches": launches,
+                    "peak_source": ("measured" if "bf16_tflops_sustained" in peaks else "fallback") +
+                                   " bf16 sustained / 6 (an FP32 product is six BF16 ones)"}
         peak = 152 * 128 * 2 * 2.07e9 / 1e12
         return {"bound": "alu", "kernel": kind, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic_from_profiles(kind, chosen), "units_per_launch": units,
@@ -523,7 +530,7 @@ def traffic_from_profiles(kind, chosen):
     current source (the summary records the source file's hash)."""
     import hashlib
     import re
-    prof, src = {("fine_colour_bwd", False): ("fine_colour_bwd_fp32_160cube_8192rays.md", "fine_simt.cu"),
+    prof, src = {("fine_colour_bwd", False): ("fine_colour_bwd_fp32_160cube_8192rays.md", "fine_tc_fp32_bwd.cu"),
                  ("fine_colour_bwd", True): ("fine_kernels_bf16_chosen_160cube_8192rays.md", "fine_tc.cu"),
                  ("adam", False): ("adam_fine_step_160cube.md", "adam.cu"),
                  ("adam", True): ("adam_fine_step_160cube.md", "adam.cu")}.get((kind, chosen), (None, None))
