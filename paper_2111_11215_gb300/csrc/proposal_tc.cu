@@ -166,7 +166,7 @@ __device__ __forceinline__ void encode_row_tmem(const ClipDf &c, uint32_t ta) {
 // Epilogue: 32-column chunk g of the accumulator (+ bias), ReLU, as BF16 into the A-operand
 // columns 16 g .. 16 g + 15 of this thread's TMEM lane.
 __device__ __forceinline__ void relu_to_tmem(uint32_t tz, uint32_t ta, const float *bias) {
-#pragma unroll 1
+#pragma unroll
     for (int g = 0; g < 2; ++g) {
         float z[32];
         tmem_ld32(tz + 32u * (uint32_t)g, z);
@@ -175,8 +175,8 @@ __device__ __forceinline__ void relu_to_tmem(uint32_t tz, uint32_t ta, const flo
         for (int k = 0; k < 32; k += 4) {
             float4 bb = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (bias) bb = *reinterpret_cast<const float4 *>(bias + 32 * g + k);
-            h[k / 2] = pack_bf16(fmaxf(z[k] + bb.x, 0.0f), fmaxf(z[k + 1] + bb.y, 0.0f));
-            h[k / 2 + 1] = pack_bf16(fmaxf(z[k + 2] + bb.z, 0.0f), fmaxf(z[k + 3] + bb.w, 0.0f));
+            h[k / 2] = relu_bf16(pack_bf16(z[k] + bb.x, z[k + 1] + bb.y));
+            h[k / 2 + 1] = relu_bf16(pack_bf16(z[k + 2] + bb.z, z[k + 3] + bb.w));
         }
         tmem_st16(ta + 16u * (uint32_t)g, h);
     }
@@ -203,11 +203,10 @@ __global__ void __launch_bounds__(TT, kFwdCtasPerSm) proposal_fwd_tc_kernel(Prop
     // one layer: D (COL_Z) = A (COL_A, TMEM) x W^T (K = 64: four k-steps of 8 columns), then wait
     auto layer = [&](unsigned char *wt) -> bool {
         if (tid == 0) {
-            uint32_t w_ = smem_u32(wt);
-            asm volatile("" : "+r"(w_));
-#pragma unroll 1
-            for (int kk = 0; kk < 4; ++kk)
-                mma_ts(tb + COL_Z, tb + COL_A + 8u * (uint32_t)kk, desc_kmajor(w_, kk), id64, kk > 0);
+            // (constant steps: with the descriptors formed anew an MMA took its thread 130 clocks, twice its own time)
+            const uint64_t w_k = desc_kmajor(smem_u32(wt), 0);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma_ts(tb + COL_Z, tb + COL_A + 8u * (uint32_t)kk, w_k + kstep(kk), id64, kk > 0);
             commit(&S.sm.mbar);
         }
         const bool w = mbar_wait(&S.sm.mbar, phase);
@@ -314,8 +313,8 @@ struct SmemB {
 
 // MN-major A operand of M = 128 whose first 64 rows are panel `base` and last 64 rows the panel
 // `lbo` bytes after it; k-step kk = 16 tile rows.
-__device__ __forceinline__ uint64_t desc_mn_pair(uint32_t base, int kk, uint32_t lbo) {
-    return sdesc(base + (uint32_t)kk * 2u * kGroupBytes, lbo, kGroupBytes);
+__device__ __forceinline__ uint64_t desc_mn_pair(uint32_t base, uint32_t lbo) {
+    return sdesc(base, lbo, kGroupBytes);
 }
 
 // ReLU epilogue of one 64-column layer accumulator: h = max(z + b, 0) into the panel, the ReLU mask
@@ -429,8 +428,8 @@ __global__ void __launch_bounds__(TT, 1) proposal_bwd_tc_kernel(PropTcArgs P) {
         uint32_t m0[2], m1[2], m2[2];
         // ---- forward: three layers ----
         if (tid == 0) {
-#pragma unroll 1
-            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(x_, kk), desc_kmajor(w0_, kk), id_fwd, kk > 0);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(x_, 0) + kstep(kk), desc_kmajor(w0_, 0) + kstep(kk), id_fwd, kk > 0);
             commit(&S.sm.mbar);
         }
         ok = mbar_wait(&S.sm.mbar, phase);
@@ -441,8 +440,8 @@ __global__ void __launch_bounds__(TT, 1) proposal_bwd_tc_kernel(PropTcArgs P) {
         fence_async_smem();
         sync_fenced();
         if (tid == 0) {
-#pragma unroll 1
-            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(h0_, kk), desc_kmajor(w1_, kk), id_fwd, kk > 0);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(h0_, 0) + kstep(kk), desc_kmajor(w1_, 0) + kstep(kk), id_fwd, kk > 0);
             commit(&S.sm.mbar);
         }
         ok = mbar_wait(&S.sm.mbar, phase);
@@ -453,8 +452,8 @@ __global__ void __launch_bounds__(TT, 1) proposal_bwd_tc_kernel(PropTcArgs P) {
         fence_async_smem();
         sync_fenced();
         if (tid == 0) {
-#pragma unroll 1
-            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(h1_, kk), desc_kmajor(w2_, kk), id_fwd, kk > 0);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(h1_, 0) + kstep(kk), desc_kmajor(w2_, 0) + kstep(kk), id_fwd, kk > 0);
             commit(&S.sm.mbar);
         }
         ok = mbar_wait(&S.sm.mbar, phase);
@@ -494,14 +493,14 @@ __global__ void __launch_bounds__(TT, 1) proposal_bwd_tc_kernel(PropTcArgs P) {
         sync_fenced();
         // ---- dW2 | db2, dW3 | db3, dH1 ----
         if (tid == 0) {
-#pragma unroll 1
+#pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-                mma(tb + BCOL_DW2, desc_mn_pair(h1_, kk, e_ - h1_), desc_mnmajor(dza_, kk), id_dw, acc | (kk > 0));
-#pragma unroll 1
+                mma(tb + BCOL_DW2, desc_mn_pair(h1_, e_ - h1_) + mnstep(kk), desc_mnmajor(dza_, 0) + mnstep(kk), id_dw, acc | (kk > 0));
+#pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-                mma(tb + BCOL_DW3, desc_mn_pair(h2_, kk, e_ - h2_), desc_mnmajor(dl_, kk), id_dw3, acc | (kk > 0));
-#pragma unroll 1
-            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(dza_, kk), desc_mnmajor(w2_, kk), id_dh, kk > 0);
+                mma(tb + BCOL_DW3, desc_mn_pair(h2_, e_ - h2_) + mnstep(kk), desc_mnmajor(dl_, 0) + mnstep(kk), id_dw3, acc | (kk > 0));
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(dza_, 0) + kstep(kk), desc_mnmajor(w2_, 0) + mnstep(kk), id_dh, kk > 0);
             commit(&S.sm.mbar);
         }
         ok = mbar_wait(&S.sm.mbar, phase);
@@ -513,11 +512,11 @@ __global__ void __launch_bounds__(TT, 1) proposal_bwd_tc_kernel(PropTcArgs P) {
         sync_fenced();
         // ---- dW1 | db1, dH0 ----
         if (tid == 0) {
-#pragma unroll 1
+#pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-                mma(tb + BCOL_DW1, desc_mn_pair(h0_, kk, e_ - h0_), desc_mnmajor(dzb_, kk), id_dw, acc | (kk > 0));
-#pragma unroll 1
-            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(dzb_, kk), desc_mnmajor(w1_, kk), id_dh, kk > 0);
+                mma(tb + BCOL_DW1, desc_mn_pair(h0_, e_ - h0_) + mnstep(kk), desc_mnmajor(dzb_, 0) + mnstep(kk), id_dw, acc | (kk > 0));
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma(tb + BCOL_Z, desc_kmajor(dzb_, 0) + kstep(kk), desc_mnmajor(w1_, 0) + mnstep(kk), id_dh, kk > 0);
             commit(&S.sm.mbar);
         }
         ok = mbar_wait(&S.sm.mbar, phase);
@@ -529,9 +528,9 @@ __global__ void __launch_bounds__(TT, 1) proposal_bwd_tc_kernel(PropTcArgs P) {
         sync_fenced();
         // ---- [dW0 | db0] (input column 39 is the constant 1) ----
         if (tid == 0) {
-#pragma unroll 1
+#pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-                mma(tb + BCOL_DW0, desc_mn_pair(x_, kk, e_ - x_), desc_mnmajor(dza_, kk), id_dw, acc | (kk > 0));
+                mma(tb + BCOL_DW0, desc_mn_pair(x_, e_ - x_) + mnstep(kk), desc_mnmajor(dza_, 0) + mnstep(kk), id_dw, acc | (kk > 0));
             commit(&S.sm.mbar);
         }
         ok = mbar_wait(&S.sm.mbar, phase);
