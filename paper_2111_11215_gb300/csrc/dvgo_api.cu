@@ -188,9 +188,9 @@ RenderArgs make_args(const dvgo_params *p, const dvgo_grid_desc *dd, const float
     if (p->mode == DVGO_MODE_FINE) {
         A.pe = reinterpret_cast<float *>(b + L.pe);
         A.texit = reinterpret_cast<double *>(b + L.texit);
-        A.rayk = reinterpret_cast<int2 *>(b + L.rayk);
+        A.rayk = reinterpret_cast<int4 *>(b + L.rayk);
+        A.rchunk = reinterpret_cast<RayChunk *>(b + L.rchunk);
         A.stau = reinterpret_cast<float *>(b + L.stau);
-        A.kidx = reinterpret_cast<unsigned short *>(b + L.kidx);
         A.scol = reinterpret_cast<float4 *>(b + L.scol);
         A.sgrad = reinterpret_cast<float4 *>(b + L.sgrad);
         A.kept = reinterpret_cast<int2 *>(b + L.kept);
@@ -203,6 +203,7 @@ RenderArgs make_args(const dvgo_params *p, const dvgo_grid_desc *dd, const float
     }
     A.max_samples = L.max_samples;
     A.cap = R > 0 ? (int)(L.max_samples / R) : 0;
+    A.nchunk = chunks_per_ray(A.cap);
     if (p->mode == DVGO_MODE_FINE && p->freespace && p->freespace->density) {
         const dvgo_freespace &f = *p->freespace;
         A.fs_density = f.density;

@@ -50,6 +50,15 @@ struct RayRec {
 };
 static_assert(sizeof(RayRec) == 128, "RayRec layout");
 
+// 32 consecutive samples of a ray of which at least one is kept, as the density pass leaves them.
+struct alignas(16) RayChunk {
+    unsigned mask;       // bit l: sample 32 index + l is kept
+    float pre;           // optical depth in front of sample 32 index
+    int index;
+    int first;           // the ray's slot of the first kept one; the others follow it
+};
+inline int chunks_per_ray(long long cap) { return (int)((cap + 31) / 32); }
+
 // Workspace header (first 256 bytes of the workspace).
 struct WsHeader {
     int flags;           // bit 0: a ray of the last forward had a zero / non-finite direction
@@ -66,7 +75,7 @@ static_assert(sizeof(WsHeader) == 256, "WsHeader size");
 
 // Workspace layout; every block 256-byte aligned.
 struct WsLayout {
-    size_t header, rays, rayout, rtarget, pe, texit, rayk, stau, kidx, scol, sgrad, kept, mask, xcache, total;
+    size_t header, rays, rayout, rtarget, pe, texit, rayk, rchunk, stau, scol, sgrad, kept, mask, xcache, total;
                                  // mask, xcache 0: none
     long long max_samples;
 };
@@ -99,9 +108,9 @@ struct RenderArgs {
     float *pe;                  // fine: per ray [d (3), sin (12), cos (12), 0 x 5] (kPeStride floats)
     double *texit;              // fine: per ray clipped exit distance
     // A ray's kept samples sit in order at the front of its cap slots: slot ray * cap + j is the j-th.
-    int2 *rayk;                 // fine: per ray (kept samples, first terminated sample or INT_MAX)
+    int4 *rayk;                 // fine: per ray (chunk records, first terminated sample or INT_MAX, T_K, kept samples)
+    RayChunk *rchunk;           // per ray, nchunk places: its chunks that hold a kept sample, in order
     float *stau;                // per slot: optical depth tau (density pass)
-    unsigned short *kidx;       // per slot: sample index k along the ray
     float4 *scol;               // per slot: (r, g, b, tau) (colour kernels)
     float4 *sgrad;              // per slot: (0, dL/do), o the output layer's value before the sigmoid
     int2 *kept;                 // compact list of kept samples: (j | k << 16, ray)
@@ -112,6 +121,7 @@ struct RenderArgs {
                                 // each, swizzled as in shared memory), reloaded by the backward
     long long max_samples;      // slots of the whole batch: R * cap
     int cap;                    // sample slots per ray (the longest possible ray)
+    int nchunk;                 // chunks_per_ray(cap)
     // outputs
     float *rgb_out, *tfinal_out, *loss_out, *dloss_out;
     // backward inputs / outputs

@@ -6,10 +6,14 @@
 //                 (Eq. fine_queries_densities), tau_k = softplus(sigma_ddot + b) * dt_k
 //                 (Eq. density_activation, post-activation), removed when
 //                 alpha_k = 1 - exp(-tau_k) < tau_f (Sec. 4.2 free space skipping).
-//                 Kept samples are packed in order at the front of the ray's slots (tau_k and the sample
-//                 index k): the passes after it walk the kept samples alone, which under the skips are a
-//                 few per cent of all; they are also appended to the batch's list for the colour
-//                 kernel (one atomic per 64 samples, order along the ray kept).
+//                 Kept samples are packed in order at the front of the ray's slots, and every 32 samples that
+//                 hold one leave a record (RayChunk): the passes after it walk these records alone,
+//                 which under the skips are a few per cent of all; the samples are also appended to the
+//                 batch's list for the colour kernel (one atomic per 64 samples, order along the ray kept).
+//                 A record keeps its samples in their lanes and the optical depth in front of them, so every
+//                 sum over a ray is associated as without the skips: weights, colours and dL/do carry
+//                 the same bits whatever was left out (scanning the packed samples moved the last bit of a
+//                 quarter of the weights, which flipped BF16 roundings of dL/do).
 //                 Early ray termination: a sample where T_k = exp(-(sum_{j<k} tau_j)) is exactly 0 in
 //                 FP32 has weight 0 and no gradient through it, so it and the rest of the ray are
 //                 not kept (nor queried), and T_K is exactly 0.
@@ -138,7 +142,8 @@ __global__ void __launch_bounds__(kDensityThreads) fine_density_kernel(RenderArg
         const RayRec rr = A.rays[r];
         flag_bad_ray(A, rr, lane);
         float carry = 0.0f;          // optical depth before this chunk
-        int nk = 0, kend = INT_MAX;
+        int nk = 0, nrec = 0, kend = INT_MAX;
+        RayChunk *recs = A.rchunk + (size_t)r * A.nchunk;
         long long u[3];              // uniform steps: lattice coordinate of sample base + lane
         if (!kExpl)
 #pragma unroll
@@ -189,6 +194,7 @@ __global__ void __launch_bounds__(kDensityThreads) fine_density_kernel(RenderArg
                     for (int a = 0; a < 3; ++a) u[a] += 64 * rr.dfx[a];
             }
             unsigned m[2];
+            float pre[2];
             bool done = false;       // the ray is terminated: T = 0 from here on
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -199,6 +205,7 @@ __global__ void __launch_bounds__(kDensityThreads) fine_density_kernel(RenderArg
                 const bool dead = done || expf(-(carry + excl)) == 0.0f;
                 if (dead) kept[h] = false;
                 const unsigned end = __ballot_sync(FULL, (dead || isinf(tau[h])) && base + 32 * h + lane < rr.n);
+                pre[h] = carry;
                 if (!done) {
                     if (end) {
                         kend = base + 32 * h + __ffs(end) - 1;
@@ -219,13 +226,16 @@ __global__ void __launch_bounds__(kDensityThreads) fine_density_kernel(RenderArg
                 if (kept[h]) {
                     const int j = nk + pos[h], k = base + 32 * h + lane;
                     A.stau[(size_t)rr.off + j] = tau[h];
-                    A.kidx[(size_t)rr.off + j] = (unsigned short)k;
                     A.kept[base_slot + pos[h]] = make_int2(j | k << 16, r);
                 }
+            if (lane == 0 && m[0]) recs[nrec] = RayChunk{m[0], pre[0], base / 32, nk};
+            nrec += m[0] ? 1 : 0;
+            if (lane == 0 && m[1]) recs[nrec] = RayChunk{m[1], pre[1], base / 32 + 1, nk + cnt0};
+            nrec += m[1] ? 1 : 0;
             nk += cnt;
             if (done) break;
         }
-        if (lane == 0) A.rayk[r] = make_int2(nk, kend);
+        if (lane == 0) A.rayk[r] = make_int4(nrec, kend, __float_as_int(kend != INT_MAX ? 0.0f : expf(-carry)), nk);
     }
 }
 
@@ -264,34 +274,39 @@ __global__ void __launch_bounds__(kLossThreads) fine_composite_kernel(RenderArgs
     float loss_part = 0.0f;
     const bool aux = A.target && (A.w_pt != 0.0f || A.w_bg != 0.0f);
     for (int r = warp; r < A.R; r += nwarps) {
-        const int2 nk = A.rayk[r];   // kept samples; a terminated ray has T_K = 0
-        const bool terminated = nk.y != INT_MAX;
-        const int n = nk.x;
+        const int4 rk = A.rayk[r];
         const size_t off = (size_t)r * A.cap;
         float tg[3] = {0.0f, 0.0f, 0.0f};
         if (aux)
             for (int ch = 0; ch < 3; ++ch) tg[ch] = A.target[3 * r + ch];
-        float carry = 0.0f, acc[3] = {0.0f, 0.0f, 0.0f}, pt = 0.0f;
-        for (int base = 0; base < n; base += 32) {
-            int k = base + lane;
-            float4 c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (k < n) c = A.scol[off + k];
-            float incl = warp_incl_scan(c.w, lane);
-            float excl = __shfl_up_sync(FULL, incl, 1);
-            if (lane == 0) excl = 0.0f;
-            float w = expf(-(carry + excl)) * -expm1f(-c.w);
-            acc[0] = fmaf(w, c.x, acc[0]);
-            acc[1] = fmaf(w, c.y, acc[1]);
-            acc[2] = fmaf(w, c.z, acc[2]);
-            const float e0 = c.x - tg[0], e1 = c.y - tg[1], e2 = c.z - tg[2];
-            pt = fmaf(w, fmaf(e0, e0, fmaf(e1, e1, e2 * e2)), pt);   // per-point rgb loss
-            carry += __shfl_sync(FULL, incl, 31);
+        float acc[3] = {0.0f, 0.0f, 0.0f}, pt = 0.0f;
+        for (int c0 = 0; c0 < rk.x; c0 += 32) {
+            const int nc = min(32, rk.x - c0);
+            RayChunk mine;
+            if (lane < nc) mine = A.rchunk[(size_t)r * A.nchunk + c0 + lane];
+#pragma unroll 2
+            for (int c = 0; c < nc; ++c) {
+                const unsigned m = __shfl_sync(FULL, mine.mask, c);
+                const float pre = __shfl_sync(FULL, mine.pre, c);
+                const int first = __shfl_sync(FULL, mine.first, c);
+                float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if ((m >> lane) & 1u) v = A.scol[off + first + __popc(m & ((1u << lane) - 1u))];
+                const float incl = warp_incl_scan(v.w, lane);
+                float excl = __shfl_up_sync(FULL, incl, 1);
+                if (lane == 0) excl = 0.0f;
+                const float w = expf(-(pre + excl)) * -expm1f(-v.w);
+                acc[0] = fmaf(w, v.x, acc[0]);
+                acc[1] = fmaf(w, v.y, acc[1]);
+                acc[2] = fmaf(w, v.z, acc[2]);
+                const float e0 = v.x - tg[0], e1 = v.y - tg[1], e2 = v.z - tg[2];
+                pt = fmaf(w, fmaf(e0, e0, fmaf(e1, e1, e2 * e2)), pt);   // per-point rgb loss
+            }
         }
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) acc[ch] = warp_sum(acc[ch]);
         if (aux) pt = warp_sum(pt);
         if (lane == 0) {
-            float TK = terminated ? 0.0f : expf(-carry);
+            const float TK = __int_as_float(rk.z);
             float rgb[3];
             for (int ch = 0; ch < 3; ++ch) rgb[ch] = fmaf(TK, A.bg[ch], acc[ch]);
             for (int ch = 0; ch < 3; ++ch) A.rgb_out[3 * r + ch] = rgb[ch];
@@ -315,15 +330,13 @@ __global__ void __launch_bounds__(kLossThreads) fine_composite_kernel(RenderArgs
 
 template <int kOrder>
 __global__ void __launch_bounds__(kRayThreads) fine_comp_bwd_kernel(RenderArgs A) {
-    __shared__ float s_pre[kRayThreads / 32][kMaxChunks];   // optical depth before each chunk, per warp
-    int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int r = warp; r < A.R; r += nwarps) {
-        const int nk = A.rayk[r].x;   // kept samples
-        if (nk == 0) continue;
+        const int4 rk = A.rayk[r];
+        if (rk.x == 0) continue;   // no kept sample
         const RayRec rr = A.rays[r];
-        const int nch = (nk + 31) >> 5;
         const float TK = A.rayout[r].w;
         const float g[3] = {A.grad_rgb[3 * r], A.grad_rgb[3 * r + 1], A.grad_rgb[3 * r + 2]};
         // auxiliary losses of the forward: the background entropy enters through T_K, the
@@ -334,43 +347,48 @@ __global__ void __launch_bounds__(kRayThreads) fine_comp_bwd_kernel(RenderArgs A
         const float gT = (A.grad_tfinal ? A.grad_tfinal[r] : 0.0f) +
                          (aux ? A.w_bg * bg_entropy_dT(TK) / (float)A.R : 0.0f);
         const float kpt = aux ? 2.0f * A.w_pt / (float)A.R : 0.0f;
-        // pass 1 (front to back): optical depth at the start of every chunk, as in the forward
-        float carry = 0.0f;
-        for (int ci = 0; ci < nch; ++ci) {
-            const int j = ci * 32 + lane;
-            float tau = j < nk ? A.stau[(size_t)rr.off + j] : 0.0f;
-            float incl = warp_incl_scan(tau, lane);
-            if (lane == 0) s_pre[wib][ci] = carry;
-            carry += __shfl_sync(FULL, incl, 31);
-        }
-        __syncwarp();
-        // pass 2 (back to front): D_k = dC/dtau_k as a suffix sum of T_{j+1} (c_j - c_{j+1})
+        // back to front: D_k = dC/dtau_k as a suffix sum of T_{j+1} (c_j - c_{j+1}), the colour of a sample that
+        // is not kept being 0
         float Dc[3] = {0.0f, 0.0f, 0.0f};
         float cnext[3] = {A.bg[0], A.bg[1], A.bg[2]};   // colour after the chunk's last sample
-        for (int ci = nch - 1; ci >= 0; --ci) {
-            const int j = ci * 32 + lane;
-            const bool valid = j < nk;
-            const size_t slot = (size_t)rr.off + j;
-            int k = 0;
-            float4 sv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (valid) {
-                k = A.kidx[slot];
-                sv = A.scol[slot];
+        float Tnext = TK;                               // T in front of it
+        int inext = (rr.n + 31) >> 5;                   // the chunk handled before this one
+        RayChunk mine;
+        for (int ci = rk.x - 1; ci >= 0; --ci) {
+            if (ci == rk.x - 1 || (ci & 31) == 31) {
+                const int q = (ci & ~31) + lane;
+                if (q < rk.x) mine = A.rchunk[(size_t)r * A.nchunk + q];
             }
+            const unsigned m = __shfl_sync(FULL, mine.mask, ci & 31);
+            const float pre = __shfl_sync(FULL, mine.pre, ci & 31);
+            const int chunk = __shfl_sync(FULL, mine.index, ci & 31), first = __shfl_sync(FULL, mine.first, ci & 31);
+            if (chunk + 1 < inext) {   // chunks without a kept sample in between: the step from 0 to the colour after them
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch) {
+                    Dc[ch] += Tnext * (0.0f - cnext[ch]);
+                    cnext[ch] = 0.0f;
+                }
+            }
+            inext = chunk;
+            const int k = chunk * 32 + lane;
+            const bool valid = k < rr.n, kept = (m >> lane) & 1u;
+            const size_t slot = (size_t)rr.off + first + __popc(m & ((1u << lane) - 1u));
+            float4 sv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (kept) sv = A.scol[slot];
             const float tau = sv.w;
             const float cc[3] = {sv.x, sv.y, sv.z};
-            float pre = s_pre[wib][ci];
-            float incl = warp_incl_scan(tau, lane);
+            const float incl = warp_incl_scan(tau, lane);
             float excl = __shfl_up_sync(FULL, incl, 1);
             if (lane == 0) excl = 0.0f;
-            float T = expf(-(pre + excl));
-            float T1 = expf(-(pre + incl));
-            float w = T * -expm1f(-tau);
+            const float T = expf(-(pre + excl));
+            const float T1 = k >= rk.y ? 0.0f : expf(-(pre + incl));   // (rk.y: the first terminated sample)
+            const float w = T * -expm1f(-tau);
+            Tnext = expf(-pre);
             float D[3];
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) {
                 float cn = __shfl_down_sync(FULL, cc[ch], 1);
-                if (lane == 31 || j + 1 >= nk) cn = (j + 1 >= nk) ? A.bg[ch] : cnext[ch];
+                if (lane == 31 || k + 1 >= rr.n) cn = (k + 1 >= rr.n) ? A.bg[ch] : cnext[ch];
                 float X = valid ? T1 * (cc[ch] - cn) : 0.0f;
                 float sx = warp_suffix_scan(X, lane);
                 D[ch] = Dc[ch] + sx;
@@ -381,12 +399,12 @@ __global__ void __launch_bounds__(kRayThreads) fine_comp_bwd_kernel(RenderArgs A
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) dtau = fmaf(g[ch], D[ch], dtau);
             // kept samples have tau > 0 or an exactly-zero sigmoid factor
-            bool act = valid && tau > 0.0f;
+            const bool act = kept && tau > 0.0f;
             Cell c;
             c.i0 = c.j0 = c.k0 = 0;
             c.fx = c.fy = c.fz = 0.0f;
             float dz = 0.0f, dt = 0.0f;
-            if (valid) {
+            if (kept) {
                 c = sample_cell(A, rr, r, k, dt);
                 dz = act ? dtau * dt * -expm1f(-tau / dt) : 0.0f;   // post: dt sigmoid(z) = dt (1 - e^{-tau/dt})
                 // for the colour backward: dL/dc_k through the sigmoid, dL/do = dL/dc c (1 - c)
@@ -425,7 +443,6 @@ __global__ void __launch_bounds__(kRayThreads) fine_comp_bwd_kernel(RenderArgs A
             for (int q = 0; q < 8; ++q)   // the run's last lane adds its total; terminated samples add 0
                 if (act && sg.tail && gq[q] != 0.0f) atomicAdd(A.grad_density + idx[q], gq[q]);
         }
-        __syncwarp();
     }
 }
 

@@ -76,24 +76,24 @@ __global__ void __launch_bounds__(256) weight_bins_kernel(RenderArgs A, int nbin
         const double bin_scale = __ddiv_rn(__dmul_rn((double)A.step, (double)nbins), __dsub_rn(t1, t0));
         for (int b = lane; b < nbins; b += 32) bins[wib][b] = 0.0f;
         __syncwarp();
-        float carry = 0.0f, wsum = 0.0f;
-        const int nk = A.rayk[r].x;   // the kept samples; the others have weight 0
+        float wsum = 0.0f;
+        const int nrec = A.rayk[r].x;   // chunks with a kept sample; the other samples have weight 0
         const size_t off = (size_t)r * A.cap;
-        for (int base = 0; base < nk; base += 32) {
-            const int j = base + lane;
-            const float tau = j < nk ? A.stau[off + j] : 0.0f;
+        for (int c = 0; c < nrec; ++c) {
+            const RayChunk ch = A.rchunk[(size_t)r * A.nchunk + c];
+            const bool kept = (ch.mask >> lane) & 1u;
+            const float tau = kept ? A.stau[off + ch.first + __popc(ch.mask & ((1u << lane) - 1u))] : 0.0f;
             const float incl = warp_incl_scan(tau, lane);
             float excl = __shfl_up_sync(0xffffffffu, incl, 1);
             if (lane == 0) excl = 0.0f;
-            const float w = expf(-(carry + excl)) * -expm1f(-tau);
-            if (j < nk) {
-                const int k = A.kidx[off + j];
+            const float w = expf(-(ch.pre + excl)) * -expm1f(-tau);
+            if (kept) {
+                const int k = ch.index * 32 + lane;
                 int b = (int)floor(__dmul_rn(__dadd_rn((double)k, (double)rr.p), bin_scale));
                 b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
                 atomicAdd(&bins[wib][b], w);
             }
             wsum += warp_sum(w);
-            carry += __shfl_sync(0xffffffffu, incl, 31);
         }
         __syncwarp();
         const bool uniform = wsum < 1e-4f;
@@ -565,9 +565,10 @@ int dvgo_weight_bins(const dvgo_params *p, const dvgo_grid_desc *dd, int n_rays,
     A.step = p->step;
     A.rays = reinterpret_cast<RayRec *>(b + L.rays);
     A.cap = (int)cap;
-    A.rayk = reinterpret_cast<int2 *>(b + L.rayk);
+    A.nchunk = chunks_per_ray(cap);
+    A.rayk = reinterpret_cast<int4 *>(b + L.rayk);
+    A.rchunk = reinterpret_cast<RayChunk *>(b + L.rchunk);
     A.stau = reinterpret_cast<float *>(b + L.stau);
-    A.kidx = reinterpret_cast<unsigned short *>(b + L.kidx);
     A.texit = reinterpret_cast<double *>(b + L.texit);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int blocks = (n_rays + 7) / 8;

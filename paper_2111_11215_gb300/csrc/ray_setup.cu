@@ -135,9 +135,9 @@ WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache, size_t m
     if (mode == DVGO_MODE_FINE) {
         L.pe = o; o += up(sizeof(float) * kPeStride * n);
         L.texit = o; o += up(sizeof(double) * n);
-        L.rayk = o; o += up(sizeof(int2) * n);
+        L.rayk = o; o += up(sizeof(int4) * n);
+        L.rchunk = o; o += up(sizeof(RayChunk) * n * chunks_per_ray((long long)(S / n)));
         L.stau = o; o += up(sizeof(float) * S);
-        L.kidx = o; o += up(sizeof(unsigned short) * S);
         L.scol = o; o += up(sizeof(float4) * S);
         L.sgrad = o; o += up(sizeof(float4) * S);
         L.kept = o; o += up(sizeof(int2) * S);
