@@ -108,9 +108,11 @@ __device__ __forceinline__ void gather_features(const RenderArgs &A, const Cell 
 }
 
 // A row of a tile as the scatter needs it: the offsets inside its lattice cell (a little below 0 or above 1 on
-// the rim of the box) and the cell (cell_base; -1 for a padding row, which come last in a tile).
+// the rim of the box) and the cell (cell_base; kNoCell for a padding row, which come last in a tile).  A packed
+// cell_base with i0 >= 1024 is negative too; kNoCell would be i0 = 2047, and i0 <= 2046.
+constexpr int kNoCell = -1;
 __device__ __forceinline__ float4 row_place(const RenderArgs &A, const Cell &c, bool live, bool packed) {
-    return make_float4(c.fx, c.fy, c.fz, __int_as_float(live ? cell_base(c, A.ny, A.nz, packed) : -1));
+    return make_float4(c.fx, c.fy, c.fz, __int_as_float(live ? cell_base(c, A.ny, A.nz, packed) : kNoCell));
 }
 
 // *p += v (four floats, 16-byte aligned, in global memory), where `on` is not zero.
@@ -172,7 +174,7 @@ __device__ __forceinline__ void scatter_rows(const RenderArgs &A, const float4 *
     const int col = 4 * px + 2 * py + pz;
     unsigned flush;   // bit j: my sum leaves for the grid after row j
     const float4 mine = place[row];
-    const unsigned live = __ballot_sync(ALL, __float_as_int(mine.w) >= 0);
+    const unsigned live = __ballot_sync(ALL, __float_as_int(mine.w) != kNoCell);
     const int n = __popc(live);
     unsigned odd_x, odd_y, odd_z;   // bit j: the base corner of row j's cell is odd along the axis
     {
@@ -185,7 +187,7 @@ __device__ __forceinline__ void scatter_rows(const RenderArgs &A, const float4 *
         const int cb = __float_as_int(mine.w), cbn = __shfl_down_sync(ALL, cb, 1);
         int dx, dy, dz;
         bool adj = cells_adjacent<PK>(cb, cbn, A.ny, A.nz, dx, dy, dz);
-        adj = adj && lane < 31 && cbn >= 0;
+        adj = adj && lane < 31 && cbn != kNoCell;
         const unsigned xp = __ballot_sync(ALL, dx > 0), xm = __ballot_sync(ALL, dx < 0);
         const unsigned yp = __ballot_sync(ALL, dy > 0), ym = __ballot_sync(ALL, dy < 0);
         const unsigned zp = __ballot_sync(ALL, dz > 0), zm = __ballot_sync(ALL, dz < 0);

@@ -154,7 +154,7 @@ __device__ __forceinline__ void produce_row(const RenderArgs &A, SmemTC &S, int 
 #pragma unroll
     for (int i = 0; i < 16; ++i) tail[i] = 0.0f;
     int slot = -1;
-    float4 place = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));
+    float4 place = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(kNoCell));
     float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f;
     if (kv.y >= 0) {
         float dt;
