@@ -149,10 +149,10 @@ __device__ __noinline__ float exact_z2(const RenderArgs &A, int e, int unit) {
 }
 
 // The signs of the units within rounding of zero, decided by the FMA chains: amb marks this lane's among
-// samples e0 .. e0 + 15 (bit k), neg holds the sign bits (sample k in bit 15 - k) and is returned corrected.  A
-// unit counts as off unless z > 0.  All lanes of the warp take part.
+// samples e0 .. e0 + 15 (bit k), on holds the bits z > 0 (sample k in bit 15 - k) and is returned corrected.  All
+// lanes of the warp take part.
 template <typename FeatT, bool PK, int kLayer>
-__device__ __noinline__ uint32_t resolve(const RenderArgs &A, int e0, int unit, uint32_t amb, uint32_t neg) {
+__device__ __noinline__ uint32_t resolve(const RenderArgs &A, int e0, int unit, uint32_t amb, uint32_t on) {
     const int lane = threadIdx.x & 31;
     for (unsigned any = __ballot_sync(FULL, amb != 0u); any; any = __ballot_sync(FULL, amb != 0u)) {
         const int src = __ffs(any) - 1, k = __ffs(__shfl_sync(FULL, amb, src)) - 1, u = __shfl_sync(FULL, unit, src);
@@ -160,12 +160,12 @@ __device__ __noinline__ uint32_t resolve(const RenderArgs &A, int e0, int unit, 
         if (lane == src) {
             amb &= amb - 1u;
             const uint32_t bit = 0x8000u >> k;
-            neg = z > 0.0f ? neg & ~bit : neg | bit;
+            on = z > 0.0f ? on | bit : on & ~bit;
         }
     }
-    return neg;
+    return on;
 }
-__device__ __forceinline__ bool off(uint32_t neg, int k) { return (neg >> (15 - k)) & 1u; }
+__device__ __forceinline__ bool off(uint32_t on, int k) { return !((on >> (15 - k)) & 1u); }
 
 // Splits 16 consecutive samples of this thread's unit (row n, samples 64 hc + 16 g ..): the three terms as
 // packed pairs (for TMEM) in w, and the chosen ones into the half panels lo / mid (row = unit).
@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             }
         }
         const float w30 = A.w3[3 * n], w31 = A.w3[3 * n + 1], w32 = A.w3[3 * n + 2], b2 = A.b2[n];
+        const float nb2 = __fsub_rn(0.0f, b2);   // (+0 for a bias of 0)
         // Where a unit's sign is looked at again: 2^-23 of a bound on the sum of magnitudes behind z (more than
         // ten times the usual difference of the two arithmetics), for inputs of magnitude 1.
         float s1 = fabsf(A.b1[n]), s2 = 0.0f;
@@ -461,7 +462,9 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             }
             if (!wait_a()) { ok = false; break; }
             // ---- epilogue 1: H1 = relu(Z1), split: TMEM (A of dW2), lo and mid into the pool ----
-            uint32_t m1[4], m2[2];   // which units are off: 16 samples a word, sample k in bit 15 - k
+            // Which units are on (z > 0): 16 samples a word, sample k in bit 15 - k.  The sign of 0 - z is set just
+            // there: not for a zero of either sign (a unit whose weights are all 0) nor for a NaN.
+            uint32_t m1[4], m2[2];
             float zz[32];
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
@@ -469,14 +472,14 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 bool near = false;   // a unit within rounding of zero
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    uint32_t neg = 0;   // sign bits, sample k in bit 15 - k
+                    uint32_t on = 0;
                     float low = 0x1p127f;
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
-                        neg = __funnelshift_l(__float_as_uint(zz[16 * q + k]), neg, 1);
+                        on = __funnelshift_l(__float_as_uint(__fsub_rn(0.0f, zz[16 * q + k])), on, 1);
                         low = fminf(low, fabsf(zz[16 * q + k]));
                     }
-                    m1[2 * half + q] = neg;
+                    m1[2 * half + q] = on;
                     near |= low < eps1 * S.gmax[4 * hc + 2 * half + q];
                 }
                 if (__any_sync(FULL, near)) {
@@ -536,7 +539,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 bool near = false;
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    uint32_t neg = 0;
+                    uint32_t on = 0;
                     float low = 0x1p127f;
 #pragma unroll
                     for (int k = 0; k < 16; k += 4) {
@@ -545,8 +548,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             float &z = zz[16 * q + k + j];
-                            const float v = z + b2, h = fmaxf(v, 0.0f);
-                            neg = __funnelshift_l(__float_as_uint(v), neg, 1);
+                            const float v = __fsub_rn(nb2, z), h = fmaxf(-v, 0.0f);   // v = -(z + b2), rounded alike
+                            on = __funnelshift_l(__float_as_uint(v), on, 1);
                             low = fminf(low, fabsf(v));
                             t3[0] = fmaf(h, d[0][j], t3[0]);
                             t3[1] = fmaf(h, d[1][j], t3[1]);
@@ -554,7 +557,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                             z = fmaf(d[2][j], w32, fmaf(d[1][j], w31, d[0][j] * w30));   // dH2
                         }
                     }
-                    m2[q] = neg;
+                    m2[q] = on;
                     near |= low < eps2 * S.gmax[4 * hc + 2 * half + q];
                 }
                 if (__any_sync(FULL, near)) {
