@@ -177,8 +177,8 @@ typedef struct {
      * (bounded) for MMAs it issued, releases its tensor memory, sets bit 1 of the workspace flag
      * word (dvgo_workspace_status then returns DVGO_ERR_DEVICE until the next forward) and returns;
      * the gradients or colours of that call are incomplete.  Range 0 .. 60,000,000.
-     * test_withhold_tile (testing aid, 0 in normal use): k > 0 makes one producer thread of the
-     * DVGO_MLP_BF16 colour kernels withhold its arrival on tile k - 1, so that the consumers' wait for that tile
+     * test_withhold_tile (testing aid, 0 in normal use): k > 0 makes one producer thread of
+     * those kernels withhold its arrival on tile k - 1, so that the consumers' wait for that tile
      * runs out -- the failure path above, taken on purpose. */
     int wait_limit_us;
     int test_withhold_tile;

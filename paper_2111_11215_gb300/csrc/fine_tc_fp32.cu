@@ -48,7 +48,7 @@ struct SplitDims {
 
 struct SplitSmall {
     float part[TM][3];   // the second half-row's share of the output layer
-    uint64_t full, empty, mma;
+    uint64_t full, empty, mma, fin;
     uint32_t tmem_base;
     int abort;
     float b3[4];
@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
         mbar_init(&S.full, NP);
         mbar_init(&S.empty, 1);
         mbar_init(&S.mma, 1);
+        mbar_init(&S.fin, 1);
         S.abort = 0;
     }
     if (warp == 0) tmem_alloc(&S.tmem_base, NCOLS);
@@ -147,7 +148,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                 for (int s = 0; s < 3; ++s) *split_chunk<KB>(xs, s, row, c) = q[s];
             }
             fence_async_smem();
-            mbar_arrive(&S.full);
+            // (testing aid: one arrival withheld on a chosen tile makes the consumers' wait run out)
+            if (!(row == 0 && tile + 1 == A.withhold_tile)) mbar_arrive(&S.full);
         }
         if (!ok) atomicExch(&S.abort, 1);
     } else {
@@ -190,11 +192,14 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
         const uint32_t idesc = idesc_bf16(128, 128, 0, 0);
         // the six products, smallest first: split of A, split of B
         constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};
-        auto wait_mma = [&]() -> bool {
-            const bool w = mbar_wait(&S.mma, mphase, A.wait_ns);
-            mphase ^= 1;
+        // waits of a warp as one; the verdicts of the warps meet at the last barrier of a tile (barrier_all)
+        auto wait = [&](uint64_t *bar, uint32_t par) {
+            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar, par, A.wait_ns));
             fence_after();
-            return w;
+        };
+        auto wait_mma = [&]() {
+            wait(&S.mma, mphase);
+            mphase ^= 1;
         };
         auto issue_layer1 = [&]() {
             const uint64_t x = desc_kmajor(smem_u32(xs), 0), w = desc_kmajor(smem_u32(w1t), 0);
@@ -206,10 +211,9 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
             commit(&S.mma);
         };
         int i = 0;
-        if (!mbar_wait(&S.full, 0, A.wait_ns)) ok = false;
-        fence_after();
+        wait(&S.full, 0);
         if (ok && tid == 0) issue_layer1();
-        for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++i) {
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
             // this row's sample slot and optical depth, needed at the end
             const int e = tile * TM + r;
             int slot = -1;
@@ -219,8 +223,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                 slot = kv.y * A.cap + (kv.x & 0xffff);
                 tau = __ldg(A.stau + slot);
             }
-            if (!wait_mma()) { ok = false; break; }
-            if (tid == 0) mbar_arrive(&S.empty);   // X is free
+            wait_mma();
+            if (ok && tid == 0) mbar_arrive(&S.empty);   // X is free
             // ---- epilogue 1: H1 = relu(Z1), split, over Z1 (read whole before any is overwritten) ----
             {
                 float z[2][32];
@@ -252,7 +256,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                 consumer_sync();
             }
             // ---- layer 2: Z2 = H1 W2, A = H1 from TMEM; inputs 0-63 and 64-127 in accumulators of their own ----
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 const uint64_t w = desc_kmajor(smem_u32(w2t), 0);
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
@@ -264,12 +268,11 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                                    w + 2 * PB[p] * kPanelStep + kstep(kk), idesc, p > 0 || kk > 4 * h);
                 commit(&S.mma);
             }
-            if (!wait_mma()) { ok = false; break; }
+            wait_mma();
             // ---- layer 1 of the next tile, beside the last epilogue ----
             if (tile + (int)gridDim.x < ntiles) {
-                if (!mbar_wait(&S.full, (i + 1) & 1, A.wait_ns)) { ok = false; break; }
-                fence_after();
-                if (tid == 0) issue_layer1();
+                wait(&S.full, (i + 1) & 1);
+                if (ok && tid == 0) issue_layer1();
             }
             // ---- epilogue 2: relu(Z2 + b2) W3, my 64 columns; the two halves of a row join ----
             float o[3] = {0.0f, 0.0f, 0.0f};
@@ -298,7 +301,10 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
                 S.part[r][1] = o[1];
                 S.part[r][2] = o[2];
             }
-            consumer_sync();
+            fence_before();
+            ok = barrier_all(1, NC, ok);
+            fence_after();
+            if (!ok) break;
             if (slot >= 0)
                 A.scol[slot] = make_float4(sigmoidf_(o[0] + S.part[r][0]), sigmoidf_(o[1] + S.part[r][1]),
                                            sigmoidf_(o[2] + S.part[r][2]), tau);
@@ -310,9 +316,11 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_fwd_split_kernel(Rende
     __syncthreads();
     fence_after();
     if (S.abort != 0) {
-        if (tid == 0) atomicOr(&A.hdr->flags, 2);
-        // an MMA batch whose completion timed out may still be running: wait (bounded) once more
-        if (tid < NC) mbar_wait(&S.mma, mphase ^ 1, A.wait_ns);
+        if (tid == 0) {
+            atomicOr(&A.hdr->flags, 2);
+            commit(&S.fin);   // MMAs may still be running: all that were issued are complete before TMEM is freed (bounded)
+            mbar_wait(&S.fin, 0, A.wait_ns);
+        }
     }
     fence_before();
     __syncthreads();

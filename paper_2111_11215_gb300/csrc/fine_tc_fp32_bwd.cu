@@ -55,7 +55,7 @@ struct BwdSmall {
     float4 de[TM][3];      // feature gradients of a tile
     float4 place[2][TM];
     ScatterTab tab[NP / 32];
-    uint64_t full, empty, mma_a, mma_b;
+    uint64_t full, empty, mma_a, mma_b, fin;
     uint32_t tmem_base;
     int abort;
     int s1max;             // largest absolute row sum of W1^T | b1 (float bits)
@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
         mbar_init(&S.empty, 1);
         mbar_init(&S.mma_a, 1);
         mbar_init(&S.mma_b, 1);
+        mbar_init(&S.fin, 1);
         S.abort = 0;
         S.s1max = 0;
     }
@@ -220,7 +221,6 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
     fence_after();
     bool ok = true;
     uint32_t pa = 0, pb = 0;   // phases of mma_a and mma_b
-    bool b_out = false;        // a batch on mma_b not waited for yet
 
     if (tid >= NC) {
         // ------------------------------- producers -------------------------------
@@ -317,7 +317,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             for (int o = 8; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(FULL, gm, o));
             if ((row & 15) == 0) S.gmax[row >> 4] = gm;
             fence_async_smem();
-            mbar_arrive(&S.full);
+            // (testing aid: one arrival withheld on a chosen tile makes the consumers' wait run out)
+            if (!(row == 0 && tile + 1 == A.withhold_tile)) mbar_arrive(&S.full);
             // de of the tile before is in place: written before the consumers' release that this thread
             // has just waited for
             if (i > 0) scatter_tile(t ^ 1);
@@ -385,18 +386,19 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
         const uint32_t id_z1 = idesc_bf16(128, 128, 0, 0), id_z2 = idesc_bf16(128, 128, 0, 1),
                        id_dh = idesc_bf16(128, 128, 1, 1);
         constexpr int PA[6] = {0, 2, 1, 0, 1, 0}, PB[6] = {2, 0, 1, 1, 0, 0};   // the six products, small first
-        auto wait_a = [&]() -> bool {
-            const bool w = mbar_wait(&S.mma_a, pa, A.wait_ns);
-            pa ^= 1;
+        // Waits of a warp as one.  The verdicts of the warps meet at the last barrier of a tile (barrier_all): until
+        // then a warp whose wait ran out keeps the others company at their barriers.
+        auto wait = [&](uint64_t *bar, uint32_t par) {
+            if (ok) ok = __all_sync(FULL, mbar_wait(bar, par, A.wait_ns));
             fence_after();
-            return w;
         };
-        auto wait_b = [&]() -> bool {
-            const bool w = mbar_wait(&S.mma_b, pb, A.wait_ns);
+        auto wait_a = [&]() {
+            wait(&S.mma_a, pa);
+            pa ^= 1;
+        };
+        auto wait_b = [&]() {
+            wait(&S.mma_b, pb);
             pb ^= 1;
-            b_out = false;
-            fence_after();
-            return w;
         };
         // MMA batches over a third of an activation held in the pool at b_ (thread 0).  Descriptors are a base
         // and steps of the address field (16-byte units), so that an MMA costs the issuing thread two adds.
@@ -445,9 +447,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
         for (int j = 0; j < 24; ++j) acc1[j] = 0.0f;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-            if (!mbar_wait(&S.full, 0, A.wait_ns)) { ok = false; break; }
-            fence_after();
-            if (tid == 0) {
+            wait(&S.full, 0);
+            if (ok && tid == 0) {
                 const uint64_t a = desc_kmajor(w1_, 0), b = desc_kmajor(pool_, 0);
 #pragma unroll
                 for (int p = 0; p < 6; ++p)
@@ -460,7 +461,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
                 for (int ch = 0; ch < 3; ++ch) ab3[ch] += S.dout[ch][n];
             }
-            if (!wait_a()) { ok = false; break; }
+            wait_a();
             // ---- epilogue 1: H1 = relu(Z1), split: TMEM (A of dW2), lo and mid into the pool ----
             // Which units are on (z > 0): 16 samples a word, sample k in bit 15 - k.  The sign of 0 - z is set just
             // there: not for a zero of either sign (a unit whose weights are all 0) nor for a NaN.
@@ -482,7 +483,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                     m1[2 * half + q] = on;
                     near |= low < eps1 * S.gmax[4 * hc + 2 * half + q];
                 }
-                if (__any_sync(FULL, near)) {
+                if (ok && __any_sync(FULL, near)) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const int k0 = 64 * hc + 32 * half + 16 * q;
@@ -510,24 +511,24 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             tmem_wait_st();
             publish();
             // ---- layer 2 ----
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 z2_batch(b0_, 0, true);
                 commit(&S.mma_a);
                 z2_batch(b1_, 1, false);
                 z2_batch(b1_, 0, false);
                 commit(&S.mma_b);
             }
-            b_out = true;
-            if (!wait_a()) { ok = false; break; }
+            wait_a();
             stage_hi(T_ACT);
             publish();
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 z2_batch(b0_, 2, false);
                 z2_batch(b0_, 1, false);
                 z2_batch(b0_, 0, false);
                 commit(&S.mma_a);
             }
-            if (!wait_b() || !wait_a()) { ok = false; break; }
+            wait_b();
+            wait_a();
             // ---- epilogue 2: dZ2, dW3, db2 (a tile's sums first, then the running ones) ----
             float t3[3] = {0.0f, 0.0f, 0.0f}, tb2 = 0.0f;
             // (dL/do of a sample is read once for both: a read of four samples' takes the load unit four clocks a
@@ -560,7 +561,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                     m2[q] = on;
                     near |= low < eps2 * S.gmax[4 * hc + 2 * half + q];
                 }
-                if (__any_sync(FULL, near)) {
+                if (ok && __any_sync(FULL, near)) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const int k0 = 64 * hc + 32 * half + 16 * q;
@@ -595,7 +596,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             for (int ch = 0; ch < 3; ++ch) a3[ch] += t3[ch];
             publish();
             // ---- dW2 and dH1 ----
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 dw2_batch(b0_, 0, true);
                 dh_batch(b0_, 0, true);
                 commit(&S.mma_a);
@@ -604,10 +605,10 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 dh_batch(b1_, 1, false);
                 dh_batch(b1_, 0, false);
             }
-            if (!wait_a()) { ok = false; break; }
+            wait_a();
             stage_hi(T_HI);
             publish();
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 dw2_batch(b0_, 2, false);
                 dw2_batch(b0_, 1, false);
                 dw2_batch(b0_, 0, false);
@@ -615,8 +616,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 dh_batch(b0_, 2, false);
                 dh_batch(b0_, 1, false);
             }
-            b_out = true;
-            if (!wait_b()) { ok = false; break; }
+            wait_b();
 #pragma unroll
             for (int g = 0; g < 4; ++g) {   // this tile's dW2, beside the MMAs of dH1
                 float v[16];
@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 for (int k = 0; k < 16; ++k) acc2[16 * g + k] += v[k];
             }
             consumer_sync();
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 // hi x hi last, units 0-63 on top of the small products, 64-127 in an accumulator of their own
                 // (dW2's, read by now)
                 const uint64_t a = desc_mnmajor(w2_, 0), b = desc_mnmajor(b0_, 0);
@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                     mma(tb + (kk < 4 ? T_Z : T_DW2), a + mnstep(kk), b + mnstep(kk), id_dh, kk != 4);
                 commit(&S.mma_a);
             }
-            if (!wait_a()) { ok = false; break; }
+            wait_a();
             // ---- epilogue 3: dZ1 = dH1 [Z1 > 0], split: TMEM (A of dW1), lo and mid into the pool ----
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
@@ -653,20 +653,20 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             tmem_wait_st();
             publish();
             // ---- de ----
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 de_batch(b1_, 3, true);    // the mid term (with all of W1's, so that it starts all three parts)
                 de_batch(b0_, 1, false);   // lo
                 commit(&S.mma_a);
             }
-            if (!wait_a()) { ok = false; break; }
+            wait_a();
             stage_hi(T_ACT);
             publish();
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 de_batch(b0_, 3, false);
                 commit(&S.mma_a);
             }
-            if (!wait_a()) { ok = false; break; }
-            if (tid == 0) mbar_arrive(&S.empty);   // the pool is free for X
+            wait_a();
+            if (ok && tid == 0) mbar_arrive(&S.empty);   // the pool is free for X
             float de[16];
             if (hc == 0) {   // lane = sample here
                 float d1[16], d2[16];
@@ -677,10 +677,9 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 for (int k = 0; k < FEAT; ++k) de[k] += d1[k] + d2[k];
             }
             // (X staged again: the producers are also done with the de of the tile before)
-            if (!mbar_wait(&S.full, 1, A.wait_ns)) { ok = false; break; }
-            fence_after();
+            wait(&S.full, 1);
             // ---- dW1, its three parts by X's terms side by side ----
-            if (tid == 0) {
+            if (ok && tid == 0) {
                 const uint64_t b = desc_mnmajor(pool_, 0);
                 const uint32_t id3 = idesc_bf16(128, 144, 0, 1), id1 = idesc_bf16(128, 48, 0, 1);
 #pragma unroll
@@ -696,7 +695,7 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
                 for (int k = 0; k < 3; ++k) S.de[n][k] = make_float4(de[4 * k], de[4 * k + 1], de[4 * k + 2], de[4 * k + 3]);
             }
-            if (!wait_a()) { ok = false; break; }
+            wait_a();
 #pragma unroll
             for (int g = 0; g < 3; ++g) {   // columns 24 hc + 8 g .. of the three parts
                 float v0[8], v1[8], v2[8];
@@ -706,7 +705,10 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
                 for (int k = 0; k < 8; ++k) acc1[8 * g + k] += v0[k] + (v1[k] + v2[k]);
             }
-            consumer_sync();   // de written, TMEM reads done
+            fence_before();
+            ok = barrier_all(1, NC, ok);   // de written, TMEM reads done
+            fence_after();
+            if (!ok) break;
             if (tid == 0) mbar_arrive(&S.empty);   // the tile is done
         }
         if (!ok) {
@@ -737,11 +739,10 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
     __syncthreads();
     fence_after();
     if (S.abort != 0) {
-        if (tid == 0) atomicOr(&A.hdr->flags, 2);
-        // an MMA batch whose completion timed out may still be running: wait (bounded) once more
-        if (tid < NC) {
-            mbar_wait(&S.mma_a, pa ^ 1, A.wait_ns);
-            if (b_out) mbar_wait(&S.mma_b, pb, A.wait_ns);
+        if (tid == 0) {
+            atomicOr(&A.hdr->flags, 2);
+            commit(&S.fin);   // MMAs may still be running: all that were issued are complete before TMEM is freed (bounded)
+            mbar_wait(&S.fin, 0, A.wait_ns);
         }
     }
     fence_before();

@@ -216,6 +216,22 @@ __device__ __forceinline__ bool mbar_test(uint64_t *mbar, uint32_t parity) {
     return done != 0;
 }
 
+// Barrier `id` of n threads (whole warps) that tells all of them whether ok held for every one.  Waits of a group of
+// warps run out one by one: a warp whose wait did goes on to the group's next such barrier without
+// waiting again or issuing anything, so that none is left alone at a barrier, which has no limit.
+__device__ __forceinline__ bool barrier_all(int id, int n, bool ok) {
+    uint32_t all;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %3, 0;\n\t"
+        "barrier.cta.red.and.pred p, %1, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(all)
+        : "r"(id), "r"(n), "r"((uint32_t)ok)
+        : "memory");
+    return all != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
