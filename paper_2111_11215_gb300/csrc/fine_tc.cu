@@ -107,6 +107,7 @@ struct alignas(1024) SmallTC {
     float dc[2][TM][3];       // dL/dc (backward)
     uint64_t full[2], empty[2];
     uint64_t mma[2];          // forward: the MMAs of consumer group 0 / 1
+    uint64_t stop[2];         // forward: all MMAs of a group that gave up
     // backward.  xl: the bulk load of X panel b from the forward's copy; z1, z2, dh, de: MMA batches
     // complete; ev[e]: consumers have finished epilogue e; fin: every MMA of the launch complete; sc: the
     // de of a tile of X buffer b has been scattered
@@ -225,6 +226,8 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         mbar_init(&S.sm.empty[1], BWD ? 4 : 1);
         mbar_init(&S.sm.mma[0], 1);
         mbar_init(&S.sm.mma[1], 1);
+        mbar_init(&S.sm.stop[0], 1);
+        mbar_init(&S.sm.stop[1], 1);
         if (BWD) {
             mbar_init(&S.sm.xl[0], 1);
             mbar_init(&S.sm.xl[1], 1);
@@ -376,11 +379,14 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
         const uint32_t tb = S.sm.tmem_base + 256u * (uint32_t)grp;
         uint64_t *mbar = &S.sm.mma[grp];
         uint32_t mphase = 0;
-        auto wait_mma = [&]() -> bool {
-            bool w = mbar_wait(mbar, mphase, A.wait_ns);
-            mphase ^= 1;
+        // waits of a warp as one; the verdicts of a group's warps meet at its last barrier of a tile (barrier_all)
+        auto wait = [&](uint64_t *bar, uint32_t par) {
+            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar, par, A.wait_ns));
             fence_after();
-            return w;
+        };
+        auto wait_mma = [&]() {
+            wait(mbar, mphase);
+            mphase ^= 1;
         };
         auto group_sync = [&]() {
             fence_before();
@@ -393,16 +399,19 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             const int b = grp;
             uint32_t x_ = smem_u32(S.x[b]), w1t_ = smem_u32(S.w1t), w2t_ = smem_u32(S.w2t), w3p_ = smem_u32(S.tp);
             asm volatile("" : "+r"(x_), "+r"(w1t_), "+r"(w2t_), "+r"(w3p_));
-            // (no abort-flag test here: two warps of a group could read it on either side of its
-            // setting and part at the group barrier; a failed producer instead leaves this wait
-            // unsatisfied for every thread of the group alike)
-            if (!mbar_wait(&S.sm.full[b], (i >> 1) & 1, A.wait_ns)) ok = false;
-            fence_after();
-            if (!ok) break;
+            // (no abort-flag test here: the group's warps could read it on either side of its setting; a failed
+            // producer leaves this wait unsatisfied for every thread of the group)
+            wait(&S.sm.full[b], (i >> 1) & 1);
+            if (!ok) {   // (the table may hold nothing yet)
+                group_sync();
+                group_sync();
+                barrier_all(2 + grp, TM, false);
+                break;
+            }
             const int slot = S.sm.slot[i & 3][r];
             const float tau = slot >= 0 ? __ldg(A.stau + slot) : 0.0f;   // goes with the colour
             // ---- layer 1: Z1 = X W1 ----
-            if (r == 0) {
+            if (ok && r == 0) {
 #pragma unroll 1
                 for (int kk = 0; kk < 4; ++kk)
                     mma(tb + COL_Z1, desc_kmajor(x_, kk), desc_kmajor(w1t_, kk), idesc_bf16(128, 128, 0, 0), kk > 0);
@@ -411,8 +420,8 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
                 commit(mbar);
                 if (A.xcache) bulk_store(A.xcache + (size_t)tile * kPanelBytes, S.x[b], kPanelBytes);   // for the backward
             }
-            if (!wait_mma()) { ok = false; break; }
-            if (r == 0) {   // X[b] is free once layer 1 and the copy have read it
+            wait_mma();
+            if (ok && r == 0) {   // X[b] is free once layer 1 and the copy have read it
                 if (A.xcache) bulk_wait_read();
                 mbar_arrive(&S.sm.empty[b]);
             }
@@ -430,14 +439,14 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             tmem_wait_st();
             group_sync();
             // ---- layer 2: Z2 = H1 W2, A = H1 from TMEM ----
-            if (r == 0) {
+            if (ok && r == 0) {
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     mma_ts(tb + F_Z2, tb + F_H1 + 8u * (uint32_t)kk, desc_kmajor(w2t_, kk), idesc_bf16(128, 128, 0, 0),
                            kk > 0);
                 commit(mbar);
             }
-            if (!wait_mma()) { ok = false; break; }
+            wait_mma();
             // ---- epilogue 2: H2 = relu(Z2 + b2), as BF16 into TMEM ----
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
@@ -455,20 +464,23 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
             tmem_wait_st();
             group_sync();
             // ---- layer 3: O = H2 W3 (N = 16, columns 0-2 used), A = H2 from TMEM ----
-            if (r == 0) {
+            if (ok && r == 0) {
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     mma_ts(tb + F_O, tb + F_H2 + 8u * (uint32_t)kk, desc_mnmajor(w3p_, kk), idesc_bf16(128, 16, 0, 1),
                            kk > 0);
                 commit(mbar);
             }
-            if (!wait_mma()) { ok = false; break; }
+            wait_mma();
             float o[16];
             tmem_ld16(taddr(tb, warp, F_O), o);
-            if (slot >= 0)
+            if (ok && slot >= 0)
                 A.scol[slot] = make_float4(sigmoidf_(o[0] + S.sm.b3[0]), sigmoidf_(o[1] + S.sm.b3[1]),
                                            sigmoidf_(o[2] + S.sm.b3[2]), tau);
-            group_sync();   // TMEM reads and panel reads done before this group's next MMAs
+            fence_before();
+            ok = barrier_all(2 + grp, TM, ok);   // TMEM and panel reads done before this group's next MMAs
+            fence_after();
+            if (!ok) break;
         }
         if (r == 0 && A.xcache) bulk_wait_all();   // the copies are complete before the kernel ends
         if (!ok) atomicExch(&S.sm.abort, 1);
@@ -700,8 +712,11 @@ __global__ void __launch_bounds__(kThreads<BWD>, 1) fine_colour_tc_kernel(Render
     const bool failed = S.sm.abort != 0;
     if (failed) {
         if (tid == 0) atomicOr(&A.hdr->flags, 2);
-        // an MMA batch whose completion timed out may still be running: wait (bounded) once more
-        if (!BWD && tid < NC) mbar_wait(&S.sm.mma[tid / TM], 0, A.wait_ns);
+        // forward: MMAs may still be running: all that were issued are complete before TMEM is freed (bounded)
+        if (!BWD && (tid == 0 || tid == TM)) {
+            commit(&S.sm.stop[tid / TM]);
+            mbar_wait(&S.sm.stop[tid / TM], 0, A.wait_ns);
+        }
     }
     if (BWD && !failed && tid < NC && ntile_mine > 0) {
         const uint32_t tb = S.sm.tmem_base;
