@@ -224,7 +224,10 @@ typedef struct {
 /* Bytes of workspace that dvgo_render_fwd / dvgo_render_bwd need for n_rays rays.  The bound
  * covers the longest possible ray: ceil(|xyz_max - xyz_min| / step) + 1 samples.  The fine stage
  * with DVGO_MLP_BF16 adds 16 KiB per 128 samples unless p->forward_only: the tensor-core forward
- * keeps every tile's BF16 MLP input rows there for the backward. */
+ * keeps every tile's BF16 MLP input rows there for the backward.  With 0 < tau_f < 1 the fine stage's
+ * size includes one bit per lattice cell for batches of many uniform samples, in which the density
+ * pass marks the cells that cannot reach tau_f; a workspace sized with tau_f = 0 is accepted too, and the
+ * results are the same (the pass then looks at every sample). */
 size_t dvgo_workspace_size(const dvgo_params *p, const dvgo_grid_desc *density, int n_rays,
                            const dvgo_samples *explicit_samples);
 

@@ -243,8 +243,10 @@ RenderArgs make_args(const dvgo_params *p, const dvgo_grid_desc *dd, const float
     return A;
 }
 
-int check_ws(const WsLayout &L, void *ws, size_t bytes) {
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 || bytes < L.total) return DVGO_ERR_WORKSPACE;
+// A workspace without room for the cell mask (sized for another tau_f) is rendered in without it.
+int check_ws(WsLayout &L, void *ws, size_t bytes) {
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 || bytes < L.need) return DVGO_ERR_WORKSPACE;
+    if (bytes < L.total) L.mask = 0;
     return DVGO_OK;
 }
 

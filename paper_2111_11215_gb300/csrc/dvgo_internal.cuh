@@ -75,8 +75,8 @@ static_assert(sizeof(WsHeader) == 256, "WsHeader size");
 
 // Workspace layout; every block 256-byte aligned.
 struct WsLayout {
-    size_t header, rays, rayout, rtarget, pe, texit, rayk, rchunk, stau, scol, sgrad, kept, mask, xcache, total;
-                                 // mask, xcache 0: none
+    size_t header, rays, rayout, rtarget, pe, texit, rayk, rchunk, stau, scol, sgrad, kept, mask, xcache, need, total;
+                                 // mask, xcache 0: none; need: total without the mask, which comes last
     long long max_samples;
 };
 
@@ -457,7 +457,7 @@ __device__ __forceinline__ float seg_sum(float v, const Seg &s, int lane) {
 // Host-side launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------------------------
 
-// mask_words, xcache: add the blocks of the cell mask and of the BF16 colour kernels' X panels (fine
+// mask_words, xcache: add the blocks of the BF16 colour kernels' X panels and of the cell mask (fine
 // mode), after all others so that the other offsets do not depend on them.
 WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache = false, size_t mask_words = 0);
 void launch_ray_setup(const RenderArgs &A, const float *rays_o, const float *rays_d, const float *jitter,

@@ -548,7 +548,9 @@ int dvgo_weight_bins(const dvgo_params *p, const dvgo_grid_desc *dd, int n_rays,
     if (p->mode != DVGO_MODE_FINE || !(p->step > 0.0f)) return DVGO_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return DVGO_ERR_WORKSPACE;
     if (n_rays == 0) return DVGO_OK;
-    const size_t need = dvgo_workspace_size(p, dd, n_rays, nullptr);
+    dvgo_params q = *p;
+    q.tau_f = 0.0f;   // (what a render with tau_f cannot do without)
+    const size_t need = dvgo_workspace_size(&q, dd, n_rays, nullptr);
     if (need == 0) return DVGO_ERR_INVALID_ARG;
     if (ws_bytes < need) return DVGO_ERR_WORKSPACE;
     double diag2 = 0.0;

@@ -145,12 +145,13 @@ WsLayout ws_layout(int R, long long max_samples, int mode, bool xcache, size_t m
     // last; counted in total, so the allocation-free forward's static scratch includes it even
     // though that forward (no auxiliary losses) never writes it
     L.rtarget = o; o += up(sizeof(float4) * n);
-    if (mask_words > 0 && mode == DVGO_MODE_FINE) { L.mask = o; o += up(sizeof(unsigned) * mask_words); }
     if (xcache && mode == DVGO_MODE_FINE) {   // 128 kept samples per tile, a 16 KiB panel each
         o = (o + 1023) & ~(size_t)1023;
         L.xcache = o;
         o += (size_t)16384 * ((S + 127) / 128);
     }
+    L.need = o;
+    if (mask_words > 0 && mode == DVGO_MODE_FINE) { o = up(o); L.mask = o; o += up(sizeof(unsigned) * mask_words); }
     L.total = o;
     L.max_samples = max_samples;
     return L;
