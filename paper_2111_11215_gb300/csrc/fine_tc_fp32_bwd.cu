@@ -5,7 +5,12 @@
 // contraction the six products that matter with FP32 accumulation, the smallest first.  Weight
 // gradients leave their TMEM accumulator after every tile and are summed over the tiles in registers, with
 // rounding (an accumulator that lived through all tiles would lose a part in 10^4 to the tensor core's
-// truncation).  A ReLU unit within rounding of zero is decided by the plain FP32 FMA chain over its inputs
+// truncation).  Within a tile the same truncation cuts every product off at the last bit of the running sum,
+// always towards 0: with one accumulator of 128 samples for hi x hi, dW1 and dW2 were 2e-6 off where an FP32
+// chain is 4e-7 off (samples of a proposal, weights over many orders of magnitude).  So hi x hi of dW1 and
+// dW2 goes to four accumulators of 32 samples, that of dH1 and de to two of 64 units; they join with rounding.
+// Errors against FP64 over 40 drawn steps, relative to the CUDA-core kernel's: MLP gradients 0.70, feature
+// gradients 0.87 (geometric means).  A ReLU unit within rounding of zero is decided by the plain FP32 FMA chain over its inputs
 // (exact_z1 / exact_z2, the order of the SIMT kernel), so the gradients do not hang on which
 // arithmetic recomputed the hidden layers.
 //
@@ -25,12 +30,13 @@
 //   dH1^T = W2 dZ2^T                A = W2 (shared, read MN-major), B = dZ2^T
 //   dZ1 = dH1 [Z1 > 0]
 //   de = dZ1 W1[0:12]^T             A = dZ1^T (shared, read MN-major), B = W1 (read MN-major)
-//   [dW1 | db1]^T += dZ1^T X        A = dZ1^T (TMEM), B = X (staged again; its three terms side by side)
-// Shared memory: W2 split 96 KB, W1 split 48 KB, and a pool of 64 KB that holds X (48 KB), then pairs of
+//   [dW1 | db1]^T += dZ1^T X        A = dZ1^T (TMEM), B = X (staged again; mid | lo and hi | mid side by side)
+// Shared memory: W2 split 96 KB, W1 split 48 KB, and a pool of 64 KB that holds X, then pairs of
 // 32 KB thirds of the activations, then X again.  Warps 0-7 consume (thread (n, half): unit n = t mod 128,
 // samples 64 half .. +63), warps 8-11 gather X, stage it twice and scatter the feature gradients of the
-// tile before.  TMEM columns: activations' split [0, 192); layer accumulator [192, 320); dW2, then the second
-// half of dH1 [320, 448); dW1 [192, 336) over both; dZ2's hi third, then de [448, 512).
+// tile before.  TMEM columns: activations' split [0, 192); layer accumulator [192, 320); dW2 [320, 448) and, over
+// H1's mid and lo thirds, [64, 192), then the second half of dH1 [320, 448); dZ2's hi third, then de [448, 512) and
+// [400, 448); dW1's six accumulators [192, 480) over them.
 
 #include "dvgo_internal.cuh"
 #include "fine_gather.cuh"
@@ -46,7 +52,8 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int TM = 128, NC = 256, NP = 128;
 constexpr int HID = 128, FEAT = 12, IN = 39, XK = 40;   // column IN of X is the constant 1 (bias)
 constexpr int KB = 3;                                   // 16-column blocks of X and W1 per split
-constexpr uint32_t T_ACT = 0, T_Z = 192, T_DW2 = 320, T_DW1 = 192, T_DE = 448, T_HI = 448, NCOLS = 512;
+constexpr uint32_t T_ACT = 0, T_DW2B = 64, T_Z = 192, T_DW2 = 320, T_DW1 = 192, T_DE = 448, T_DE2 = 400, T_HI = 448, NCOLS = 512;
+constexpr int DW1 = 16 * KB;                            // columns of a dW1 accumulator
 
 struct BwdSmall {
     alignas(16) float dout[3][TM];   // dL/do
@@ -286,12 +293,17 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
 #pragma unroll
             for (int c8 = 0; c8 < XK / 8; ++c8) split8(v + 8 * c8, w.q[c8]);
         };
+        // the terms side by side, 48 columns each: mid, lo from the first panel's start, hi, mid from the third's
         auto stage = [&](const Row &w) {
 #pragma unroll
-            for (int c = 0; c < 2 * KB; ++c)
-#pragma unroll
-                for (int s = 0; s < 3; ++s)
-                    *split_chunk<KB>(pool, s, row, c) = c < XK / 8 ? w.q[c][s] : make_uint4(0u, 0u, 0u, 0u);
+            for (int c = 0; c < 2 * KB; ++c) {
+                const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+                const uint4 hi = c < XK / 8 ? w.q[c][0] : z, mid = c < XK / 8 ? w.q[c][1] : z, lo = c < XK / 8 ? w.q[c][2] : z;
+                *split_chunk<KB>(pool, 0, row, c) = mid;
+                *split_chunk<KB>(pool, 1, row, c) = lo;
+                *split_chunk<KB>(pool + 2 * kPanelBytes, 0, row, c) = hi;
+                *split_chunk<KB>(pool + 2 * kPanelBytes, 1, row, c) = mid;
+            }
         };
         auto scatter_tile = [&](int t) {
             scatter_rows<PK>(A, S.place[t], [&](int r, int k) { return &S.de[r][k]; }, S.tab[row >> 5], row);
@@ -419,13 +431,24 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             for (int kk = 0; kk < 8; ++kk)
                 mma_ts(tb + T_DW2, tb + T_ACT + 64u * sa + 8u * kk, b + kstep(kk), id_z1, !first || kk > 0);
         };
+        // hi x hi of dW2, k-steps 4 r .. + 3 (dZ2's hi third in b0): two to an accumulator
+        auto dw2_hi = [&](int r) {
+            const uint64_t b = desc_kmajor(b0_, 0);
+#pragma unroll
+            for (int kk = 4 * r; kk < 4 * r + 4; ++kk)
+                mma_ts(tb + (kk & 2 ? T_DW2B : T_DW2), tb + T_ACT + 8u * kk, b + kstep(kk), id_z1,
+                       (kk & 1) || (r == 0 && !(kk & 2)));
+            commit(&S.mma_b);
+        };
         // [de hi | de mid | de lo] (+)= dZ1 [W1 hi | W1 mid | W1 lo]^T, the first `terms` of W1 (16 columns each; an
-        // MMA this narrow costs the same for 16 columns as for 48).  The three parts join in FP32.
-        auto de_batch = [&](uint32_t b_, int terms, bool first) {
+        // MMA this narrow costs the same for 16 columns as for 48).  The three parts join in FP32; of dZ1's hi third,
+        // which comes last, units 64-127 go to an accumulator of their own.
+        auto de_batch = [&](uint32_t b_, int terms, bool first, bool hi) {
             const uint64_t a = desc_mnmajor(b_, 0), b = desc_mnmajor(w1_ + 2 * kPanelBytes + 32u, 0);
             const uint32_t id = idesc_bf16(128, 16 * terms, 1, 1);
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) mma(tb + T_DE, a + mnstep(kk), b + mnstep(kk), id, !first || kk > 0);
+            for (int kk = 0; kk < 8; ++kk)
+                mma(tb + (hi && kk >= 4 ? T_DE2 : T_DE), a + mnstep(kk), b + mnstep(kk), id, hi ? kk != 4 : (!first || kk > 0));
         };
         // copies a hi third from TMEM columns `from` into the pool's first buffer
         auto stage_hi = [&](uint32_t from) {
@@ -454,7 +477,8 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 for (int p = 0; p < 6; ++p)
 #pragma unroll
                     for (int kk = 0; kk < KB; ++kk)
-                        mma(tb + T_Z, a + kstep(PA[p] * KB + kk), b + kstep(PB[p] * KB + kk), id_z1, (p | kk) != 0);
+                        mma(tb + T_Z, a + kstep(PA[p] * KB + kk), b + (PB[p] == 0 ? 2 * kPanelStep : 0) + kstep((PB[p] == 2 ? KB : 0) + kk),
+                            id_z1, (p | kk) != 0);
                 commit(&S.mma_a);
             }
             if (hc == 0) {
@@ -579,10 +603,9 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                     const int g = 2 * half + q;
                     float z[16];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        z[k] = off(m2[q], k) ? 0.0f : zz[16 * q + k];
-                        tb2 += z[k];
-                    }
+                    for (int k = 0; k < 16; ++k) z[k] = off(m2[q], k) ? 0.0f : zz[16 * q + k];
+#pragma unroll
+                    for (int k = 0; k < 16; k += 4) tb2 += (z[k] + z[k + 1]) + (z[k + 2] + z[k + 3]);
                     uint32_t w[3][8];
                     split16(z, w);
                     store16(buf0, n, g, w[2]);
@@ -603,7 +626,6 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 dw2_batch(b1_, 1, false);
                 dw2_batch(b1_, 0, false);
                 dh_batch(b1_, 1, false);
-                dh_batch(b1_, 0, false);
             }
             wait_a();
             stage_hi(T_HI);
@@ -611,28 +633,38 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             if (ok && tid == 0) {
                 dw2_batch(b0_, 2, false);
                 dw2_batch(b0_, 1, false);
-                dw2_batch(b0_, 0, false);
                 commit(&S.mma_b);
-                dh_batch(b0_, 2, false);
-                dh_batch(b0_, 1, false);
+                dh_batch(b1_, 0, false);
             }
-            wait_b();
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {   // this tile's dW2, beside the MMAs of dH1
-                float v[16];
-                tmem_ld16(taddr(tb, warp, T_DW2 + 64 * hc + 16 * g), v);
-#pragma unroll
-                for (int k = 0; k < 16; ++k) acc2[16 * g + k] += v[k];
-            }
-            consumer_sync();
+            wait_b();   // H1's mid and lo thirds have been read: room for a second accumulator of dW2
             if (ok && tid == 0) {
-                // hi x hi last, units 0-63 on top of the small products, 64-127 in an accumulator of their own
-                // (dW2's, read by now)
-                const uint64_t a = desc_mnmajor(w2_, 0), b = desc_mnmajor(b0_, 0);
+                dw2_hi(0);
+                dh_batch(b0_, 2, false);
+            }
+            // hi x hi of dH1 last: units 0-63 on top of the small products, 64-127 in an accumulator of their own
+            // (dW2's, read by then)
+            const uint64_t dh_a = desc_mnmajor(w2_, 0), dh_b = desc_mnmajor(b0_, 0);
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    mma(tb + (kk < 4 ? T_Z : T_DW2), a + mnstep(kk), b + mnstep(kk), id_dh, kk != 4);
-                commit(&S.mma_a);
+            for (int r = 0; r < 2; ++r) {   // this tile's dW2, beside the MMAs of dH1
+                wait_b();
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    float v[16], u[16];
+                    tmem_ld16x2(taddr(tb, warp, T_DW2 + 64 * hc + 16 * g), v, taddr(tb, warp, T_DW2B + 64 * hc + 16 * g), u);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) acc2[16 * g + k] += v[k] + u[k];
+                }
+                consumer_sync();
+                if (ok && tid == 0) {
+                    if (r == 0) {
+                        dw2_hi(1);
+                        dh_batch(b0_, 1, false);
+                    }
+#pragma unroll
+                    for (int kk = 4 * r; kk < 4 * r + 4; ++kk)
+                        mma(tb + (r == 0 ? T_Z : T_DW2), dh_a + mnstep(kk), dh_b + mnstep(kk), id_dh, kk != 4);
+                    if (r == 1) commit(&S.mma_a);
+                }
             }
             wait_a();
             // ---- epilogue 3: dZ1 = dH1 [Z1 > 0], split: TMEM (A of dW1), lo and mid into the pool ----
@@ -654,15 +686,15 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             publish();
             // ---- de ----
             if (ok && tid == 0) {
-                de_batch(b1_, 3, true);    // the mid term (with all of W1's, so that it starts all three parts)
-                de_batch(b0_, 1, false);   // lo
+                de_batch(b1_, 3, true, false);    // the mid term (with all of W1's, so that it starts all three parts)
+                de_batch(b0_, 1, false, false);   // lo
                 commit(&S.mma_a);
             }
             wait_a();
             stage_hi(T_ACT);
             publish();
             if (ok && tid == 0) {
-                de_batch(b0_, 3, false);
+                de_batch(b0_, 3, false, true);
                 commit(&S.mma_a);
             }
             wait_a();
@@ -670,25 +702,34 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
             float de[16];
             if (hc == 0) {   // lane = sample here
                 float d1[16], d2[16];
-                tmem_ld16(taddr(tb, warp, T_DE + 16), d1);
-                tmem_ld16(taddr(tb, warp, T_DE + 32), d2);
-                tmem_ld16(taddr(tb, warp, T_DE), de);
+                tmem_ld16x2(taddr(tb, warp, T_DE + 16), d1, taddr(tb, warp, T_DE2 + 16), d2);
+#pragma unroll
+                for (int k = 0; k < FEAT; ++k) de[k] = d1[k] + d2[k];
+                tmem_ld16x2(taddr(tb, warp, T_DE + 32), d1, taddr(tb, warp, T_DE2 + 32), d2);
 #pragma unroll
                 for (int k = 0; k < FEAT; ++k) de[k] += d1[k] + d2[k];
+                tmem_ld16x2(taddr(tb, warp, T_DE), d1, taddr(tb, warp, T_DE2), d2);
+#pragma unroll
+                for (int k = 0; k < FEAT; ++k) de[k] += d1[k] + d2[k];
+                fence_before();
+                asm volatile("bar.sync 2, 128;" ::: "memory");   // (dW1's accumulators take these columns)
+                fence_after();
             }
             // (X staged again: the producers are also done with the de of the tile before)
             wait(&S.full, 1);
-            // ---- dW1, its three parts by X's terms side by side ----
+            // ---- dW1: the small products in two accumulators side by side, hi x hi in four of its own ----
             if (ok && tid == 0) {
-                const uint64_t b = desc_mnmajor(pool_, 0);
-                const uint32_t id3 = idesc_bf16(128, 144, 0, 1), id1 = idesc_bf16(128, 48, 0, 1);
+                const uint64_t ml = desc_mnmajor(pool_, 0), hm = desc_mnmajor(pool_ + 2 * kPanelBytes, 0);
+                const uint32_t id = idesc_bf16(128, DW1, 0, 1), id2 = idesc_bf16(128, 2 * DW1, 0, 1);
 #pragma unroll
-                for (int p = 0; p < 3; ++p) {   // dZ1's mid (starting all parts), lo, hi
-                    const int sa = p == 0 ? 1 : (p == 1 ? 2 : 0);
+                for (int kk = 0; kk < 8; ++kk) mma_ts(tb + T_DW1, tb + T_ACT + 8u * kk, ml + mnstep(kk), id2, kk != 0);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_ts(tb + T_DW1, tb + T_ACT + 64u * sa + 8u * kk, b + mnstep(kk), p == 1 ? id1 : id3, (p | kk) != 0);
-                }
+                for (int kk = 0; kk < 8; ++kk) mma_ts(tb + T_DW1, tb + T_ACT + 64u + 8u * kk, hm + mnstep(kk), id2, 1u);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) mma_ts(tb + T_DW1 + DW1, tb + T_ACT + 128u + 8u * kk, hm + mnstep(kk), id, 1u);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    mma_ts(tb + T_DW1 + DW1 * (2 + kk / 2), tb + T_ACT + 8u * kk, hm + mnstep(kk), id, kk & 1);
                 commit(&S.mma_a);
             }
             if (hc == 0) {
@@ -696,14 +737,18 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 for (int k = 0; k < 3; ++k) S.de[n][k] = make_float4(de[4 * k], de[4 * k + 1], de[4 * k + 2], de[4 * k + 3]);
             }
             wait_a();
+            {   // columns 24 hc ..
+                float t[24], v[24];
+                const uint32_t from = taddr(tb, warp, T_DW1 + 24 * hc);
+                tmem_ld24(from, t);
 #pragma unroll
-            for (int g = 0; g < 3; ++g) {   // columns 24 hc + 8 g .. of the three parts
-                float v0[8], v1[8], v2[8];
-                tmem_ld8(taddr(tb, warp, T_DW1 + 24 * hc + 8 * g), v0);
-                tmem_ld8(taddr(tb, warp, T_DW1 + 48 + 24 * hc + 8 * g), v1);
-                tmem_ld8(taddr(tb, warp, T_DW1 + 96 + 24 * hc + 8 * g), v2);
+                for (int q = 1; q < 6; ++q) {
+                    tmem_ld24(from + DW1 * q, v);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) acc1[8 * g + k] += v0[k] + (v1[k] + v2[k]);
+                    for (int k = 0; k < 24; ++k) t[k] += v[k];
+                }
+#pragma unroll
+                for (int k = 0; k < 24; ++k) acc1[k] += t[k];
             }
             fence_before();
             ok = barrier_all(1, NC, ok);   // de written, TMEM reads done
@@ -726,12 +771,25 @@ __global__ void __launch_bounds__(NC + NP, 1) fine_colour_bwd_split_kernel(Rende
                 else if (c == IN) atomicAdd(gB1 + n, acc1[j]);
             }
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) {
-                atomicAdd(gW3 + 3 * n + ch, a3[ch]);
-                const float s = warp_sum(ab3[ch]);
-                if (hc == 0 && lane == 0) atomicAdd(gB3 + ch, s);
+            for (int ch = 0; ch < 3; ++ch) ab3[ch] = warp_sum(ab3[ch]);
+            // one sum a CTA: the halves of a unit and the warps of db3 join in the pool, which is free
+            float4 *half = reinterpret_cast<float4 *>(pool), *rows = half + HID;
+            if (hc == 1) half[n] = make_float4(a3[0], a3[1], a3[2], ab2);
+            if (lane == 0 && warp > 0 && hc == 0) rows[warp] = make_float4(ab3[0], ab3[1], ab3[2], 0.0f);
+            consumer_sync();
+            if (hc == 0) {
+                const float4 o = half[n];
+                atomicAdd(gW3 + 3 * n, a3[0] + o.x);
+                atomicAdd(gW3 + 3 * n + 1, a3[1] + o.y);
+                atomicAdd(gW3 + 3 * n + 2, a3[2] + o.z);
+                atomicAdd(gB2 + n, ab2 + o.w);
             }
-            atomicAdd(gB2 + n, ab2);
+            if (tid == 0) {
+                const float4 r1 = rows[1], r2 = rows[2], r3 = rows[3];
+                atomicAdd(gB3, (ab3[0] + r1.x) + (r2.x + r3.x));
+                atomicAdd(gB3 + 1, (ab3[1] + r1.y) + (r2.y + r3.y));
+                atomicAdd(gB3 + 2, (ab3[2] + r1.z) + (r2.z + r3.z));
+            }
         }
     }
 
