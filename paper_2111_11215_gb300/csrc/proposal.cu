@@ -199,14 +199,35 @@ __device__ __forceinline__ void weight_grad(const float *HT, const float *DT, fl
     }
 }
 
-// sin / cos of the double-float argument a (|a| below a few hundred), reduced by 2 pi in double-float
-// arithmetic (2 pi = 6.28318548... - 1.7484556e-7, to 2^-47) and evaluated in FP32.  The reduction in FP64,
-// 18 per row, had the FP64 pipe busy for 17 us a tile.
+// sin / cos of the double-float argument a, reduced by 2 pi in double-float arithmetic (2 pi = 6.28318548... -
+// 1.7484556e-7) and evaluated in FP32.  The argument and its reduction are each off by up to 2^-47 of what they are
+// formed from, which is far below an FP32 rounding of the result up to kDfReach; beyond it encode_row_fp64.  The
+// reduction in FP64, 18 per row, had the FP64 pipe busy for 17 us a tile.
 __device__ __forceinline__ void sincos_reduced(Df a, float *s, float *c) {
     const Df two_pi = {6.283185482025146484375f, -1.74845553146951715e-7f};
     const float n = rintf(a.hi * 0.15915494f);
     const Df red = df_add(a, df_neg(df_mul_f(two_pi, n)));
     sincosf(red.hi, s, c);
+}
+
+// The same part of an input row with positions and argument reductions in FP64, for rays that reach further
+// out than kDfReach.
+__device__ __noinline__ void encode_row_fp64(const PropArgs &P, int r, int bin, int part, int row, float *xt) {
+    const Clip c = clip_ray(P.box, P.ro, P.rd, r);
+    const double tb = __dadd_rn(c.lo, __ddiv_rn(__dmul_rn((double)bin + 0.5, __dsub_rn(c.hi, c.lo)), (double)NB));
+    const double two_pi = 6.283185307179586;
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        const double x = __dadd_rn((double)P.ro[3 * r + a], __dmul_rn(tb, c.dn[a]));
+        if (part == 0) xt[a * PLD + row] = (float)x;
+        for (int k = 3 * part; k < 3 * part + 3; ++k) {
+            const double arg = ldexp(x, k);
+            float sv, cv;
+            sincosf((float)fma(-rint(arg / two_pi), two_pi, arg), &sv, &cv);
+            xt[(3 + a * NFQ + k) * PLD + row] = sv;
+            xt[(3 + 3 * NFQ + a * NFQ + k) * PLD + row] = cv;
+        }
+    }
 }
 
 template <bool BWD>
@@ -262,23 +283,26 @@ __global__ void __launch_bounds__(PNT, 1) proposal_kernel(PropArgs P) {
 #pragma unroll
                 for (int a = 0; a < 3; ++a) x[a] = bin_position(cl, tb, a);
             }
-            if (part == 0) {
+            if (part == 0) S.xt[PIN * PLD + row] = 1.0f;
+            // part 0: positions and k = 0..2, part 1: k = 3..5 for every axis
+            if (cl.hit & 2) {
+                encode_row_fp64(P, 2 * tile + (row >> 6), row & 63, part, row, S.xt);
+            } else {
+                if (part == 0)
 #pragma unroll
-                for (int a = 0; a < 3; ++a) S.xt[a * PLD + row] = x[a].hi;
-                S.xt[PIN * PLD + row] = 1.0f;
+                    for (int a = 0; a < 3; ++a) S.xt[a * PLD + row] = x[a].hi;
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int kk = 0; kk < 3; ++kk) {
+                        const int k = 3 * part + kk;
+                        const float p2 = (float)(1 << k);
+                        float sv, cv;
+                        sincos_reduced(Df{x[a].hi * p2, x[a].lo * p2}, &sv, &cv);
+                        S.xt[(3 + a * NFQ + k) * PLD + row] = sv;
+                        S.xt[(3 + 3 * NFQ + a * NFQ + k) * PLD + row] = cv;
+                    }
             }
-            // part 0: k = 0..2, part 1: k = 3..5 for every axis
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk) {
-                    const int k = 3 * part + kk;
-                    const float p2 = (float)(1 << k);
-                    float sv, cv;
-                    sincos_reduced(Df{x[a].hi * p2, x[a].lo * p2}, &sv, &cv);
-                    S.xt[(3 + a * NFQ + k) * PLD + row] = sv;
-                    S.xt[(3 + 3 * NFQ + a * NFQ + k) * PLD + row] = cv;
-                }
         }
         __syncthreads();
         float acc[4][8];

@@ -13,8 +13,11 @@ constexpr int kPropBins = 64;
 struct ClipDf {
     Df t0, w, dn[3];
     float o[3];
-    int hit;
+    int hit;        // 0; 1; 3: and its origin or exit lies further out than kDfReach
 };
+// Coordinates and distances up to which double-float positions do for the FP32 network: 2^5 x 2^12 x 2^-47 =
+// 2^-30 in an encoded argument.
+constexpr double kDfReach = 4096.0;
 
 // Box clips (FP64, as in the renderer) of the rays of the CTA's tiles k0 .. k0 + 63 (its k-th tile
 // is blockIdx.x + k gridDim.x, rays 2 tile and 2 tile + 1), one ray per thread (the first 128).
@@ -34,6 +37,7 @@ __device__ __forceinline__ void clip_tile_rays(int R, const float *ro, const flo
         const Clip q = slab_clip(o, d, mn, mx, t_near, t_far);
         c.hit = q.hi > q.lo;
         if (c.hit) {
+            if (fmax(q.hi, fmax(fabs(o[0]), fmax(fabs(o[1]), fabs(o[2])))) > kDfReach) c.hit = 3;
             c.t0 = df_from_double(q.lo);
             c.w = df_from_double(__dmul_rn(__dsub_rn(q.hi, q.lo), 1.0 / kPropBins));   // exact: a power of two
 #pragma unroll
