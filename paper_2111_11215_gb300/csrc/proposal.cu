@@ -535,9 +535,12 @@ __global__ void __launch_bounds__(kPdfThreads) sample_pdf_kernel(int R, BoxD B, 
                 }
             }
             // (a lane's last bin ends where the scan starts the next lane, 1e-15 off its own sum: a bin of
-            // probability 0 may be met there, and the fraction leave [0, 1])
-            float frac = qb.hi == 0.0f ? 0.0f : __fdiv_rn(df_add(u, df_neg(Qb)).hi, qb.hi);
-            frac = frac < 0.0f ? 0.0f : (frac > 1.0f ? 1.0f : frac);
+            // probability 0 may be met there, and the fraction leave [0, 1].  Below the first bin and above the last
+            // a jitter outside [0, 1) extrapolates; a NaN among the probabilities, or none above 0, gives NaN.)
+            float frac = __fdiv_rn(df_add(u, df_neg(Qb)).hi, qb.hi);
+            if (qb.hi == 0.0f && Qtot.hi > 0.0f) frac = 0.0f;
+            if (b > 0 && frac < 0.0f) frac = 0.0f;
+            if (b < nb - 1 && frac > 1.0f) frac = 1.0f;
             const Df t = df_add(t0, df_mul(df_two_sum((float)b, frac), w));
             const Df tn = {__shfl_down_sync(0xffffffffu, t.hi, 1), __shfl_down_sync(0xffffffffu, t.lo, 1)};
             if (j < ns) to[j] = t.hi;
