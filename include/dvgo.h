@@ -207,7 +207,9 @@ typedef struct {
  *                  cos(2^k d_c) (c-major)] and, with n_freq_pos > 0, the same encoding of the
  *                  world-space query point x appended: [x (3), sin(2^k x_c), cos(2^k x_c)];
  *   ReLU after the hidden layers, sigmoid on the output (Sec. 2 Eq. nerf_mlp output activation,
- *   Sec. 4.2 Eq. fine_queries_rgb, Supp. A: C = 12, k_d = 4, k_x = 5, in = 72). */
+ *   Sec. 4.2 Eq. fine_queries_rgb, Supp. A: C = 12, k_d = 4, k_x = 5, in = 72).
+ * ReLU(NaN) = 0 and a unit that is not above 0 passes no gradient.  Infinite features and weights go through the
+ *   DVGO_MLP_FP32 forward as through FP32 arithmetic; its backward with in = 39 takes them for NaN. */
 typedef struct {
     const float *w1, *b1, *w2, *b2, *w3, *b3;
 } dvgo_mlp;
