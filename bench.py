@@ -530,7 +530,7 @@ def traffic_from_profiles(kind, chosen):
     current source (the summary records the source file's hash)."""
     import hashlib
     import re
-    prof, src = {("fine_colour_bwd", False): ("fine_colour_bwd_fp32_160cube_8192rays.md", "fine_tc_fp32_bwd.cu"),
+    prof, src = {("fine_colour_bwd", False): ("fine_colour_kernels_160cube_8192rays.md", "fine_tc_fp32_bwd.cu"),
                  ("fine_colour_bwd", True): ("fine_kernels_bf16_chosen_160cube_8192rays.md", "fine_tc.cu"),
                  ("adam", False): ("adam_fine_step_160cube.md", "adam.cu"),
                  ("adam", True): ("adam_fine_step_160cube.md", "adam.cu")}.get((kind, chosen), (None, None))

@@ -491,7 +491,8 @@ int dvgo_sample_pdf(const dvgo_params *p, const dvgo_grid_desc *density_desc, in
                     const float *rays_d, const float *probs, int n_bins, int n_samples, const float *jitter,
                     float eta, float *t_out, float *dt_out, void *stream);
 
-/* Kernel kinds for the optional per-kernel timing below. */
+/* Kernel kinds for the optional per-kernel timing below.  (DVGO_K_SCAN keeps its number; no kernel of that kind is
+ * launched: every ray owns a fixed range of sample slots.) */
 enum {
     DVGO_K_RAY_SETUP = 0, DVGO_K_SCAN = 1, DVGO_K_COARSE_FWD = 2, DVGO_K_COARSE_BWD = 3,
     DVGO_K_FINE_DENSITY = 4, DVGO_K_FINE_COLOUR_FWD = 5, DVGO_K_FINE_COMPOSITE = 6,

@@ -33,6 +33,7 @@ DVGO_NOALLOC_SCRATCH_BYTES = 2621696
 DVGO_ACT_POST, DVGO_ACT_PRE, DVGO_ACT_IN = 0, 1, 2   # Sec. 3 interpolation / activation orders
 DVGO_LAYOUT_CANONICAL, DVGO_LAYOUT_PACKED = 0, 1     # grid storage layouts
 
+# ("scan" keeps its number; no kernel of that kind is launched)
 KERNEL_KINDS = ("ray_setup", "scan", "coarse_fwd", "coarse_bwd", "fine_density", "fine_colour_fwd",
                 "fine_composite", "fine_comp_bwd", "fine_colour_bwd", "adam", "aux", "weight_bins", "proposal_fwd",
                 "proposal_bwd", "sample_pdf", "view_counts")

@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_bwd_kernel(RenderArgs A
     }
 }
 
-// Two rays per block; every ray has its own warp up to 32 blocks per SM, then the warps stride.
+// Two rays per block; every ray has its own warp up to 64 blocks (128 rays) per SM in the grid, then the warps stride.
 int coarse_grid(int R) {
     const int want = (R + 1) / 2, cap = num_sms() * 64;
     return want > cap ? cap : (want < 1 ? 1 : want);

@@ -122,12 +122,16 @@ struct SmemTC {
     unsigned char tp[kPanelBytes];        // tail panel: row = hidden unit / sample; W3 in columns 0-2,
                                           // X tails in 16-31 / 32-47, W1 tail in 48-63
     unsigned char x[2][kPanelBytes];      // X (double-buffered): row = sample
-    unsigned char h1[2 * kPanelBytes];    // H1, later dZ1
+    // The backward's consumers hold no barrier among themselves; a buffer is rewritten once the MMA batches they
+    // wait for were the last to read it: H1 (read by layer 2 and dW2) after the next tile's z1; H2 (read by
+    // dW3) by dZ1 after dh, dZ1 (read by de and dW1) by the next H2 after the next z2; dZ2 (read by dH1 and dW2)
+    // after the next z2.  The forward keeps its hidden layers in tensor memory.
+    unsigned char h1[2 * kPanelBytes];    // H1
     // backward: columns 0-15: [dout_r, dout_g, dout_b, 1, ...] (MMA operand); bytes 32-79 and 80-127
     // of every row (16-byte chunks 2-4 and 5-7): de[0:12] in FP32 for X buffer 0 and 1.  It follows
     // H1 directly, so [H1 | dout] is one MN-major operand of N = 144 (panels 16 KiB apart)
     unsigned char dout[kPanelBytes];
-    unsigned char h2[2 * kPanelBytes];    // H2
+    unsigned char h2[2 * kPanelBytes];    // H2, then dZ1
     SmallTC sm;
     // backward only (the forward allocates the struct up to here)
     unsigned char dz2[2 * kPanelBytes];   // dZ2

@@ -10,14 +10,15 @@
 // chain is 4e-7 off (samples of a proposal, weights over many orders of magnitude).  So hi x hi of dW1 and
 // dW2 goes to four accumulators of 32 samples, that of dH1 and de to two of 64 units; they join with rounding.
 // Errors against FP64 over 40 drawn steps, relative to the CUDA-core kernel's: MLP gradients 0.70, feature
-// gradients 0.87 (geometric means).  A ReLU unit within rounding of zero is decided by the plain FP32 FMA chain over its inputs
-// (exact_z1 / exact_z2, the order of the SIMT kernel), so the gradients do not hang on which
-// arithmetic recomputed the hidden layers.
+// gradients 0.87 (geometric means).  A ReLU unit within rounding of zero is decided by the plain FP32 FMA
+// chain over its inputs (exact_z1 / exact_z2, the order of the SIMT kernel), so the gradients do not hang
+// on which arithmetic recomputed the hidden layers.
 //
-// Bound: the serial chain of a tile -- seven MMA batches (12 k clocks of the tensor pipe at M = N = 128) and,
-// between them, three epilogues that split 16 k values each on two warps per scheduler; shared memory
-// (weights and 64 KB of activations) leaves no room for a second tile beside it.  160^3, 8,192 rays,
-// 1.38 M samples: 4610 us on the CUDA cores (45 % of their FP32 rate), 1245 us here, 33 k clocks a tile.
+// Bound: the serial chain of a tile -- nine MMA batches and, between them, three epilogues that split 16 k values
+// each on two warps per scheduler; shared memory (weights and 64 KB of activations) leaves no room for a
+// second tile beside it.  160^3, 8,192 rays, 1.38 M samples: 4610 us on the CUDA cores (45 % of their FP32
+// rate), 1320 us here, 18.6 us a tile, the tensor pipe active for 35 % of it (1240 us and 38 % with one
+// accumulator for hi x hi of each weight gradient).
 //
 // Per tile of M = 128 kept samples, with dout = dL/do from the compositing backward; activations are kept
 // transposed (TMEM lane = hidden unit, column = sample), so that a thread owns a unit: the sums over the

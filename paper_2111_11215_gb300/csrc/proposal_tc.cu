@@ -312,7 +312,7 @@ struct SmemB {
 };
 
 // MN-major A operand of M = 128 whose first 64 rows are panel `base` and last 64 rows the panel
-// `lbo` bytes after it; k-step kk = 16 tile rows.
+// `lbo` bytes after it (k-step 0; mnstep for the others).
 __device__ __forceinline__ uint64_t desc_mn_pair(uint32_t base, uint32_t lbo) {
     return sdesc(base, lbo, kGroupBytes);
 }
