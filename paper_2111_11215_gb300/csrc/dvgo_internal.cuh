@@ -57,7 +57,7 @@ struct alignas(16) RayChunk {
     int index;
     int first;           // the ray's slot of the first kept one; the others follow it
 };
-inline int chunks_per_ray(long long cap) { return (int)((cap + 31) / 32); }
+__host__ __device__ inline int chunks_per_ray(long long cap) { return (int)((cap + 31) / 32); }
 
 // Workspace header (first 256 bytes of the workspace).
 struct WsHeader {
@@ -69,7 +69,11 @@ struct WsHeader {
                          // thousands, which in FP32 cost the loss 1e-6 (two-ray blocks, 8192 rays)
     int aux;             // 1: the last forward had a target and auxiliary loss weights (rtarget valid)
     int xcache;          // 1: the last forward stored the colour kernels' input panels (xcache valid)
-    int pad[56];
+    // where the last fine forward left its state (0 rays: none): a reader with another step, ray count or kind of
+    // samples would otherwise take the slots' place from its own parameters, and other data for records
+    int n_rays, cap;
+    unsigned long long texit_at, rayk_at, rchunk_at, stau_at;   // bytes from here
+    int pad[46];
 };
 static_assert(sizeof(WsHeader) == 256, "WsHeader size");
 

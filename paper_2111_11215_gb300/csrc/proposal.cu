@@ -69,20 +69,32 @@ __global__ void __launch_bounds__(256) weight_bins_kernel(RenderArgs A, int nbin
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    // the state lies where the forward's own parameters put it
+    const WsHeader &H = *A.hdr;
+    const char *base = reinterpret_cast<const char *>(A.hdr);
+    const double *texit = reinterpret_cast<const double *>(base + H.texit_at);
+    const int4 *rayk = reinterpret_cast<const int4 *>(base + H.rayk_at);
+    const RayChunk *rchunk = reinterpret_cast<const RayChunk *>(base + H.rchunk_at);
+    const float *stau = reinterpret_cast<const float *>(base + H.stau_at);
+    const int n_rays = H.n_rays, cap = H.cap, nchunk = chunks_per_ray(cap);
     for (int r = warp; r < A.R; r += nwarps) {
+        if (r >= n_rays) {   // not a ray of the forward
+            for (int b = lane; b < nbins; b += 32) labels[(size_t)r * nbins + b] = 1.0f / nbins;
+            continue;
+        }
         const RayRec rr = A.rays[r];
-        const double t0 = rr.t_enter, t1 = A.texit[r];
+        const double t0 = rr.t_enter, t1 = texit[r];
         // bin of sample k: floor((t_k - t_enter) / (t_exit - t_enter) nbins), t_k - t_enter = (k + p) step
         const double bin_scale = __ddiv_rn(__dmul_rn((double)A.step, (double)nbins), __dsub_rn(t1, t0));
         for (int b = lane; b < nbins; b += 32) bins[wib][b] = 0.0f;
         __syncwarp();
         float wsum = 0.0f;
-        const int nrec = A.rayk[r].x;   // chunks with a kept sample; the other samples have weight 0
-        const size_t off = (size_t)r * A.cap;
+        const int nrec = rayk[r].x;   // chunks with a kept sample; the other samples have weight 0
+        const size_t off = (size_t)r * cap;
         for (int c = 0; c < nrec; ++c) {
-            const RayChunk ch = A.rchunk[(size_t)r * A.nchunk + c];
+            const RayChunk ch = rchunk[(size_t)r * nchunk + c];
             const bool kept = (ch.mask >> lane) & 1u;
-            const float tau = kept ? A.stau[off + ch.first + __popc(ch.mask & ((1u << lane) - 1u))] : 0.0f;
+            const float tau = kept ? stau[off + ch.first + __popc(ch.mask & ((1u << lane) - 1u))] : 0.0f;
             const float incl = warp_incl_scan(tau, lane);
             float excl = __shfl_up_sync(0xffffffffu, incl, 1);
             if (lane == 0) excl = 0.0f;
@@ -580,25 +592,14 @@ int dvgo_weight_bins(const dvgo_params *p, const dvgo_grid_desc *dd, int n_rays,
     const size_t need = dvgo_workspace_size(&q, dd, n_rays, nullptr);
     if (need == 0) return DVGO_ERR_INVALID_ARG;
     if (ws_bytes < need) return DVGO_ERR_WORKSPACE;
-    double diag2 = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        const double L = (double)dd->xyz_max[a] - (double)dd->xyz_min[a];
-        diag2 = diag2 + L * L;
-    }
-    const long long cap = (long long)(ceil(sqrt(diag2) / (double)p->step) + 1.0);
-    const WsLayout L = ws_layout(n_rays, cap * n_rays, DVGO_MODE_FINE);
+    const WsLayout L = ws_layout(n_rays, 0, DVGO_MODE_FINE);   // (header and ray records: the same in every layout)
     RenderArgs A;
     memset(&A, 0, sizeof(A));
     char *b = static_cast<char *>(const_cast<void *>(workspace));
     A.R = n_rays;
     A.step = p->step;
+    A.hdr = reinterpret_cast<WsHeader *>(b + L.header);
     A.rays = reinterpret_cast<RayRec *>(b + L.rays);
-    A.cap = (int)cap;
-    A.nchunk = chunks_per_ray(cap);
-    A.rayk = reinterpret_cast<int4 *>(b + L.rayk);
-    A.rchunk = reinterpret_cast<RayChunk *>(b + L.rchunk);
-    A.stau = reinterpret_cast<float *>(b + L.stau);
-    A.texit = reinterpret_cast<double *>(b + L.texit);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int blocks = (n_rays + 7) / 8;
     if (blocks > num_sms() * 16) blocks = num_sms() * 16;

@@ -46,6 +46,16 @@ __global__ void __launch_bounds__(kSetupThreads) ray_setup_kernel(RenderArgs A, 
         A.hdr->loss_acc = 0.0;
         A.hdr->aux = (A.target && (A.w_pt != 0.0f || A.w_bg != 0.0f)) ? 1 : 0;
         A.hdr->xcache = A.xcache != nullptr ? 1 : 0;
+        const bool fine = A.rayk != nullptr;
+        const auto at = [&](const void *p) {
+            return fine ? (unsigned long long)(static_cast<const char *>(p) - reinterpret_cast<const char *>(A.hdr)) : 0ull;
+        };
+        A.hdr->n_rays = fine ? A.R : 0;
+        A.hdr->cap = A.cap;
+        A.hdr->texit_at = at(A.texit);
+        A.hdr->rayk_at = at(A.rayk);
+        A.hdr->rchunk_at = at(A.rchunk);
+        A.hdr->stau_at = at(A.stau);
     }
     if (r >= A.R) return;
     double o[3] = {(double)rays_o[3 * r], (double)rays_o[3 * r + 1], (double)rays_o[3 * r + 2]};
